@@ -64,6 +64,24 @@ void free_ctx(amm_ctx* c) {
   delete c;
 }
 
+// Lanes per cell of the gradient and update kernels (amm_tuning; amm_autotune
+// measures them): with few cells more lanes put the chip's threads to work and
+// shorten each one's chain of gathers, with many they only repeat the
+// per-cell work.  Measured (us, gradients / update of one step):
+//   FP32, cells   1 lane         2 lanes        4 lanes        8 lanes
+//     1.6 k       11.9 / 12      11.9 / 10.2    11.9 / 10.2    11.8 / 9.6
+//    64 k         26 / 20        22 / 19        22 / 22        29 / 32
+//   262 k         78 / 55        64 / 49        63 / 53        82 / 80
+//   1.4 M        331 / 217      271 / 192      281 / 236      398 / 369
+//   FP64, cells
+//     8.2 k (2D)  67 / 18        51 / 16        44 / 10        63 / 12
+//    91 k        344 / 68       328 / 61       414 / 76       608 / 78
+void default_lanes(amm_ctx* c) {
+  const int64_t few = 40000;   // threads below which more lanes still pay in the update
+  c->update_lanes = 8 * c->n <= few ? 8 : (4 * c->n <= few ? 4 : 2);
+  c->grad_lanes = c->n <= (c->is_fp64() ? 30000 : 300000) ? 4 : 2;
+}
+
 template <typename F64, typename F32>
 cudaError_t dispatch(amm_ctx* c, F64 f64, F32 f32) {
   return c->is_fp64() ? f64() : f32();
@@ -244,6 +262,7 @@ int amm_create(amm_ctx** out, int dim, int64_t n, const double* gen, int64_t nf,
   c->box_cells = bc;
   c->box_faces = bf;
   c->nf_cap = nf;
+  default_lanes(c);
   int dev = 0;
   cudaError_t e0 = cudaGetDevice(&dev);
   if (e0 != cudaSuccess) {

@@ -267,8 +267,8 @@ struct amm_ctx {
   void* ekmax = nullptr;           // [n] real
   unsigned char* kept = nullptr;   // [n]
   int headroom = 7;
-  int grad_lanes = 4;              // lanes per cell in the gradient kernel
-  int update_lanes = 4;            // lanes per cell in the update kernel
+  int grad_lanes = 4;              // lanes per cell in the gradient kernel (amm_create's rule, amm_set_tuning)
+  int update_lanes = 2;            // lanes per cell in the update kernel (likewise)
   int flux_block = 256;            // threads (faces) per CTA of the flux kernel
   float tuned_ms = 0.f;
   int persistent = 0;              // 1: one cooperative launch per step (amm_advance)

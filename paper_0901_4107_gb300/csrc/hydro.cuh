@@ -885,31 +885,54 @@ __global__ void __launch_bounds__(B, sizeof(real) == 4 ? 4 * FACE_TILE / B : FAC
 }
 
 // ------------------------------------------------------------ A8+A1+A9
-// Fixed-point image of an FP32 value: x * 2^s as an int64, truncated toward
-// zero, with s = 188 - headroom - eb and eb the biased exponent of the largest
-// magnitude of the component, so every |x| 2^s < 2^(62 - headroom) and a sum
-// over at most 2^headroom terms cannot overflow; the image is added to `acc`
-// with the sign of x flipped when `flip` is set (the incidence's side).
-// Built from the float's bits on the integer pipe (a float-to-int64
-// conversion instruction would run on GB300's narrow FP64 pipe): with the
-// 24-bit significand M and biased exponent e <= eb, the image is
-// floor(M 2^(e - eb + 38 - headroom)) = (M 2^38) >> (eb + headroom - e), one
-// right shift.  Zero (e = 0; denormals are flushed in the FP32 form) adds 0;
-// Inf/NaN sets `bad`.  ebh = eb + headroom.
-__device__ __forceinline__ void add_fixed(long long& acc, float x, int ebh, bool flip, bool& bad) {
-  const unsigned u = __float_as_uint(x);
-  const int e = (int)((u >> 23) & 0xffu);
-  bad |= (e == 255);
-  const unsigned long long M = (e != 0) ? (unsigned long long)((u & 0x7fffffu) | 0x800000u) : 0ull;
-  const long long X = (long long)((M << 38) >> min((unsigned)(ebh - e), 63u));
-  const long long neg = -(long long)(((u >> 31) ^ (unsigned)flip) & 1u);   // 0 or all ones
-  acc += (X ^ neg) - neg;
+// Exact sums of FP32 values as integers: the image of x is the multiple of
+// 2^-s nearest to it, s = 188 - headroom - eb with eb the biased exponent of
+// the component's largest magnitude, so every |x| 2^s < 2^(62 - headroom) and
+// a sum over fewer than 2^(headroom - 1) terms fits an int64.  The image is
+// taken in three digits of 22, L2 and L3 bits (together 62 - headroom), each by
+// adding 1.5 2^23: an FP32 number t with |t| <= 2^22 then carries the nearest
+// integer in its low bits, and t minus that integer is exact and at most 1/2.
+// A digit is summed over the incidences in 32 bits (the raw bits are added;
+// the constants' sum is taken off at the end), at most FIX_RUN of them before
+// the digits are put together.
+//
+// Shifting the significand by the exponent difference took about 16 integer
+// instructions per component, on a pipe with half the FP32 rate (79% busy);
+// this takes 8 on the FP32 pipe and 3 integer adds.
+struct FixDigits {
+  unsigned a, b, c;   // (modulo 2^32)
+};
+constexpr float FIX_MAGIC = 12582912.0f;   // 1.5 2^23
+constexpr int FIX_RUN = 256;               // 256 2^22 < 2^31
+
+__device__ __forceinline__ int fixed_low_bits(int headroom) { return 40 - headroom; }   // L2 + L3
+
+// x 2^s1 = a + b 2^-L2 + c 2^-(L2+L3), s1 the exponent of `scale` (negated to
+// flip the sign); m2 = 2^L2, m3 = 2^L3
+__device__ __forceinline__ void add_fixed(FixDigits& d, float x, float scale, float m2, float m3) {
+  const float u = __fmaf_rn(x, scale, FIX_MAGIC);
+  const float r = __fmaf_rn(x, scale, -__fadd_rn(u, -FIX_MAGIC));
+  const float v = __fmaf_rn(r, m2, FIX_MAGIC);
+  const float t = __fmaf_rn(r, m2, -__fadd_rn(v, -FIX_MAGIC));
+  const float w = __fmaf_rn(t, m3, FIX_MAGIC);
+  d.a += __float_as_uint(u);
+  d.b += __float_as_uint(v);
+  d.c += __float_as_uint(w);
 }
 
-// 2^(eb - 188 + headroom) in FP64 (exact)
-__device__ __forceinline__ double fixed_scale(int eb, int headroom) {
-  return __longlong_as_double((long long)(1023 + eb - 188 + headroom) << 52);
+// the digits of `count` added values as one integer
+__device__ __forceinline__ long long fixed_total(const FixDigits& d, int count, int l2, int l3) {
+  const unsigned k = (unsigned)count * __float_as_uint(FIX_MAGIC);   // (modulo 2^32, like the sums)
+  return (long long)(int)(d.a - k) * (1ll << (l2 + l3)) + (long long)(int)(d.b - k) * (1ll << l3) +
+         (long long)(int)(d.c - k);
 }
+
+// the first digit's scale 2^(148 - eb); the exponent is held within FP32's
+// (largest magnitudes below 2^-105 keep a coarser image)
+__device__ __forceinline__ int fixed_exponent(int eb) { return min(148 - eb, 127); }
+
+// 2^-k in FP64 (exact), |k| < 1023
+__device__ __forceinline__ double pow2_neg(int k) { return __longlong_as_double((long long)(1023 - k) << 52); }
 
 // rho^gamma in the bulk precision (the FP32 forms' entropy switch takes it
 // in FP32, like the rest of their bulk arithmetic)
@@ -922,73 +945,148 @@ __device__ __forceinline__ double rho_pow_gamma(const HydroView<real>& v, double
   }
 }
 
+// the biased exponent of the step's largest |A F| of a component
+template <typename real>
+__device__ __forceinline__ int largest_exponent(const HydroView<real>& v, int box, int a) {
+  return (int)((v.fmax_bits[FMAX_STRIDE * box + a] >> 23) & 0xffu);
+}
+
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// barrier of the first N threads of a CTA (the others have left, or N is all)
+template <int N>
+__device__ __forceinline__ void finish_barrier() {
+  if constexpr (N == CELL_TILE)
+    __syncthreads();
+  else if constexpr (N > 32)
+    asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
+  else
+    __syncwarp();
+}
+
+constexpr int UPD_BATCH = 2;
+static_assert(FIX_RUN % UPD_BATCH == 0, "a run is whole batches");
 // G consecutive lanes share a cell (as in the gradient kernel); lane l sums
-// the cell's incidences l, l+G, ...; the lane partial sums are combined with
-// shuffles and lane 0 applies the update.  ENT: the entropy switch of
+// the cell's incidences l, l+G, ..., and the lane sums are combined with
+// shuffles.  The cells of the CTA are then finished by its first CELL_TILE / G
+// threads, one each, and the others leave: finishing takes about thirty FP64
+// instructions per cell, and the narrow FP64 pipe takes a whole warp's time for
+// each whether 8 or 32 of its lanes are on.  What bounds it: the latency of the
+// chain list -> face index -> flux (long scoreboard; DRAM at a third, issue at a
+// third), so two fluxes and the next two indices are in flight per lane.
+// 1.4 M cells of 7.8 faces, 4 lanes per cell with lane 0 of each group
+// finishing its own cell: 471 us; 2 lanes, as here: 192 us (1 lane 217, 4
+// lanes 236).  ENT: the entropy switch of
 // Sec. 3.5 (a sixth flux component, the entropy, and the per-cell choice
 // between the advected entropy and the energy update).
 template <typename real, int G, bool ENT = false>
 __device__ __forceinline__ void update_item(const HydroView<real>& v, int wi) {
   constexpr int CELLS = CELL_TILE / G;
   constexpr int NA = ENT ? 6 : 5;
+  constexpr bool F32 = sizeof(real) == 4;
   const Tile t = v.ctiles[wi / G];
-  const int lane = (int)threadIdx.x % G;
-  const int i = t.begin + (int)(wi % G) * CELLS + (int)threadIdx.x / G;
-  const bool valid = i < t.end;
-  const int q0 = valid ? v.csr_off[i] : 0;
-  const int q1 = valid ? v.csr_off[i + 1] : 0;
+  const int tid = (int)threadIdx.x;
+  const int lane = tid % G;
+  const int first = t.begin + (int)(wi % G) * CELLS;   // the CTA's first cell
+  const int ig = first + tid / G;                      // the group's cell
+  const int q0 = ig < t.end ? v.csr_off[ig] : 0;
+  const int q1 = ig < t.end ? v.csr_off[ig + 1] : 0;
   const size_t n = (size_t)v.n;
-  double q[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  const int l3 = fixed_low_bits(v.headroom) / 2, l2 = fixed_low_bits(v.headroom) - l3;
   double d[NA];
   real mach = (real)1;
   bool bad = false;
-  // per tile (one box): the fixed-point exponents and dt times the scale of
-  // each component's sums, so a cell's update is one FMA per component
-  __shared__ int s_eb[6];
-  __shared__ double s_dts[6];
-  if (threadIdx.x == 0) {
-    const double dt = box_dt(v, t.box);
-    for (int a = 0; a < NA; a++) {
-      const int eb = (int)((v.fmax_bits[FMAX_STRIDE * t.box + a] >> 23) & 0xffu);
-      s_eb[a] = eb;
-      s_dts[a] = (sizeof(real) == 4 && v.fixed_acc) ? dt * fixed_scale(eb, v.headroom) : dt;
-    }
+  // the finishing threads' state, on its way while the fluxes are gathered
+  if (tid < CELLS && first + tid < t.end) {
+#pragma unroll
+    for (int a = 0; a < 5; a++) prefetch_l2(v.Q + a * n + first + tid);
   }
-  __syncthreads();
-  if (sizeof(real) == 4 && v.fixed_acc) {
-    // Exact sums: every face flux is converted once to an int64 multiple of
-    // 2^-s (s per box and component, from the step's largest |A F|) and the
+  // dt times the weight of each component's sums, so a cell's update is one FMA
+  // per component (one thread, while the others gather: FP64)
+  __shared__ double s_dts[6];
+  if (tid == CELL_TILE - 1) {
+    const double dt = box_dt(v, t.box);
+    for (int a = 0; a < NA; a++)
+      s_dts[a] = (F32 && v.fixed_acc) ? dt * pow2_neg(fixed_exponent(largest_exponent(v, t.box, a)) + l2 + l3) : dt;
+  }
+  if (F32 && v.fixed_acc) {
+    // Exact sums: every face flux is converted to an integer multiple of 2^-s
+    // (s per box and component, from the step's largest |A F|) and the
     // integers are added; both cells of a face add the identical integer
     // with opposite signs, so the update conserves exactly and does not
     // depend on the summation order.  One rounding per cell remains, when
     // the integer total is scaled back to FP64.
-    int ebh[NA];
-#pragma unroll
-    for (int a = 0; a < NA; a++) ebh[a] = s_eb[a] + v.headroom;
+    const float m2 = __int_as_float((127 + l2) << 23), m3 = __int_as_float((127 + l3) << 23);
+    float scale[NA];
     long long acc[NA];
+    bool inf = false;
 #pragma unroll
-    for (int a = 0; a < NA; a++) acc[a] = 0;
-#pragma unroll 4
-    for (int e = q0 + lane; e < q1; e += G) {
-      const int2 r = v.csr[e];
-      const int k = r.x >> 1;
-      const R4<real> f = v.flux[k];
-      float fv[NA];
-      fv[0] = (float)f.x; fv[1] = (float)f.y; fv[2] = (float)f.z; fv[3] = (float)f.w; fv[4] = (float)v.fluxE[k];
-      if constexpr (ENT) {
-        fv[5] = (float)v.fluxS[k];
-        const real mf = v.machf[k];
-        mach = mf > mach ? mf : mach;
+    for (int a = 0; a < NA; a++) {
+      const int eb = largest_exponent(v, t.box, a);
+      inf |= eb == 255;
+      scale[a] = __int_as_float((127 + fixed_exponent(eb)) << 23);
+      acc[a] = 0;
+    }
+    for (int c0 = q0 + lane; c0 < q1; c0 += FIX_RUN * G) {
+      const int c1 = min(q1, c0 + FIX_RUN * G);
+      FixDigits dg[NA];
+#pragma unroll
+      for (int a = 0; a < NA; a++) dg[a].a = dg[a].b = dg[a].c = 0;
+      // two incidences at a time, their fluxes in flight together and the next
+      // ones' face indices behind them; past the end zeros are added (an
+      // unrolled loop's remainder would wait for each of its loads in turn)
+      int kx[UPD_BATCH];
+#pragma unroll
+      for (int u = 0; u < UPD_BATCH; u++) kx[u] = c0 + u * G < c1 ? v.csr[c0 + u * G].x : 0;
+      int count = 0;
+      for (int e = c0; e < c1; e += UPD_BATCH * G) {
+        float fv[UPD_BATCH][NA], sg[UPD_BATCH];
+#pragma unroll
+        for (int u = 0; u < UPD_BATCH; u++) {
+          const int k = kx[u] >> 1;
+          sg[u] = (kx[u] & 1) ? -1.0f : 1.0f;
+#pragma unroll
+          for (int a = 0; a < NA; a++) fv[u][a] = 0.0f;
+          if (e + u * G < c1) {
+            const R4<real> f = v.flux[k];
+            fv[u][0] = (float)f.x; fv[u][1] = (float)f.y; fv[u][2] = (float)f.z; fv[u][3] = (float)f.w;
+            fv[u][4] = (float)v.fluxE[k];
+            if constexpr (ENT) {
+              fv[u][5] = (float)v.fluxS[k];
+              const real mf = v.machf[k];
+              mach = mf > mach ? mf : mach;
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < UPD_BATCH; u++) {
+          const int en = e + (UPD_BATCH + u) * G;
+          kx[u] = en < c1 ? v.csr[en].x : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < UPD_BATCH; u++)
+#pragma unroll
+          for (int a = 0; a < NA; a++) add_fixed(dg[a], fv[u][a] * sg[u], scale[a], m2, m3);
+        count += UPD_BATCH;
       }
 #pragma unroll
-      for (int a = 0; a < NA; a++) add_fixed(acc[a], fv[a], ebh[a], (r.x & 1) != 0, bad);
+      for (int a = 0; a < NA; a++) acc[a] += fixed_total(dg[a], count, l2, l3);
+    }
+    if (inf) {
+      // a flux of this box is not finite: find the cells it touches
+      for (int e = q0 + lane; e < q1; e += G) {
+        const int k = v.csr[e].x >> 1;
+        const R4<real> f = v.flux[k];
+        bad |= !(isfinite((float)f.x) && isfinite((float)f.y) && isfinite((float)f.z) && isfinite((float)f.w) &&
+                 isfinite((float)v.fluxE[k]));
+        if constexpr (ENT) bad |= !isfinite((float)v.fluxS[k]);
+      }
+      bad = group_max<G>((int)bad) != 0;
     }
 #pragma unroll
-    for (int a = 0; a < NA; a++) acc[a] = group_sum<G>(acc[a]);
-    bad = group_max<G>((int)bad) != 0;
-    if (lane == 0) {
-#pragma unroll
-      for (int a = 0; a < NA; a++) d[a] = __ll2double_rn(acc[a]);
+    for (int a = 0; a < NA; a++) {
+      acc[a] = group_sum<G>(acc[a]);
+      d[a] = __longlong_as_double(acc[a]);   // converted by the finishing thread
     }
   } else {
     double acc[NA];
@@ -1019,8 +1117,35 @@ __device__ __forceinline__ void update_item(const HydroView<real>& v, int wi) {
     for (int a = 0; a < NA; a++) d[a] = group_sum<G>(acc[a]);
   }
   if constexpr (ENT) mach = group_max<G>(mach);
+  if constexpr (G > 1) {
+    // hand the groups' sums to the first CELLS threads
+    __shared__ double s_d[NA][CELLS];
+    __shared__ real s_mach[ENT ? CELLS : 1];
+    __shared__ unsigned char s_bad[CELLS];
+    if (lane == 0) {
+#pragma unroll
+      for (int a = 0; a < NA; a++) s_d[a][tid / G] = d[a];
+      if constexpr (ENT) s_mach[tid / G] = mach;
+      s_bad[tid / G] = bad;
+    }
+    __syncthreads();
+    if (tid >= CELLS) return;
+#pragma unroll
+    for (int a = 0; a < NA; a++) d[a] = s_d[a][tid];
+    if constexpr (ENT) mach = s_mach[tid];
+    bad = s_bad[tid] != 0;
+  } else {
+    __syncthreads();
+  }
+  const int i = first + tid;
+  const bool valid = i < t.end;
+  double q[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   unsigned nonpos = 0, keep = 0;
-  if (valid && lane == 0) {
+  if (valid) {
+    if (F32 && v.fixed_acc) {
+#pragma unroll
+      for (int a = 0; a < NA; a++) d[a] = __ll2double_rn(__double_as_longlong(d[a]));
+    }
 #pragma unroll
     for (int a = 0; a < 5; a++)
       q[a] = bad ? __longlong_as_double(0x7ff8000000000000ll) : v.Q[a * n + i] - s_dts[a] * d[a];
@@ -1055,15 +1180,18 @@ __device__ __forceinline__ void update_item(const HydroView<real>& v, int wi) {
     const real P = prims_from_Q(v, i, q[0], q[1], q[2], q[3], q[4]);
     nonpos = (!(q[0] > 0.0) || !(P > (real)0)) ? 1u : 0u;
   }
-  // per-block FP64 sums in a fixed order (bit reproducible).  Within a warp,
+  // per-block FP64 sums in a fixed order (bit reproducible), by the warps that
+  // finish cells.  Within a warp,
   // a butterfly that halves the components each lane carries at each of the
   // first three levels (5 components padded to 8): 9 FP64 adds per lane, where
   // a shuffle tree per component takes 25 on GB300's narrow FP64 pipe.  Lane
   // 4c then holds the warp's sum of component c; the warps' sums are added in
   // warp order.
-  __shared__ double red[CELL_TILE / 32][5];
+  constexpr int FIN_WARPS = CELLS / 32;
+  __shared__ double red[FIN_WARPS][5];
+  __shared__ unsigned s_keep[ENT ? FIN_WARPS : 1];
   {
-    const int l = (int)threadIdx.x & 31;
+    const int l = tid & 31;
     const bool b4 = (l & 16) != 0, b3 = (l & 8) != 0, b2 = (l & 4) != 0;
     double w4[4];
 #pragma unroll
@@ -1079,28 +1207,38 @@ __device__ __forceinline__ void update_item(const HydroView<real>& v, int wi) {
     w1 += __shfl_xor_sync(0xffffffffu, w1, 2);
     w1 += __shfl_xor_sync(0xffffffffu, w1, 1);
     const int c = l >> 2;   // 4 b4 + 2 b3 + b2
-    if ((l & 3) == 0 && c < 5) red[threadIdx.x >> 5][c] = w1;
+    if ((l & 3) == 0 && c < 5) red[tid >> 5][c] = w1;
   }
-  const unsigned nbad = __syncthreads_count(nonpos);
-  if constexpr (ENT) {
-    const unsigned nkeep = __syncthreads_count(keep);
-    if (threadIdx.x == 0 && nkeep) atomicAdd(&v.stats->kept, (unsigned long long)nkeep);
-  }
-  if (threadIdx.x < 5) {
-    double s = red[0][threadIdx.x];
-    for (int w = 1; w < CELL_TILE / 32; w++) s += red[w][threadIdx.x];
-    v.partial[5 * (size_t)wi + threadIdx.x] = s;
-  }
-  if (threadIdx.x == 0 && nbad) {
-    atomicAdd(&v.stats->nonpos, (unsigned long long)nbad);
+  // counts by warp (rarely or cheaply added), sums over the finishing warps
+  const unsigned wbad = __ballot_sync(0xffffffffu, nonpos != 0u);
+  if ((tid & 31) == 0 && wbad) {
+    atomicAdd(&v.stats->nonpos, (unsigned long long)__popc(wbad));
     atomicOr(&v.stats->status, (unsigned)ST_NONPOS);
     atomicOr(v.box_status + t.box, (unsigned)ST_NONPOS);
   }
-  __syncthreads();   // `red` is reused by the next work item of a persistent CTA
+  if constexpr (ENT) {
+    const unsigned wkeep = __ballot_sync(0xffffffffu, keep != 0u);
+    if ((tid & 31) == 0) s_keep[tid >> 5] = (unsigned)__popc(wkeep);
+  }
+  finish_barrier<CELLS>();
+  if (tid < 5) {
+    double s = red[0][tid];
+    for (int w = 1; w < FIN_WARPS; w++) s += red[w][tid];
+    v.partial[5 * (size_t)wi + tid] = s;
+  }
+  if constexpr (ENT) {
+    if (tid == 5) {
+      unsigned nkeep = 0;
+      for (int w = 0; w < FIN_WARPS; w++) nkeep += s_keep[w];
+      if (nkeep) atomicAdd(&v.stats->kept, (unsigned long long)nkeep);
+    }
+  }
+  // (a persistent CTA, G == 1, goes on to its next work item)
+  if constexpr (G == 1) __syncthreads();
 }
 
 template <typename real, int G, bool ENT>
-__global__ void __launch_bounds__(CELL_TILE) k_update(HydroView<real> v) {
+__global__ void __launch_bounds__(CELL_TILE, sizeof(real) == 4 ? 4 : 1) k_update(HydroView<real> v) {
   update_item<real, G, ENT>(v, blockIdx.x);
 }
 
@@ -1128,28 +1266,43 @@ __global__ void __launch_bounds__(CELL_TILE) k_partial_sums(HydroView<real> v) {
   }
 }
 
-// one CTA per box: ordered sum of the box's block partials; time step record
-constexpr int FINISH_THREADS = 512;
+// One CTA per box: sum of the box's block partials in a fixed order; time step
+// record.  The partials are read as one run of doubles: a thread count that is
+// a multiple of 5 keeps each thread on one component, so the loads are
+// coalesced and eight are in flight per thread (latency bound; with one
+// 40-byte record per thread and a barrier per halving this took 41 us for 22k
+// records).
+constexpr int FINISH_THREADS = 1024;
 template <typename real, int NT>
 __device__ __forceinline__ void finish_item(const HydroView<real>& v, int b, int count_step) {
-  const int t0 = v.box_first_ctile[b] * v.update_lanes, t1 = v.box_first_ctile[b + 1] * v.update_lanes;
-  __shared__ double red[5][NT];
-  double s[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  for (int tt = t0 + (int)threadIdx.x; tt < t1; tt += NT)
+  constexpr int NU = NT / 5 * 5;       // threads that read
+  const int tid = (int)threadIdx.x;
+  const size_t t0 = 5 * (size_t)v.box_first_ctile[b] * v.update_lanes;
+  const size_t t1 = 5 * (size_t)v.box_first_ctile[b + 1] * v.update_lanes;
+  __shared__ double red[NT];
+  double s = 0.0;
+  if (tid < NU) {
+#pragma unroll 1
+    for (size_t q = t0 + tid; q < t1; q += 8 * NU) {
+      double x[8];
 #pragma unroll
-    for (int a = 0; a < 5; a++) s[a] += v.partial[5 * (size_t)tt + a];
+      for (int u = 0; u < 8; u++) x[u] = q + (size_t)u * NU < t1 ? v.partial[q + (size_t)u * NU] : 0.0;
 #pragma unroll
-  for (int a = 0; a < 5; a++) red[a][threadIdx.x] = s[a];
-  __syncthreads();
-  for (int st = NT / 2; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st) {
-#pragma unroll
-      for (int a = 0; a < 5; a++) red[a][threadIdx.x] += red[a][threadIdx.x + st];
+      for (int u = 0; u < 8; u++) s += x[u];
     }
-    __syncthreads();
   }
-  if (threadIdx.x < 5) v.totals[5 * b + threadIdx.x] = red[threadIdx.x][0];
-  if (threadIdx.x == 0 && count_step) {
+  red[tid] = s;
+  __syncthreads();
+  // warp c sums component c: the reading threads c, c + 5, ...
+  const int c = tid >> 5;
+  if (c < 5) {
+    double r = 0.0;
+    for (int q = c + 5 * (tid & 31); q < NU; q += 160) r += red[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if ((tid & 31) == 0) v.totals[5 * b + c] = r;
+  }
+  if (tid == NT - 1 && count_step) {
     v.dt_used[b] = box_dt(v, b);
     if (b == 0) atomicAdd(&v.stats->steps, 1ull);
   }
@@ -1157,7 +1310,7 @@ __device__ __forceinline__ void finish_item(const HydroView<real>& v, int b, int
 }
 
 template <typename real>
-__global__ void k_finish(HydroView<real> v, int count_step) {
+__global__ void __launch_bounds__(FINISH_THREADS) k_finish(HydroView<real> v, int count_step) {
   finish_item<real, FINISH_THREADS>(v, blockIdx.x, count_step);
 }
 
