@@ -27,24 +27,27 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + NP_W1, OFF_W2 = OFF_B1 + NP_B1, OFF_
               OFF_W3 = OFF_B2 + NP_B2, OFF_B3 = OFF_W3 + NP_W3, NPARAMS = OFF_B3 + 1;
 
 __device__ __forceinline__ float silu(float z) { return z / (1.0f + __expf(-z)); }
-__device__ __forceinline__ float dsilu(float z) {
-  const float s = 1.0f / (1.0f + __expf(-z));
-  return s * (1.0f + z * (1.0f - s));
+
+// parameter i of the FP32 master vector into the kernels' weights (BF16
+// matrices, FP32 biases; the padding columns of W1 stay zero)
+__device__ __forceinline__ void mlp_pack_one(int i, float x, MlpDevice* out) {
+  if (i < OFF_B1)
+    out->W1[i / MLP_IN * 16 + i % MLP_IN] = __float2bfloat16_rn(x);
+  else if (i < OFF_W2)
+    out->b1[i - OFF_B1] = x;
+  else if (i < OFF_B2)
+    out->W2[i - OFF_W2] = __float2bfloat16_rn(x);
+  else if (i < OFF_W3)
+    out->b2[i - OFF_B2] = x;
+  else if (i < OFF_B3)
+    out->W3[i - OFF_W3] = __float2bfloat16_rn(x);
+  else
+    out->b3 = x;
 }
 
-// BF16 weights + FP32 biases from FP32 master parameters
 __global__ void k_mlp_pack(const float* p, MlpDevice* out) {
-  for (int i = threadIdx.x; i < MLP_HID * 16; i += blockDim.x) {
-    const int o = i / 16, k = i % 16;
-    out->W1[i] = __float2bfloat16_rn(k < MLP_IN ? p[OFF_W1 + o * MLP_IN + k] : 0.0f);
-  }
-  for (int i = threadIdx.x; i < MLP_HID * MLP_HID; i += blockDim.x) out->W2[i] = __float2bfloat16_rn(p[OFF_W2 + i]);
-  for (int i = threadIdx.x; i < MLP_HID; i += blockDim.x) {
-    out->W3[i] = __float2bfloat16_rn(p[OFF_W3 + i]);
-    out->b1[i] = p[OFF_B1 + i];
-    out->b2[i] = p[OFF_B2 + i];
-  }
-  if (threadIdx.x == 0) out->b3 = p[OFF_B3];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < NPARAMS) mlp_pack_one(i, p[i], out);
 }
 
 // Shared-memory image of one CTA's operands
@@ -167,28 +170,43 @@ __global__ void __launch_bounds__(MLP_TILE) k_mlp_forward(const MlpDevice* M, co
 
 
 // ---------------------------------------------------------------- training
-// Shared memory of the gradient kernel (one CTA per SM: it holds 512 TMEM
-// columns).  Operands are K-major no-swizzle tiles (tc.cuh).
+// Gradient kernel.  A CTA of 8 warps takes tiles of 128 samples; sample r is
+// row r of every MMA and lane r of tensor memory, and the two warps that can
+// read a quadrant of 32 lanes split the 64 columns.  Two CTAs share an SM
+// (208 of 256 tensor-memory columns and 63 KB each), so one computes
+// element-wise while the other waits for its tensor cores.
+//
+// What bounds it: the element-wise passes (two exponentials and two
+// reciprocals per hidden unit and sample, about 20 FP32 instructions) and the
+// barriers between the five stages of a tile; the tensor pipe is nearly idle.
+// So every sigmoid is taken once, its derivative kept in registers; the column
+// sums (bias and output-weight gradients, FP32) are a warp butterfly that
+// halves the columns a lane carries, 31 shuffles for 32 columns, accumulated
+// in a register per lane over the CTA's tiles; and the weight gradients read
+// the activations and deltas where the forward and backward MMAs left them, as
+// MN-major operands, instead of from transposed copies.
+// 2^20 samples: 2.05 ms with one CTA of 4 warps per SM, serial column sums and
+// transposed copies; 0.16 ms now (a step at 2048 samples: 70 us, 16 now).
+constexpr int TR_THREADS = 256;
+constexpr int TR_HX = 80;    // columns of the activation tile: H1 | X
+constexpr int TR_DZ = 128;   // columns of the delta tile: dZ2 | dZ1
+
 struct TrainSmem {
-  alignas(1024) uint8_t a1[MLP_TILE * 16 * 2];        // X        [128 x 16]
-  alignas(1024) uint8_t a2[MLP_TILE * MLP_HID * 2];   // H1       [128 x 64]
-  alignas(1024) uint8_t a3[MLP_TILE * MLP_HID * 2];   // dZ2      [128 x 64]
-  alignas(1024) uint8_t aw[128 * MLP_TILE * 2];       // [dZ2^T; dZ1^T]  [128 x 128 samples]
-  alignas(1024) uint8_t bw[80 * MLP_TILE * 2];        // [H1^T; X^T]     [80 x 128 samples]
+  alignas(1024) uint8_t hx[MLP_TILE * TR_HX * 2];     // [H1 (64) | X (16)]   [128 x 80]
+  alignas(1024) uint8_t dz[MLP_TILE * TR_DZ * 2];     // [dZ2 (64) | dZ1 (64)] [128 x 128]
   alignas(1024) uint8_t b1[MLP_HID * 16 * 2];         // W1       [64 x 16]
   alignas(1024) uint8_t b2[MLP_HID * MLP_HID * 2];    // W2       [64 x 64]
-  alignas(1024) uint8_t b2t[MLP_HID * MLP_HID * 2];   // W2^T     [64 x 64]
-  float red[MLP_TILE][MLP_HID + 1];                   // per-sample rows for column sums
-  float bias1[MLP_HID], bias2[MLP_HID], w3[MLP_HID], bias3;
-  float acc_b1[MLP_HID], acc_b2[MLP_HID], acc_w3[MLP_HID], acc_b3, acc_loss;
-  float lsum[MLP_TILE], dsum[MLP_TILE];
+  float bias1[MLP_HID], bias2[MLP_HID], w3[MLP_HID];
+  float ysum[2][MLP_TILE];
+  float colsum[4][3][MLP_HID];                        // per quadrant: dW3, db2, db1
+  float lsum[4], dsum[4];
   uint64_t mbar;
   uint32_t tmem;
   uint32_t ok;
 };
 
-// TMEM columns: [0,64) Z1, [64,128) Z2, [128,192) dH1, [256,336) weight grads
-constexpr int TC_Z1 = 0, TC_Z2 = 64, TC_DH1 = 128, TC_DW = 256;
+// TMEM columns: [0,64) Z1, [64,128) Z2 then dH1, [128,208) weight gradients
+constexpr int TC_Z1 = 0, TC_Z2 = 64, TC_DH1 = 64, TC_DW = 128, TC_COLS = 256;
 
 __device__ __forceinline__ void tr_sync() {
   tc::fence_async_smem();
@@ -197,253 +215,273 @@ __device__ __forceinline__ void tr_sync() {
   tc::fence_after_sync();
 }
 
-// column sums of red[0..127][0..63] into acc (thread j < 64 owns column j;
-// fixed row order)
-__device__ __forceinline__ void tr_colsum(TrainSmem& s, float* acc) {
-  __syncthreads();
-  if (threadIdx.x < MLP_HID) {
-    float a = 0.0f;
-    for (int r = 0; r < MLP_TILE; r++) a += s.red[r][threadIdx.x];
-    acc[threadIdx.x] += a;
+// sums over the warp's 32 rows of v[0..31] (destroyed): lane l gets column l's
+__device__ __forceinline__ float tr_colsum(float* v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < o; j++) {
+      const float keep = up ? v[j + o] : v[j], send = up ? v[j] : v[j + o];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
   }
-  __syncthreads();
+  return v[0];
 }
+
+// 32 columns of row t from column c0 of a K-major tile with K columns, as BF16
+__device__ __forceinline__ void tr_store32(uint8_t* tile, int t, int c0, int K, const float* v) {
+#pragma unroll
+  for (int q = 0; q < 4; q++) tc::st_bf16x8(tile, tc::kmajor_offset(t, c0 + 8 * q, K), v + 8 * q);
+}
+
+// the logistic function from the hardware's exponential and reciprocal (each
+// good to a few ulp)
+__device__ __forceinline__ float logistic(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
 
 // Gradient of L = sum over the batch of (y - t)^2 / n_total with respect to
 // every parameter; each CTA processes tiles blockIdx.x, blockIdx.x+gridDim.x,
 // ... of the batch and writes its partial sums to part[blockIdx.x][NPARAMS+1]
 // (the last entry is its share of the loss).
-__global__ void __launch_bounds__(MLP_TILE, 1) k_mlp_grads(const MlpDevice* M, const float* x, const float* tgt,
-                                                          const int* idx, int64_t n, float inv_n, float* part,
-                                                          unsigned* status) {
+__global__ void __launch_bounds__(TR_THREADS, 2) k_mlp_grads(const MlpDevice* M, const float* x, const float* tgt,
+                                                            const int* idx, int64_t n, float inv_n, float* part,
+                                                            unsigned* status) {
   extern __shared__ uint8_t smem_raw[];
   TrainSmem& s = *reinterpret_cast<TrainSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int t = threadIdx.x;
-  const int warp = t >> 5;
-  if (t < 32) tc::tmem_alloc(&s.tmem, 512);
+  const int warp = t >> 5, lane = t & 31;
+  const int quad = warp & 3, half = warp >> 2;   // tensor-memory lanes 32 quad.., columns 32 half..
+  const int row = 32 * quad + lane;              // the sample of the tile
+  const int c0 = 32 * half;
+  if (t < 32) tc::tmem_alloc(&s.tmem, TC_COLS);
   if (t == 0) {
     tc::mbar_init(&s.mbar, 1);
     s.ok = 1;
-    s.acc_b3 = 0.0f;
-    s.acc_loss = 0.0f;
   }
-  if (t < MLP_HID) s.acc_b1[t] = s.acc_b2[t] = s.acc_w3[t] = 0.0f;
-  // weights: W1, W2 and W2^T in the operand layout
-  for (int i = t; i < MLP_HID * 16; i += MLP_TILE)
-    *reinterpret_cast<__nv_bfloat16*>(s.b1 + tc::kmajor_offset(i / 16, i % 16, 16)) = M->W1[i];
-  for (int i = t; i < MLP_HID * MLP_HID; i += MLP_TILE) {
-    const int o = i / MLP_HID, k = i % MLP_HID;
-    *reinterpret_cast<__nv_bfloat16*>(s.b2 + tc::kmajor_offset(o, k, MLP_HID)) = M->W2[i];
-    *reinterpret_cast<__nv_bfloat16*>(s.b2t + tc::kmajor_offset(k, o, MLP_HID)) = M->W2[i];
-  }
+  // weights into the operand layout, 16 bytes (8 columns) at a time
+  const uint4* w1 = reinterpret_cast<const uint4*>(M->W1);
+  const uint4* w2 = reinterpret_cast<const uint4*>(M->W2);
+  if (t < MLP_HID * 2) *reinterpret_cast<uint4*>(s.b1 + tc::kmajor_offset(t / 2, 8 * (t % 2), 16)) = w1[t];
+  for (int i = t; i < MLP_HID * MLP_HID / 8; i += TR_THREADS)
+    *reinterpret_cast<uint4*>(s.b2 + tc::kmajor_offset(i / 8, 8 * (i % 8), MLP_HID)) = w2[i];
   if (t < MLP_HID) {
     s.bias1[t] = M->b1[t];
     s.bias2[t] = M->b2[t];
     s.w3[t] = __bfloat162float(M->W3[t]);
   }
-  if (t == 0) s.bias3 = M->b3;
+  const float bias3 = M->b3;
   tr_sync();
-  const uint32_t idesc64 = tc::make_idesc(128, 64), idesc80 = tc::make_idesc(128, 80);
+  const uint32_t tm = s.tmem;
+  const uint32_t hx = tc::smem_addr(s.hx), dz = tc::smem_addr(s.dz), sb1 = tc::smem_addr(s.b1), sb2 = tc::smem_addr(s.b2);
+  const uint32_t idesc64 = tc::make_idesc(128, 64);
   const int64_t tiles = (n + MLP_TILE - 1) / MLP_TILE;
+  float a_w3 = 0.0f, a_b2 = 0.0f, a_b1 = 0.0f;   // column c0 + lane, this quadrant's rows
+  float a_loss = 0.0f, a_b3 = 0.0f;              // this row (half 0)
   uint32_t phase = 0;
   bool first = true;
+  auto wait = [&] {
+    if (!tc::mbar_wait(&s.mbar, phase)) s.ok = 0;
+    phase ^= 1u;
+    tc::fence_after_sync();
+  };
   for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const int64_t row = tile * MLP_TILE + t;
-    const bool valid = row < n;
-    const int64_t src = valid ? (idx ? (int64_t)idx[row] : row) : 0;
+    const int64_t r = tile * MLP_TILE + row;
+    const bool valid = r < n;
+    const int64_t src = valid ? (idx ? (int64_t)idx[r] : r) : 0;
     float xi[16] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     float ti = 0.0f;
     if (valid) {
-      for (int j = 0; j < MLP_IN; j++) xi[j] = x[src * MLP_IN + j];
+      if (half == 0) {
+#pragma unroll
+        for (int j = 0; j < MLP_IN; j++) xi[j] = x[src * MLP_IN + j];
+      }
       ti = tgt[src];
     }
-    // X into A1 (row t) and into the rows 64.. of Bw (column t)
-    tc::st_bf16x8(s.a1, tc::kmajor_offset(t, 0, 16), xi);
-    tc::st_bf16x8(s.a1, tc::kmajor_offset(t, 8, 16), xi + 8);
-#pragma unroll
-    for (int j = 0; j < 16; j++)
-      *reinterpret_cast<__nv_bfloat16*>(s.bw + tc::kmajor_offset(64 + j, t, MLP_TILE)) =
-          __float2bfloat16_rn(valid ? xi[j] : 0.0f);
+    // the previous tile's weight-gradient MMAs still read the tiles
+    if (!first) wait();
+    if (half == 0) {
+      tc::st_bf16x8(s.hx, tc::kmajor_offset(row, 64, TR_HX), xi);
+      tc::st_bf16x8(s.hx, tc::kmajor_offset(row, 72, TR_HX), xi + 8);
+    }
     tr_sync();
     if (t == 0) {
-      tc::mma_bf16(s.tmem + TC_Z1, tc::kmajor_desc(tc::smem_addr(s.a1), 16), tc::kmajor_desc(tc::smem_addr(s.b1), 16),
-                   idesc64, false);
+      tc::mma_bf16(tm + TC_Z1, tc::kmajor_desc(hx + 8 * 128, TR_HX), tc::kmajor_desc(sb1, 16), idesc64, false);
       tc::mma_commit(&s.mbar);
     }
-    if (!tc::mbar_wait(&s.mbar, phase)) s.ok = 0;
-    phase ^= 1u;
-    tc::fence_after_sync();
-    // H1 = silu(Z1 + b1) -> A2 (row t) and Bw rows 0..63 (column t)
+    wait();
+    // H1 = silu(Z1 + b1), its derivative kept
+    float d1[32];
+    {
+      float z[32];
+      tc::tmem_ld32(tc::tmem_lane_addr(tm, quad, TC_Z1 + c0), z);
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-      float z[16];
-      tc::tmem_ld16(tc::tmem_lane_addr(s.tmem, warp, TC_Z1 + 16 * c), z);
-#pragma unroll
-      for (int j = 0; j < 16; j++) {
-        z[j] = silu(z[j] + s.bias1[16 * c + j]);
-        *reinterpret_cast<__nv_bfloat16*>(s.bw + tc::kmajor_offset(16 * c + j, t, MLP_TILE)) =
-            __float2bfloat16_rn(valid ? z[j] : 0.0f);
+      for (int j = 0; j < 32; j++) {
+        const float zz = z[j] + s.bias1[c0 + j], sg = logistic(zz), h = zz * sg;
+        d1[j] = sg + h * (1.0f - sg);
+        z[j] = h;
       }
-      tc::st_bf16x8(s.a2, tc::kmajor_offset(t, 16 * c, MLP_HID), z);
-      tc::st_bf16x8(s.a2, tc::kmajor_offset(t, 16 * c + 8, MLP_HID), z + 8);
+      tr_store32(s.hx, row, c0, TR_HX, z);
     }
     tr_sync();
     if (t == 0) {
 #pragma unroll
       for (int kb = 0; kb < 4; kb++)
-        tc::mma_bf16(s.tmem + TC_Z2, tc::kmajor_desc(tc::smem_addr(s.a2) + 256 * kb, MLP_HID),
-                     tc::kmajor_desc(tc::smem_addr(s.b2) + 256 * kb, MLP_HID), idesc64, kb > 0);
+        tc::mma_bf16(tm + TC_Z2, tc::kmajor_desc(hx + 256 * kb, TR_HX), tc::kmajor_desc(sb2 + 256 * kb, MLP_HID), idesc64,
+                     kb > 0);
       tc::mma_commit(&s.mbar);
     }
-    if (!tc::mbar_wait(&s.mbar, phase)) s.ok = 0;
-    phase ^= 1u;
-    tc::fence_after_sync();
-    // y, residual, dy = 2 (y - t) / n_total
-    float y = s.bias3;
+    wait();
+    // y from both halves' columns, residual, dy = 2 (y - t) / n_total
+    float h2[32], d2[32];
+    tc::tmem_ld32(tc::tmem_lane_addr(tm, quad, TC_Z2 + c0), h2);
+    {
+      float y = 0.0f;
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-      float z[16];
-      tc::tmem_ld16(tc::tmem_lane_addr(s.tmem, warp, TC_Z2 + 16 * c), z);
-#pragma unroll
-      for (int j = 0; j < 16; j++) y += s.w3[16 * c + j] * silu(z[j] + s.bias2[16 * c + j]);
-    }
-    const float r = valid ? (y - ti) : 0.0f;
-    const float dy = 2.0f * r * inv_n;
-    s.lsum[t] = r * r * inv_n;
-    s.dsum[t] = dy;
-    // dW3 = sum dy h2 ; dZ2 = dy w3 silu'(Z2 + b2) -> A3 (row t), Aw rows 0..63 (column t)
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-      float z[16], d[16];
-      tc::tmem_ld16(tc::tmem_lane_addr(s.tmem, warp, TC_Z2 + 16 * c), z);
-#pragma unroll
-      for (int j = 0; j < 16; j++) {
-        const float zz = z[j] + s.bias2[16 * c + j];
-        s.red[t][16 * c + j] = dy * silu(zz);
-        d[j] = dy * s.w3[16 * c + j] * dsilu(zz);
-        *reinterpret_cast<__nv_bfloat16*>(s.aw + tc::kmajor_offset(16 * c + j, t, MLP_TILE)) =
-            __float2bfloat16_rn(d[j]);
+      for (int j = 0; j < 32; j++) {
+        const float zz = h2[j] + s.bias2[c0 + j], sg = logistic(zz), w = s.w3[c0 + j];
+        h2[j] = zz * sg;
+        d2[j] = w * (sg + h2[j] * (1.0f - sg));
+        y += w * h2[j];
       }
-      tc::st_bf16x8(s.a3, tc::kmajor_offset(t, 16 * c, MLP_HID), d);
-      tc::st_bf16x8(s.a3, tc::kmajor_offset(t, 16 * c + 8, MLP_HID), d + 8);
+      s.ysum[half][row] = y;
     }
-    tr_colsum(s, s.acc_w3);
-    if (t == 0) {  // loss and db3 = sum dy, in sample order
-      float l = 0.0f, b = 0.0f;
-      for (int q = 0; q < MLP_TILE; q++) {
-        l += s.lsum[q];
-        b += s.dsum[q];
-      }
-      s.acc_loss += l;
-      s.acc_b3 += b;
+    __syncthreads();
+    const float res = valid ? (bias3 + s.ysum[0][row] + s.ysum[1][row] - ti) : 0.0f;
+    const float dy = 2.0f * res * inv_n;
+    if (half == 0) {
+      a_loss += res * res * inv_n;
+      a_b3 += dy;
     }
-    // db2 = sum dZ2 in FP32 (the BF16 copy in A3 is for the tensor core)
+    // dW3 = sum dy h2; dZ2 = dy w3 silu'(Z2 + b2), db2 = sum dZ2 in FP32 (the
+    // BF16 copy is for the tensor core)
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-      float z[16];
-      tc::tmem_ld16(tc::tmem_lane_addr(s.tmem, warp, TC_Z2 + 16 * c), z);
-#pragma unroll
-      for (int j = 0; j < 16; j++) s.red[t][16 * c + j] = dy * s.w3[16 * c + j] * dsilu(z[j] + s.bias2[16 * c + j]);
+    for (int j = 0; j < 32; j++) {
+      h2[j] *= dy;
+      d2[j] *= dy;
     }
-    tr_colsum(s, s.acc_b2);
+    tr_store32(s.dz, row, c0, TR_DZ, d2);
     tr_sync();
-    // dH1 = dZ2 W2
+    // dH1 = dZ2 W2 (W2's tile read along its rows), over Z2, which is read
     if (t == 0) {
 #pragma unroll
       for (int kb = 0; kb < 4; kb++)
-        tc::mma_bf16(s.tmem + TC_DH1, tc::kmajor_desc(tc::smem_addr(s.a3) + 256 * kb, MLP_HID),
-                     tc::kmajor_desc(tc::smem_addr(s.b2t) + 256 * kb, MLP_HID), idesc64, kb > 0);
+        tc::mma_bf16(tm + TC_DH1, tc::kmajor_desc(dz + 256 * kb, TR_DZ), tc::mnmajor_desc(sb2 + 2048 * kb, MLP_HID),
+                     idesc64 | tc::IDESC_B_MN, kb > 0);
       tc::mma_commit(&s.mbar);
     }
-    if (!tc::mbar_wait(&s.mbar, phase)) s.ok = 0;
-    phase ^= 1u;
-    tc::fence_after_sync();
-    // dZ1 = dH1 silu'(Z1 + b1) -> Aw rows 64..127 (column t); db1 = sum dZ1
+    a_w3 += tr_colsum(h2);
+    a_b2 += tr_colsum(d2);
+    wait();
+    // dZ1 = dH1 silu'(Z1 + b1), db1 = sum dZ1
+    {
+      float z[32];
+      tc::tmem_ld32(tc::tmem_lane_addr(tm, quad, TC_DH1 + c0), z);
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-      float z[16], h[16];
-      tc::tmem_ld16(tc::tmem_lane_addr(s.tmem, warp, TC_Z1 + 16 * c), z);
-      tc::tmem_ld16(tc::tmem_lane_addr(s.tmem, warp, TC_DH1 + 16 * c), h);
+      for (int j = 0; j < 32; j++) z[j] *= d1[j];
+      tr_store32(s.dz, row, 64 + c0, TR_DZ, z);
+      tr_sync();
+      // weight gradients: D[128 x 80] += [dZ2 | dZ1]^T [H1 | X], both tiles
+      // read along their rows; waited for before the tiles are written again
+      if (t == 0) {
 #pragma unroll
-      for (int j = 0; j < 16; j++) {
-        const float d = valid ? h[j] * dsilu(z[j] + s.bias1[16 * c + j]) : 0.0f;
-        s.red[t][16 * c + j] = d;
-        *reinterpret_cast<__nv_bfloat16*>(s.aw + tc::kmajor_offset(64 + 16 * c + j, t, MLP_TILE)) =
-            __float2bfloat16_rn(d);
+        for (int kb = 0; kb < MLP_TILE / 16; kb++)
+          tc::mma_bf16(tm + TC_DW, tc::mnmajor_desc(dz + 2 * (TR_DZ / 8) * 128 * kb, TR_DZ),
+                       tc::mnmajor_desc(hx + 2 * (TR_HX / 8) * 128 * kb, TR_HX),
+                       tc::make_idesc(128, TR_HX) | tc::IDESC_A_MN | tc::IDESC_B_MN, !(first && kb == 0));
+        tc::mma_commit(&s.mbar);
       }
+      a_b1 += tr_colsum(z);
     }
-    tr_colsum(s, s.acc_b1);
-    tr_sync();
-    // weight gradients: D[128 x 80] += Aw[128 x 128] Bw[80 x 128]^T
-    if (t == 0) {
-#pragma unroll
-      for (int kb = 0; kb < MLP_TILE / 16; kb++)
-        tc::mma_bf16(s.tmem + TC_DW, tc::kmajor_desc(tc::smem_addr(s.aw) + 256 * kb, MLP_TILE),
-                     tc::kmajor_desc(tc::smem_addr(s.bw) + 256 * kb, MLP_TILE), idesc80, !(first && kb == 0));
-      tc::mma_commit(&s.mbar);
-    }
-    if (!tc::mbar_wait(&s.mbar, phase)) s.ok = 0;
-    phase ^= 1u;
-    tc::fence_after_sync();
     first = false;
   }
-  // partial gradients of this CTA
+  if (!first) wait();
+  // partial gradients of this CTA (it has a tile: the grid is at most their number)
   float* out = part + (size_t)blockIdx.x * (NPARAMS + 1);
-  if (!first) {
+  {
     // rows 0..63 x columns 0..63: dW2[o][i]; rows 64..127 x columns 64..69: dW1[i][j]
-    if (warp < 2) {
+    float z[32];
+    if (quad < 2) {
+      tc::tmem_ld32(tc::tmem_lane_addr(tm, quad, TC_DW + c0), z);
 #pragma unroll
-      for (int c = 0; c < 4; c++) {
-        float z[16];
-        tc::tmem_ld16(tc::tmem_lane_addr(s.tmem, warp, TC_DW + 16 * c), z);
+      for (int j = 0; j < 32; j++) out[OFF_W2 + row * MLP_HID + c0 + j] = first ? 0.0f : z[j];
+    } else if (half == 0) {
+      tc::tmem_ld16(tc::tmem_lane_addr(tm, quad, TC_DW + 64), z);
 #pragma unroll
-        for (int j = 0; j < 16; j++) out[OFF_W2 + t * MLP_HID + 16 * c + j] = z[j];
-      }
-    } else {
-      float z[16];
-      tc::tmem_ld16(tc::tmem_lane_addr(s.tmem, warp, TC_DW + 64), z);
-#pragma unroll
-      for (int j = 0; j < MLP_IN; j++) out[OFF_W1 + (t - 64) * MLP_IN + j] = z[j];
+      for (int j = 0; j < MLP_IN; j++) out[OFF_W1 + (row - 64) * MLP_IN + j] = first ? 0.0f : z[j];
     }
-  } else {
-    for (int i = t; i < NP_W2; i += MLP_TILE) out[OFF_W2 + i] = 0.0f;
-    for (int i = t; i < NP_W1; i += MLP_TILE) out[OFF_W1 + i] = 0.0f;
   }
-  if (t < MLP_HID) {
-    out[OFF_B1 + t] = s.acc_b1[t];
-    out[OFF_B2 + t] = s.acc_b2[t];
-    out[OFF_W3 + t] = s.acc_w3[t];
+  s.colsum[quad][0][c0 + lane] = a_w3;
+  s.colsum[quad][1][c0 + lane] = a_b2;
+  s.colsum[quad][2][c0 + lane] = a_b1;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a_loss += __shfl_xor_sync(0xffffffffu, a_loss, o);
+    a_b3 += __shfl_xor_sync(0xffffffffu, a_b3, o);
   }
-  if (t == 0) {
-    out[OFF_B3] = s.acc_b3;
-    out[NPARAMS] = s.acc_loss;
+  if (half == 0 && lane == 0) {
+    s.lsum[quad] = a_loss;
+    s.dsum[quad] = a_b3;
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (t == 0 && !s.ok) atomicOr(status, (unsigned)ST_TIMEOUT);
-  if (t < 32) tc::tmem_dealloc(s.tmem, 512);
+  tc::fence_after_sync();
+  if (t < 3 * MLP_HID) {
+    const int a = t / MLP_HID, c = t % MLP_HID;
+    const int off = a == 0 ? OFF_W3 : (a == 1 ? OFF_B2 : OFF_B1);
+    out[off + c] = (s.colsum[0][a][c] + s.colsum[1][a][c]) + (s.colsum[2][a][c] + s.colsum[3][a][c]);
+  }
+  if (t == TR_THREADS - 1) {
+    out[OFF_B3] = (s.dsum[0] + s.dsum[1]) + (s.dsum[2] + s.dsum[3]);
+    out[NPARAMS] = (s.lsum[0] + s.lsum[1]) + (s.lsum[2] + s.lsum[3]);
+    if (!s.ok) atomicOr(status, (unsigned)ST_TIMEOUT);
+  }
+  if (t < 32) tc::tmem_dealloc(tm, TC_COLS);
 }
 
-// ordered sum of the per-CTA partials (bit reproducible)
-__global__ void k_mlp_reduce(const float* part, int nparts, float* grads) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i > NPARAMS) return;
+// The CTAs' partial gradients added in a fixed order (bit reproducible) and,
+// for a training step (lr > 0), Adam (Kingma & Ba) on the FP32 master
+// parameters and their BF16 copies: one launch where the sum, the step and a
+// one-CTA repack took three (20 us of a 110 us step at 2048 samples).  32
+// parameters per CTA; 8 groups of threads share a parameter's partials.
+struct AdamStep {
+  float *p, *m, *v;
+  MlpDevice* packed;
+  float lr, b1, b2, eps, c1, c2;
+};
+constexpr int RED_PARAMS = 32, RED_GROUPS = 8;
+__global__ void __launch_bounds__(RED_PARAMS * RED_GROUPS) k_mlp_reduce(const float* part, int nparts, float* grads,
+                                                                      AdamStep st) {
+  __shared__ float red[RED_GROUPS][RED_PARAMS];
+  const int lane = threadIdx.x % RED_PARAMS, g = threadIdx.x / RED_PARAMS;
+  const int i = blockIdx.x * RED_PARAMS + lane;
   float a = 0.0f;
-  for (int c = 0; c < nparts; c++) a += part[(size_t)c * (NPARAMS + 1) + i];
+  if (i <= NPARAMS) {
+    int c = g;
+    for (; c + 7 * RED_GROUPS < nparts; c += 8 * RED_GROUPS) {
+      float q[8];
+#pragma unroll
+      for (int u = 0; u < 8; u++) q[u] = part[(size_t)(c + u * RED_GROUPS) * (NPARAMS + 1) + i];
+#pragma unroll
+      for (int u = 0; u < 8; u++) a += q[u];
+    }
+    for (; c < nparts; c += RED_GROUPS) a += part[(size_t)c * (NPARAMS + 1) + i];
+  }
+  red[g][lane] = a;
+  __syncthreads();
+  if (g != 0 || i > NPARAMS) return;
+#pragma unroll
+  for (int q = 1; q < RED_GROUPS; q++) a += red[q][lane];
   grads[i] = a;
-}
-
-// Adam (Kingma & Ba) on the FP32 master parameters, then the BF16 repack
-__global__ void k_mlp_adam(float* p, const float* g, float* m, float* v, float lr, float b1, float b2, float eps,
-                           float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= NPARAMS) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.0f - b1) * gi;
-  const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  if (st.lr > 0.0f && i < NPARAMS) {
+    const float mi = st.b1 * st.m[i] + (1.0f - st.b1) * a;
+    const float vi = st.b2 * st.v[i] + (1.0f - st.b2) * a * a;
+    st.m[i] = mi;
+    st.v[i] = vi;
+    const float p = st.p[i] - st.lr * (mi / st.c1) / (sqrtf(vi / st.c2) + st.eps);
+    st.p[i] = p;
+    mlp_pack_one(i, p, st.packed);
+  }
 }
 
 // normalised features and pbar from face states (rhoL, uL, pL, rhoR, uR, pR)
@@ -569,19 +607,27 @@ int ensure_train(amm_mlp* m, int ctas) {
   return AMM_OK;
 }
 
-// gradients of the batch into m->grads (device), loss in m->grads[NPARAMS]
-int run_grads(amm_mlp* m, const float* x, const float* t, const int* idx, int64_t n) {
+// gradients of the batch into m->grads (device), loss in m->grads[NPARAMS];
+// lr > 0: also an Adam step with them
+int run_grads(amm_mlp* m, const float* x, const float* t, const int* idx, int64_t n, float lr) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t tiles = (n + amm::MLP_TILE - 1) / amm::MLP_TILE;
-  const int ctas = (int)std::min<int64_t>(tiles, (int64_t)sms);
+  const int ctas = (int)std::min<int64_t>(tiles, 2 * (int64_t)sms);   // two per SM
   int rc = ensure_train(m, ctas);
   if (rc != AMM_OK) return rc;
-  amm::k_mlp_grads<<<ctas, amm::MLP_TILE, train_smem_bytes(), m->stream>>>(m->packed, x, t, idx, n, 1.0f / (float)n,
+  amm::k_mlp_grads<<<ctas, amm::TR_THREADS, train_smem_bytes(), m->stream>>>(m->packed, x, t, idx, n, 1.0f / (float)n,
                                                                           m->partial, m->status);
   MCU(cudaGetLastError());
-  amm::k_mlp_reduce<<<(amm::NPARAMS + 256) / 256, 256, 0, m->stream>>>(m->partial, ctas, m->grads);
+  amm::AdamStep st{m->params, m->adam_m, m->adam_v, m->packed, lr, 0.9f, 0.999f, 1e-8f, 1.0f, 1.0f};
+  if (lr > 0.0f) {
+    m->adam_t++;
+    st.c1 = 1.0f - powf(st.b1, (float)m->adam_t);
+    st.c2 = 1.0f - powf(st.b2, (float)m->adam_t);
+  }
+  amm::k_mlp_reduce<<<(amm::NPARAMS + amm::RED_PARAMS) / amm::RED_PARAMS, amm::RED_PARAMS * amm::RED_GROUPS, 0,
+                      m->stream>>>(m->partial, ctas, m->grads, st);
   MCU(cudaGetLastError());
   return AMM_OK;
 }
@@ -606,6 +652,7 @@ int amm_mlp_create(amm_mlp** out, double gamma, void* stream) {
   if (cudaMalloc(&m->packed, sizeof(amm::MlpDevice)) != cudaSuccess) return bail(AMM_ERR_CUDA);
   if (cudaMalloc(&m->status, sizeof(unsigned)) != cudaSuccess) return bail(AMM_ERR_CUDA);
   if (cudaMemset(m->params, 0, sizeof(float) * amm::NPARAMS) != cudaSuccess) return bail(AMM_ERR_CUDA);
+  if (cudaMemset(m->packed, 0, sizeof(amm::MlpDevice)) != cudaSuccess) return bail(AMM_ERR_CUDA);
   if (cudaMemset(m->status, 0, sizeof(unsigned)) != cudaSuccess) return bail(AMM_ERR_CUDA);
   if (cudaFuncSetAttribute(amm::k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem_bytes()) !=
       cudaSuccess)
@@ -635,7 +682,7 @@ int amm_mlp_set_params(amm_mlp* m, const float* params) {
   for (int i = 0; i < amm::NPARAMS; i++)
     if (!std::isfinite(params[i])) return mfail(m, AMM_ERR_INVALID_ARG, "non-finite parameter");
   MCU(cudaMemcpyAsync(m->params, params, sizeof(float) * amm::NPARAMS, cudaMemcpyHostToDevice, m->stream));
-  amm::k_mlp_pack<<<1, 256, 0, m->stream>>>(m->params, m->packed);
+  amm::k_mlp_pack<<<(amm::NPARAMS + 255) / 256, 256, 0, m->stream>>>(m->params, m->packed);
   MCU(cudaGetLastError());
   MCU(cudaStreamSynchronize(m->stream));
   return AMM_OK;
@@ -664,7 +711,7 @@ int amm_mlp_forward(amm_mlp* m, const float* x_device, int64_t n, float* y_devic
 int amm_mlp_grads(amm_mlp* m, const float* x_device, const float* t_device, const int32_t* idx_device, int64_t n,
                   float* grads, float* loss) {
   if (!m || !x_device || !t_device || n < 1 || !grads) return mfail(m, AMM_ERR_INVALID_ARG, "bad argument");
-  int rc = run_grads(m, x_device, t_device, idx_device, n);
+  int rc = run_grads(m, x_device, t_device, idx_device, n, 0.0f);
   if (rc != AMM_OK) return rc;
   std::vector<float> g(amm::NPARAMS + 1);
   unsigned st = 0;
@@ -680,16 +727,8 @@ int amm_mlp_grads(amm_mlp* m, const float* x_device, const float* t_device, cons
 int amm_mlp_train_step(amm_mlp* m, const float* x_device, const float* t_device, const int32_t* idx_device, int64_t n,
                        float lr, float* loss_device) {
   if (!m || !x_device || !t_device || n < 1 || !(lr > 0.0f)) return mfail(m, AMM_ERR_INVALID_ARG, "bad argument");
-  int rc = run_grads(m, x_device, t_device, idx_device, n);
+  int rc = run_grads(m, x_device, t_device, idx_device, n, lr);
   if (rc != AMM_OK) return rc;
-  m->adam_t++;
-  const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = 1.0f - powf(b1, (float)m->adam_t), c2 = 1.0f - powf(b2, (float)m->adam_t);
-  amm::k_mlp_adam<<<(amm::NPARAMS + 255) / 256, 256, 0, m->stream>>>(m->params, m->grads, m->adam_m, m->adam_v, lr, b1,
-                                                                    b2, 1e-8f, c1, c2);
-  MCU(cudaGetLastError());
-  amm::k_mlp_pack<<<1, 256, 0, m->stream>>>(m->params, m->packed);
-  MCU(cudaGetLastError());
   if (loss_device)
     MCU(cudaMemcpyAsync(loss_device, m->grads + amm::NPARAMS, sizeof(float), cudaMemcpyDeviceToDevice, m->stream));
   return AMM_OK;
