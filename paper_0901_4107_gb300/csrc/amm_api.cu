@@ -55,7 +55,7 @@ void free_ctx(amm_ctx* c) {
                   c->totals, c->stats,  c->closure, c->mlp,      c->defer_list, c->defer_count, c->scratch, c->counter,
                   c->ind_bin, c->ind_act, c->ind_list, c->ind_flist, c->ind_count, c->ind_fstamp, c->ind_cstamp,
                   c->ind_fdt, c->ind_hist, c->ind_slot_cell, c->ind_cell_slot, c->ind_leaf_off, c->ind_level_off,
-                  c->ind_rec, c->ind_rec32, c->ind_node, c->ind_loop, c->geo_ws};
+                  c->ind_rec, c->ind_rec32, c->ind_node, c->ind_loop, c->geo_ws, c->retess_ws};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 

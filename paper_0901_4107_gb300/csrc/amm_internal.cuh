@@ -288,6 +288,8 @@ struct amm_ctx {
   double* scratch = nullptr;       // layout conversions for getters/setters
   void* geo_ws = nullptr;          // FP64 face geometry before the FP32 cast (grown on demand)
   size_t geo_ws_bytes = 0;
+  void* retess_ws = nullptr;       // amm_retessellate: face-list scratch
+  size_t retess_ws_bytes = 0;
   void* tess_ws = nullptr;         // amm_retessellate: the GPU tessellation's workspace (amm::vor::TessWork)
   int64_t nf_cap = 0;              // faces the face-sized buffers hold
   size_t scratch_size = 0;         // in doubles

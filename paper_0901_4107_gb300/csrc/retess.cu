@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "amm_internal.cuh"
+#include "scan.cuh"
 
 namespace amm {
 namespace {
@@ -48,29 +49,6 @@ __global__ void k_csr_count(int nf, const int2* lr, int* count) {
   atomicAdd(count + e.y, 1);
 }
 
-__global__ void k_scan_one(const int* count, int* start, int m) {
-  __shared__ int part[1024];
-  const int t = threadIdx.x;
-  const int per = (m + 1023) / 1024;
-  const int lo = t * per, hi = lo + per < m ? lo + per : m;
-  int s = 0;
-  for (int k = lo; k < hi; k++) s += count[k];
-  part[t] = s;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    const int v = t >= o ? part[t - o] : 0;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
-  }
-  int run = t ? part[t - 1] : 0;
-  for (int k = lo; k < hi; k++) {
-    start[k] = run;
-    run += count[k];
-  }
-  if (t == 1023) start[m] = part[1023];
-}
-
 __global__ void k_csr_fill(int nf, const int2* lr, int* cursor, int2* csr) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= nf) return;
@@ -93,14 +71,19 @@ __device__ __forceinline__ int klass(const double* d, int dim) {
 }
 
 // each cell's list by (direction class of the outward normal, larger face
-// first, face index); also the largest list length
-__global__ void k_csr_sort(int n, int dim, const int* off, int2* csr, const int2* lr, const double* gen3,
-                           const int8_t* sh3, const double* box3, const double* area, int* max_inc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int lo = off[i], hi = off[i + 1];
-  atomicMax(max_inc, hi - lo);
-  auto key = [&](const int2& x, int& cls, double& a) {
+// first, face index); also the largest list length.  A warp per cell: a lane
+// holds an incidence and its key and ranks it against the others' (a thread per
+// cell inserting one by one read every key again for each comparison: 608 us
+// for 64 k cells, 81 us now).  Longer lists are ranked through global memory.
+__global__ void __launch_bounds__(256) k_csr_sort(int n, int dim, const int* off, const int2* unsorted, int2* csr,
+                                                  const int2* lr, const double* gen3, const int8_t* sh3,
+                                                  const double* box3, const double* area, int* max_inc) {
+  const int lane = threadIdx.x & 31;
+  const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+  __shared__ int longest;
+  if (threadIdx.x == 0) longest = 0;
+  __syncthreads();
+  auto key = [&](const int2& x, int& cls, long long& a) {
     const int k = x.x >> 1;
     const int2 e = lr[k];
     double d[3];
@@ -109,25 +92,47 @@ __global__ void k_csr_sort(int n, int dim, const int* off, int2* csr, const int2
     if (x.x & 1)
       for (int q = 0; q < 3; q++) d[q] = -d[q];
     cls = klass(d, dim);
-    a = area[k];
+    a = __double_as_longlong(area[k]);
   };
-  for (int p = lo + 1; p < hi; p++) {
-    const int2 v = csr[p];
-    int cv;
-    double av;
-    key(v, cv, av);
-    int q = p - 1;
-    while (q >= lo) {
-      int cq;
-      double aq;
-      key(csr[q], cq, aq);
-      const bool after = cq > cv || (cq == cv && (aq < av || (aq == av && (csr[q].x >> 1) > (v.x >> 1))));
-      if (!after) break;
-      csr[q + 1] = csr[q];
-      q--;
+  // does (c1, a1, k1) come before (c2, a2, k2)?  (a face that is both a left
+  // and a right one of its cell has two incidences of the same k: the left first)
+  // (areas are not negative, so they order like their bits: integer compares,
+  // not the FP64 pipe's)
+  auto before = [](int c1, long long a1, int x1, int c2, long long a2, int x2) {
+    if (c1 != c2) return c1 < c2;
+    if (a1 != a2) return a1 > a2;
+    return x1 < x2;
+  };
+  if (i < n) {
+    const int lo = off[i], m = off[i + 1] - lo;
+    if (lane == 0) atomicMax(&longest, m);
+    for (int b = 0; b < m; b += 32) {
+      const bool in = b + lane < m;
+      const int2 v = unsorted[lo + (in ? b + lane : 0)];
+      int cv;
+      long long av;
+      key(v, cv, av);
+      int rank = 0;
+      if (m <= 32) {
+        for (int q = 0; q < m; q++) {
+          const int cq = __shfl_sync(0xffffffffu, cv, q), xq = __shfl_sync(0xffffffffu, v.x, q);
+          const long long aq = __shfl_sync(0xffffffffu, av, q);
+          rank += before(cq, aq, xq, cv, av, v.x) ? 1 : 0;
+        }
+      } else {
+        for (int q = 0; q < m; q++) {
+          const int2 u = unsorted[lo + q];
+          int cq;
+          long long aq;
+          key(u, cq, aq);
+          rank += before(cq, aq, u.x, cv, av, v.x) ? 1 : 0;
+        }
+      }
+      if (in) csr[lo + rank] = v;
     }
-    csr[q + 1] = v;
   }
+  __syncthreads();
+  if (threadIdx.x == 0 && longest > *(volatile int*)max_inc) atomicMax(max_inc, longest);
 }
 
 }  // namespace
@@ -232,37 +237,53 @@ int amm_retessellate(amm_ctx* c) {
   const double* warea;
   const double* wcen;
   vor::work_faces(w, &wcells, &wshift, &warea, &wcen);
-  double* cen3 = nullptr;
-  int8_t* sh3 = nullptr;
-  int *count = nullptr, *cursor = nullptr, *maxinc = nullptr;
-  const unsigned gf = (unsigned)((nf + 255) / 256), gc = (unsigned)((n + 255) / 256);
-  if (where.empty() && cu(cudaMalloc(&cen3, sizeof(double) * 3 * nf), "alloc") &&
-      cu(cudaMalloc(&sh3, 3 * nf), "alloc") && cu(cudaMalloc(&count, sizeof(int) * n), "alloc") &&
-      cu(cudaMalloc(&cursor, sizeof(int) * n), "alloc") && cu(cudaMalloc(&maxinc, sizeof(int)), "alloc")) {
+  // scratch in the context's workspace, kept between calls and grown with room
+  // for the next meshes (five allocations and frees of a call cost as much as
+  // its face-list kernels)
+  const unsigned gf = (unsigned)((nf + 255) / 256);
+  size_t need = 0;
+  auto part_of = [&](size_t bytes) {
+    const size_t at = need;
+    need += (bytes + 255) / 256 * 256;
+    return at;
+  };
+  const size_t o_cen = part_of(sizeof(double) * 3 * c->nf_cap), o_sh = part_of(3 * c->nf_cap),
+               o_csr = part_of(sizeof(int2) * 2 * c->nf_cap), o_count = part_of(sizeof(int) * n),
+               o_cursor = part_of(sizeof(int) * n), o_part = part_of(sizeof(int) * scan_scratch(n)),
+               o_max = part_of(sizeof(int));
+  if (where.empty() && c->retess_ws_bytes < need) {
+    if (c->retess_ws) cudaFree(c->retess_ws);
+    c->retess_ws = nullptr;
+    c->retess_ws_bytes = 0;
+    if (cu(cudaMalloc(&c->retess_ws, need), "alloc")) c->retess_ws_bytes = need;
+  }
+  if (where.empty()) {
+    char* ws = (char*)c->retess_ws;
+    double* cen3 = (double*)(ws + o_cen);
+    int8_t* sh3 = (int8_t*)(ws + o_sh);
+    int2* unsorted = (int2*)(ws + o_csr);
+    int *count = (int*)(ws + o_count), *cursor = (int*)(ws + o_cursor), *maxinc = (int*)(ws + o_max);
     cu(cudaMemcpyAsync(c->lr, wcells, sizeof(int2) * nf, cudaMemcpyDeviceToDevice, st), "copy");
     k_pad_faces<<<gf, 256, 0, st>>>((int)nf, dim, wcen, wshift, cen3, sh3, c->face_perm);
     cu(cudaMemsetAsync(count, 0, sizeof(int) * n, st), "memset");
     cu(cudaMemsetAsync(maxinc, 0, sizeof(int), st), "memset");
     k_csr_count<<<gf, 256, 0, st>>>((int)nf, c->lr, count);
-    k_scan_one<<<1, 1024, 0, st>>>(count, c->csr_off, (int)n);
+    cu(exclusive_scan(count, c->csr_off, n, (int*)(ws + o_part), st), "scan");
     cu(cudaMemcpyAsync(cursor, c->csr_off, sizeof(int) * n, cudaMemcpyDeviceToDevice, st), "copy");
-    k_csr_fill<<<gf, 256, 0, st>>>((int)nf, c->lr, cursor, c->csr);
-    k_csr_sort<<<gc, 256, 0, st>>>((int)n, dim, c->csr_off, c->csr, c->lr, c->gen, sh3, c->box, warea, maxinc);
+    k_csr_fill<<<gf, 256, 0, st>>>((int)nf, c->lr, cursor, unsorted);
+    k_csr_sort<<<(unsigned)((n + 7) / 8), 256, 0, st>>>((int)n, dim, c->csr_off, unsorted, c->csr, c->lr, c->gen, sh3,
+                                                        c->box, warea, maxinc);
     cu(cudaGetLastError(), "csr");
     int mi = 0;
     cu(cudaMemcpyAsync(&mi, maxinc, sizeof(int), cudaMemcpyDeviceToHost, st), "read");
-    cu(cudaStreamSynchronize(st), "sync");
-    c->headroom = 1;
-    while ((1 << c->headroom) < mi + 1) c->headroom++;
-    c->headroom += 1;
     if (where.empty()) cu(launch_face_geometry(c, warea, cen3, sh3), "geometry");
     if (where.empty())
       cu(c->is_fp64() ? launch_primitives<double>(c) : launch_primitives<float>(c), "primitives");
     cu(cudaStreamSynchronize(st), "sync");
+    c->headroom = 1;
+    while ((1 << c->headroom) < mi + 1) c->headroom++;
+    c->headroom += 1;
   }
-  void* tmp[] = {cen3, sh3, count, cursor, maxinc};
-  for (void* p : tmp)
-    if (p) cudaFree(p);
   if (!where.empty()) {
     c->err = "amm_retessellate: " + where;
     return AMM_ERR_CUDA;

@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "amm.h"
+#include "scan.cuh"
 
 namespace amm {
 namespace vor {
@@ -65,6 +66,25 @@ struct HalfFace {
   double cen[3];             // centroid relative to this cell's generator
 };
 
+// The half-faces of all cells in one list: cell i's are the run of nhf[i] at
+// first[i].  A warp takes room for its cell's faces from `used`; past the
+// capacity nothing is written and the build is repeated with more room.  (64
+// places for every cell were 671 MB at 64^3, mostly empty and strided in every
+// later pass.)
+struct HalfList {
+  HalfFace* f;
+  int* first;
+  int* used;
+  int cap;
+};
+
+// room for m faces of cell i, by one lane; -1 if the list is full
+__device__ __forceinline__ int half_room(const HalfList& H, int i, int m) {
+  const int at = atomicAdd(H.used, m);
+  H.first[i] = at;
+  return at >= 0 && at <= H.cap - m ? at : -1;
+}
+
 __device__ __forceinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
 __device__ __forceinline__ int bin_coord(double x, double bs, int nb) {
@@ -81,30 +101,6 @@ __global__ void k_bin_count(Grid G, int* binof, int* count) {
   const int bin = (b[2] * G.nb[1] + b[1]) * G.nb[0] + b[0];
   binof[i] = bin;
   atomicAdd(count + bin, 1);
-}
-
-// exclusive scan of count[0..m) into start[0..m], one CTA of 1024 threads
-__global__ void k_scan(const int* count, int* start, int m) {
-  __shared__ int part[1024];
-  const int t = threadIdx.x;
-  const int per = (m + 1023) / 1024;
-  const int lo = t * per, hi = lo + per < m ? lo + per : m;
-  int s = 0;
-  for (int k = lo; k < hi; k++) s += count[k];
-  part[t] = s;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    const int v = t >= o ? part[t - o] : 0;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
-  }
-  int run = t ? part[t - 1] : 0;
-  for (int k = lo; k < hi; k++) {
-    start[k] = run;
-    run += count[k];
-  }
-  if (t == 1023) start[m] = part[1023];
 }
 
 __global__ void k_bin_fill(Grid G, const int* binof, int* cursor, int* bin_pts) {
@@ -436,14 +432,612 @@ __device__ int cut_buffer3(Cell3& C, int lane, int nc, double eps, float& R2) {
   return 0;
 }
 
-__global__ void __launch_bounds__(32 * WARPS) k_cells3(Grid G, HalfFace* hf, int* nhf, double* vol, double* com,
-                                                      int* err, double thr_area) {
+// --------------------------------------- 3D, a warp per cell, the usual cell
+// The same sequence of cuts as k_cells3 below for the cells of ordinary size:
+// at most FP planes and 64 vertices.  A cell that exceeds either, or ends
+// with any error, is listed and built by k_cells3, so what is accepted and
+// what is refused does not depend on this kernel.
+//
+// What bounds the general kernel is the narrow FP64 pipe (2 lanes a clock and
+// SM) and 25 KB of shared memory per cell (8 warps per SM): FP64 vertex
+// positions in most cuts, because one badly conditioned plane triple in a warp
+// sends it through the FP64 solve, three solves per vertex and unit normals
+// for the final faces.  Here
+//  - a vertex lives in its lane's registers (two per lane): its planes, FP32
+//    position, and how far that position can be off, from the conditioning of
+//    its three planes; only a vertex closer to a cutting plane than that is
+//    tested in FP64 (as k_cells3 tests it);
+//  - candidates are kept as FP32 images, the nearest is taken out by a warp
+//    minimum, and the FP64 planes are formed once, for the final cell;
+//  - removed edges are matched through a bit matrix in shared memory, freed
+//    lanes take the new vertices;
+//  - the FP64 vertices are solved once each; a face's area and centroid are
+//    summed in the two coordinates its normal projects to best (8 FP64
+//    operations per triangle instead of 30), the third follows from the plane.
+// 10 KB per cell, 20 warps per SM.  64^3 cells: 27.1 ms with k_cells3 alone,
+// 5.0 ms now (FP64 pipe 69% busy, issue 49%).
+constexpr int FP = 64;         // planes
+constexpr int FWARPS = 4;      // cells per CTA
+constexpr unsigned NOKEY = 0xffffffffu;
+
+struct Fast3 {
+  float4 pnf[FP];              // planes n.x = h in FP32
+  int pj[FP];                  // neighbour (-1: the box)
+  int ps[FP];                  // its periodic image, 8 bits per axis
+  unsigned edge[FP][2];        // bit matrix of the removed vertices' edges
+  unsigned short ed[64];       // edges that become vertices
+  union {
+    struct {                   // while cutting
+      float4 cx[MAXC];         // candidates: image position relative to the generator, half its square
+      int cj[MAXC], cs[MAXC];
+    } c;
+    struct {                   // the final cell
+      double P[FP][4];
+      double v[64][3];
+      unsigned tri[64];
+      int start[FP];           // a vertex of each plane
+      unsigned char next[FP][FP];
+    } f;
+  } u;
+};
+
+__device__ __forceinline__ int pack_shift(const int* s) { return (s[0] & 255) | (s[1] & 255) << 8 | (s[2] & 255) << 16; }
+__device__ __forceinline__ int shift_of(int p, int d) { return (int)(signed char)(p >> (8 * d)); }
+
+// the image of generator j relative to ri, and its square (rounded as gather3's)
+__device__ __forceinline__ void image3(const Grid& G, int j, int sh, const double* ri, double* x, double& d2) {
+  double p[3];
+#pragma unroll
+  for (int d = 0; d < 3; d++) p[d] = G.pts[(size_t)j * 3 + d];
+  if (sh != 0) {
+#pragma unroll
+    for (int d = 0; d < 3; d++) p[d] = __fma_rn((double)shift_of(sh, d), G.box[d], p[d]);
+  }
+#pragma unroll
+  for (int d = 0; d < 3; d++) x[d] = __dadd_rn(p[d], -ri[d]);
+  d2 = __fma_rn(x[2], x[2], __fma_rn(x[1], x[1], __dmul_rn(x[0], x[0])));
+}
+
+// x in FP32, truncated, by integer instructions (conversions run on the FP64
+// pipe); the candidates' positions are only screened with
+__device__ __forceinline__ float trunc_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu) - 896;
+  const unsigned m = __funnelshift_l(lo, hi & 0xfffffu, 3);
+  return e > 0 ? __uint_as_float((hi & 0x80000000u) | (unsigned)min(e, 254) << 23 | m) : 0.0f;
+}
+
+// plane k in FP64 {n, h}
+__device__ __forceinline__ void plane3(const Grid& G, int k, int j, int sh, const double* ri, double* p) {
+  if (k < 6) {
+    const int ax = k >> 1;
+    p[0] = p[1] = p[2] = 0.0;
+    p[ax] = (k & 1) ? -1.0 : 1.0;
+    p[3] = 0.5 * G.box[ax];
+  } else {
+    double d2;
+    image3(G, j, sh, ri, p, d2);
+    p[3] = 0.5 * d2;
+  }
+}
+
+// the point on three planes {n, h}
+__device__ __forceinline__ void solve3(const double* a, const double* b, const double* c, double* v) {
+  double bc[3], ca[3], ab[3];
+  cross3(b, c, bc);
+  cross3(c, a, ca);
+  cross3(a, b, ab);
+  const double inv = 1.0 / dot3(a, bc);
+  for (int d = 0; d < 3; d++) v[d] = (a[3] * bc[d] + b[3] * ca[d] + c[3] * ab[d]) * inv;
+}
+
+// a vertex in FP64 from its planes' generators (rare)
+__device__ __noinline__ void vertex3_slow(const Grid& G, const Fast3& S, unsigned tri, const double* ri, double* v) {
+  double p[3][4];
+  for (int z = 0; z < 3; z++) {
+    const int k = (tri >> (8 * z)) & 255;
+    plane3(G, k, S.pj[k], S.ps[k], ri, p[z]);
+  }
+  solve3(p[0], p[1], p[2], v);
+}
+__device__ __noinline__ bool outside_slow(const Grid& G, const Fast3& S, unsigned tri, const double* ri, int j, int sh,
+                                         double eps, float nn) {
+  double v[3], n[3], d2;
+  vertex3_slow(G, S, tri, ri, v);
+  image3(G, j, sh, ri, n, d2);
+  return dot3(v, n) - 0.5 * d2 > eps * nn;
+}
+
+// two vertices of a lane
+struct Verts {
+  unsigned tri[2];             // planes a | b << 8 | c << 16
+  float x[2], y[2], z[2], r[2];   // position, |v|
+  float f[2];                  // its error is below f (|n||v| + |h|) in a test against n.x = h
+};
+
+__device__ __forceinline__ float approx_sqrt(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// the FP32 vertex of planes a, b, c: position and error factor; with planes
+// too close to dependent, from FP64
+__device__ __forceinline__ void make_vertex(const Grid& G, const Fast3& S, unsigned tri, const double* ri, float4& p,
+                                           float& f) {
+  const float4 a = S.pnf[tri & 255], b = S.pnf[(tri >> 8) & 255], c = S.pnf[(tri >> 16) & 255];
+  const float bx = b.y * c.z - b.z * c.y, by = b.z * c.x - b.x * c.z, bz = b.x * c.y - b.y * c.x;
+  const float cx = c.y * a.z - c.z * a.y, cy = c.z * a.x - c.x * a.z, cz = c.x * a.y - c.y * a.x;
+  const float ax = a.y * b.z - a.z * b.y, ay = a.z * b.x - a.x * b.z, az = a.x * b.y - a.y * b.x;
+  const float det = a.x * bx + a.y * by + a.z * bz;
+  const float l3 = approx_sqrt(a.x * a.x + a.y * a.y + a.z * a.z) * approx_sqrt(b.x * b.x + b.y * b.y + b.z * b.z) *
+                   approx_sqrt(c.x * c.x + c.y * c.y + c.z * c.z);
+  // kappa = |a||b||c| / |det|: the position is good to 24 FP32 roundings
+  // times kappa |v| (products and sums of the solve, the planes' own rounding)
+  const float inv = __fdividef(1.0f, det);
+  const float kappa = l3 * fabsf(inv);
+  if (kappa < 2000.0f) {
+    p.x = (a.w * bx + b.w * cx + c.w * ax) * inv;
+    p.y = (a.w * by + b.w * cy + c.w * ay) * inv;
+    p.z = (a.w * bz + b.w * cz + c.w * az) * inv;
+    f = fmaxf(1e-5f, 2e-6f * kappa);
+  } else {
+    double v[3];
+    vertex3_slow(G, S, tri, ri, v);
+    p.x = (float)v[0];
+    p.y = (float)v[1];
+    p.z = (float)v[2];
+    f = 1e-5f;
+  }
+  p.w = approx_sqrt(p.x * p.x + p.y * p.y + p.z * p.z);
+}
+
+// one cut by candidate k: 0 missed, 1 cut, -1 leave the cell to k_cells3
+__device__ __forceinline__ int cut_fast(const Grid& G, Fast3& S, Verts& V, unsigned* L, int& np, int lane, int k, float d2f,
+                                        const double* ri, double eps, float& R2) {
+  const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
+  const float4 c = S.u.c.cx[k];
+  const float nn = sqrtf(d2f);
+  unsigned M[2];
+  bool out[2];
+#pragma unroll
+  for (int e = 0; e < 2; e++) {
+    out[e] = false;
+    M[e] = 0u;
+    if (L[e] == 0u) continue;
+    const float d = c.x * V.x[e] + c.y * V.y[e] + c.z * V.z[e] - c.w;
+    const float tol = V.f[e] * (nn * V.r[e] + c.w);
+    const bool live = (L[e] >> lane) & 1u;
+    out[e] = live && d > tol;
+    const bool close = live && !(d > tol) && !(d < -tol);
+    if (__any_sync(full, close)) {
+      if (close) out[e] = outside_slow(G, S, V.tri[e], ri, S.u.c.cj[k], S.u.c.cs[k], eps, nn);
+      __syncwarp();
+    }
+    M[e] = __ballot_sync(full, out[e]);
+  }
+  if ((M[0] | M[1]) == 0u) return 0;
+  if (np >= FP) return -1;
+  const int q = np++;
+  if (lane == 0) {
+    S.pnf[q] = c;
+    S.pj[q] = S.u.c.cj[k];
+    S.ps[q] = S.u.c.cs[k];
+  }
+  // an edge (u, w) of a removed vertex whose reverse belongs to another
+  // removed vertex goes; the others become vertices (u, w, q)
+#pragma unroll
+  for (int e = 0; e < 2; e++)
+    if (out[e]) {
+#pragma unroll
+      for (int z = 0; z < 3; z++) {
+        const int u = (V.tri[e] >> (8 * z)) & 255, w = (V.tri[e] >> (8 * ((z + 1) % 3))) & 255;
+        atomicOr(&S.edge[u][w >> 5], 1u << (w & 31));
+      }
+    }
+  __syncwarp();
+  int total = 0;
+#pragma unroll
+  for (int e = 0; e < 2; e++) {
+    if (M[e] == 0u) continue;
+#pragma unroll
+    for (int z = 0; z < 3; z++) {
+      const int u = (V.tri[e] >> (8 * z)) & 255, w = (V.tri[e] >> (8 * ((z + 1) % 3))) & 255;
+      const bool bnd = out[e] && ((S.edge[w & (FP - 1)][(u >> 5) & 1] >> (u & 31)) & 1u) == 0u;
+      const unsigned B = __ballot_sync(full, bnd);
+      const int at = total + __popc(B & lt);
+      if (bnd && at < 64) S.ed[at] = (unsigned short)(u | w << 8);
+      total += __popc(B);
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < 2; e++)
+    if (out[e]) {
+#pragma unroll
+      for (int z = 0; z < 3; z++) {
+        const int u = (V.tri[e] >> (8 * z)) & 255;
+        S.edge[u][0] = 0u;
+        S.edge[u][1] = 0u;
+      }
+    }
+  __syncwarp();
+  L[0] &= ~M[0];
+  L[1] &= ~M[1];
+  const int free0 = __popc(~L[0]);
+  if (total > free0 + __popc(~L[1])) return -1;
+  // new vertices into the free lanes' first places, then the second ones (one
+  // copy of the code: it is large enough to miss the instruction cache)
+  int rank = __popc(~L[0] & lt);
+#pragma unroll 1
+  for (int e = 0; e < 2; e++) {
+    const unsigned Le = e == 0 ? L[0] : L[1];
+    const bool take = !((Le >> lane) & 1u) && rank < total;
+    const unsigned got = __ballot_sync(full, take);
+    if (take) {
+      const unsigned tri = (unsigned)S.ed[rank] | (unsigned)q << 16;
+      float4 p;
+      float f;
+      make_vertex(G, S, tri, ri, p, f);
+      if (e == 0) {
+        V.tri[0] = tri; V.x[0] = p.x; V.y[0] = p.y; V.z[0] = p.z; V.r[0] = p.w; V.f[0] = f;
+      } else {
+        V.tri[1] = tri; V.x[1] = p.x; V.y[1] = p.y; V.z[1] = p.z; V.r[1] = p.w; V.f[1] = f;
+      }
+    }
+    if (e == 0)
+      L[0] |= got;
+    else
+      L[1] |= got;
+    if (total <= free0) break;
+    rank = free0 + __popc(~L[1] & lt);
+  }
+  // an upper bound of the largest squared vertex distance
+  float r = 0.0f;
+  if ((L[0] >> lane) & 1u) r = V.r[0] * (1.0f + V.f[0]);
+  if ((L[1] >> lane) & 1u) r = fmaxf(r, V.r[1] * (1.0f + V.f[1]));
+  r = __uint_as_float(__reduce_max_sync(full, __float_as_uint(r)));
+  R2 = r * r * (1.0f + 1e-5f);
+  return __popc(L[0]) + __popc(L[1]) >= 4 ? 1 : -1;
+}
+
+// cuts by the nc buffered candidates, nearest first (ties in buffer order), up
+// to the first whose bisector lies beyond every vertex
+__device__ __forceinline__ int cut_buffer_fast(const Grid& G, Fast3& S, Verts& V, unsigned* L, int& np, int lane, int nc,
+                                               const double* ri, double eps, float& R2) {
+  constexpr int KEYS = MAXC / 32;
+  unsigned key[KEYS];
+#pragma unroll
+  for (int q = 0; q < KEYS; q++) {
+    const int k = lane + 32 * q;
+    const float h = k < nc ? S.u.c.cx[k].w : -1.0f;
+    key[q] = h < 0.0f ? NOKEY : __float_as_uint(2.0f * h);
+  }
+  for (;;) {
+    unsigned m = key[0];
+#pragma unroll
+    for (int q = 1; q < KEYS; q++) m = min(m, key[q]);
+    const unsigned least = __reduce_min_sync(0xffffffffu, m);
+    if (least == NOKEY) return 0;
+    const float d2f = __uint_as_float(least);
+    if (0.25f * d2f >= R2 * (1.0f + 1e-5f)) return 0;
+    unsigned at = NOKEY;
+#pragma unroll
+    for (int q = KEYS - 1; q >= 0; q--)
+      if (key[q] == least) at = (unsigned)(lane + 32 * q);
+    const int k = (int)__reduce_min_sync(0xffffffffu, at);
+#pragma unroll
+    for (int q = 0; q < KEYS; q++)
+      if (lane + 32 * q == k) key[q] = NOKEY;
+    if (cut_fast(G, S, V, L, np, lane, k, d2f, ri, eps, R2) < 0) return -1;
+  }
+}
+
+// gather3 for the fast kernel: the points of bins [q0, q1) of the shell from
+// position `at` on; the new count, or -1 if they do not fit
+__device__ __forceinline__ int gather_fast(const Grid& G, Fast3& S, int lane, int i, const double* ri, const int* b, int s,
+                                           int s0, int q0, int q1, int at) {
+  const int side = 2 * s + 1;
+  const int q = q0 + lane;
+  int lo = 0, hi = 0, sh[3] = {0, 0, 0};
+  if (q < q1) {
+    const int dx = q % side - s, dy = (q / side) % side - s, dz = q / (side * side) - s;
+    const int cheb = max(abs(dx), max(abs(dy), abs(dz)));
+    if (cheb >= s0) {
+      const int c[3] = {b[0] + dx, b[1] + dy, b[2] + dz};
+      int w[3];
+      for (int d = 0; d < 3; d++) {
+        sh[d] = floordiv(c[d], G.nb[d]);
+        w[d] = c[d] - sh[d] * G.nb[d];
+      }
+      const int bin = (w[2] * G.nb[1] + w[1]) * G.nb[0] + w[0];
+      lo = G.bin_start[bin];
+      hi = G.bin_start[bin + 1];
+    }
+  }
+  const int cnt = hi - lo;
+  int pre = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, pre, o);
+    if (lane >= o) pre += y;
+  }
+  const int total = __shfl_sync(0xffffffffu, pre, 31);
+  if (at + total > MAXC) return -1;
+  int slot = at + pre - cnt;
+  const int code = pack_shift(sh);
+  for (int k = lo; k < hi; k++) {
+    S.u.c.cj[slot] = G.bin_pts[k];
+    S.u.c.cs[slot] = code;
+    slot++;
+  }
+  __syncwarp();
+  // positions, the candidates spread over the lanes
+  for (int k = at + lane; k < at + total; k += 32) {
+    const int j = S.u.c.cj[k], cs = S.u.c.cs[k];
+    double x[3], d2;
+    image3(G, j, cs, ri, x, d2);
+    const float d2f = (j == i && cs == 0) ? -1.0f : (float)d2;   // -1: the generator itself, skipped
+    S.u.c.cx[k] = make_float4(trunc_f32(x[0]), trunc_f32(x[1]), trunc_f32(x[2]), 0.5f * d2f);
+  }
+  __syncwarp();
+  return at + total;
+}
+
+__global__ void __launch_bounds__(32 * FWARPS, 5) k_cells3_fast(const __grid_constant__ Grid G, HalfList H, int* nhf, double* vol, double* com,
+                                                              const int* binof, int* left, int* nleft, double thr_area) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  Fast3& S = reinterpret_cast<Fast3*>(smem)[w];
+  const double eps = 1e-12 * fmin(G.bs[0], fmin(G.bs[1], G.bs[2]));
+  for (int k = lane; k < 2 * FP; k += 32) (&S.edge[0][0])[k] = 0u;
+  // per launch, in FP32 (scalar FP64 costs a warp as much as a vector's)
+  const float hb[3] = {(float)(0.5 * G.box[0]), (float)(0.5 * G.box[1]), (float)(0.5 * G.box[2])};
+  const float bsf[3] = {(float)G.bs[0], (float)G.bs[1], (float)G.bs[2]};
+  const float R2box = 0.25f * (float)(G.box[0] * G.box[0] + G.box[1] * G.box[1] + G.box[2] * G.box[2]) * (1.0f + 1e-5f);
+  const int smax = max(G.nb[0], max(G.nb[1], G.nb[2])) + 2;
+  for (int i = blockIdx.x * FWARPS + w; i < G.n; i += gridDim.x * FWARPS) {
+    const double ri[3] = {G.pts[(size_t)i * 3], G.pts[(size_t)i * 3 + 1], G.pts[(size_t)i * 3 + 2]};
+    // the initial cell: the box of the periodic domain around the generator
+    if (lane < 6) {
+      const int ax = lane >> 1;
+      const float sg = (lane & 1) ? -1.0f : 1.0f;
+      S.pnf[lane] = make_float4(ax == 0 ? sg : 0.0f, ax == 1 ? sg : 0.0f, ax == 2 ? sg : 0.0f, ax == 0 ? hb[0] : (ax == 1 ? hb[1] : hb[2]));
+      S.pj[lane] = -1;
+      S.ps[lane] = 0;
+    }
+    Verts V;
+    {
+      // corner (sx, sy, sz): planes +-x, +-y, +-z, ordered so det(n_a, n_b, n_c) > 0
+      const int sx = (lane & 1) ? -1 : 1, sy = (lane & 2) ? -1 : 1, sz = (lane & 4) ? -1 : 1;
+      const unsigned a = (sx > 0) ? 0 : 1, b = (sy > 0) ? 2 : 3, c = (sz > 0) ? 4 : 5;
+      const bool pos = sx * sy * sz > 0;
+      V.tri[0] = (pos ? a : b) | (pos ? b : a) << 8 | c << 16;
+      V.tri[1] = 0u;
+      V.x[0] = sx * hb[0];
+      V.y[0] = sy * hb[1];
+      V.z[0] = sz * hb[2];
+      V.r[0] = sqrtf(V.x[0] * V.x[0] + V.y[0] * V.y[0] + V.z[0] * V.z[0]);
+      V.f[0] = 1e-5f;
+      V.x[1] = V.y[1] = V.z[1] = V.r[1] = V.f[1] = 0.0f;
+    }
+    unsigned L[2] = {0xffu, 0u};   // the lanes' live vertices
+    int np = 6;
+    __syncwarp();
+    float R2 = R2box;
+    const int bin = binof[i];
+    const int b[3] = {bin % G.nb[0], bin / G.nb[0] % G.nb[1], bin / G.nb[0] / G.nb[1]};
+    int rc = 1;   // 1: incomplete, 0: done, -1: for k_cells3
+    for (int s = 2; s <= smax && rc == 1; s++) {
+      const int s0 = (s == 2) ? 0 : s;
+      const int side = 2 * s + 1, nq = side * side * side;
+      int nc = 0, q0 = 0;
+      for (;;) {
+        const int at = gather_fast(G, S, lane, i, ri, b, s, s0, q0, min(nq, q0 + 32), nc);
+        if (at >= 0) {
+          nc = at;
+          q0 += 32;
+          if (q0 < nq) continue;
+        } else if (nc == 0) {
+          rc = -1;   // more points in 32 bins than the buffer holds
+          break;
+        }
+        // all gathered, or the buffer full: cut by what it holds
+        if (cut_buffer_fast(G, S, V, L, np, lane, nc, ri, eps, R2) < 0) {
+          rc = -1;
+          break;
+        }
+        __syncwarp();
+        nc = 0;
+        if (q0 >= nq) break;
+      }
+      if (rc < 0) break;
+      // the distance to the boundary of the searched cube, rounded down
+      float bound = 1e30f;
+      for (int d = 0; d < 3; d++) {
+        const float x = (float)ri[d];
+        const float lo = (float)(b[d] - s) * bsf[d], hi = (float)(b[d] + s + 1) * bsf[d];
+        bound = fminf(bound, fminf(x - lo, hi - x) - 1e-6f * (2.0f * hb[d] + (float)s * bsf[d]));
+      }
+      if (bound > 0.0f && bound * bound >= 4.0f * R2) rc = 0;
+    }
+    // a face of the initial box that survived: not closed
+    {
+      bool open = false;
+#pragma unroll
+      for (int e = 0; e < 2; e++)
+        if ((L[e] >> lane) & 1u)
+          open |= (V.tri[e] & 255) < 6 || ((V.tri[e] >> 8) & 255) < 6 || ((V.tri[e] >> 16) & 255) < 6;
+      if (__any_sync(full, open)) rc = -1;
+    }
+    int nf = 0;
+    double sum[4] = {0.0, 0.0, 0.0, 0.0};   // volume, first moment
+    __syncwarp();
+    if (rc == 0) {
+      if (L[1] != 0u && __popc(L[0]) + __popc(L[1]) <= 32) {
+        // all vertices into the first places: one FP64 solve per lane, not two
+        if ((L[1] >> lane) & 1u) S.u.f.tri[__popc(L[1] & ((1u << lane) - 1u))] = V.tri[1];
+        __syncwarp();
+        const int rank = __popc(~L[0] & ((1u << lane) - 1u));
+        const bool take = !((L[0] >> lane) & 1u) && rank < __popc(L[1]);
+        if (take) V.tri[0] = S.u.f.tri[rank];
+        L[0] |= __ballot_sync(full, take);
+        L[1] = 0u;
+        __syncwarp();
+      }
+      // FP64 planes; for each plane and neighbouring plane the vertex with the
+      // two in this order; a vertex of each plane
+      for (int k = lane; k < np; k += 32) {
+        plane3(G, k, S.pj[k], S.ps[k], ri, S.u.f.P[k]);
+        S.u.f.start[k] = 64;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int e = 0; e < 2; e++)
+        if ((L[e] >> lane) & 1u) {
+          const int t = lane + 32 * e;
+          const int pa = V.tri[e] & 255, pb = (V.tri[e] >> 8) & 255, pc = (V.tri[e] >> 16) & 255;
+          S.u.f.tri[t] = V.tri[e];
+          S.u.f.next[pa][pb] = (unsigned char)t;
+          S.u.f.next[pb][pc] = (unsigned char)t;
+          S.u.f.next[pc][pa] = (unsigned char)t;
+          atomicMin(&S.u.f.start[pa], t);
+          atomicMin(&S.u.f.start[pb], t);
+          atomicMin(&S.u.f.start[pc], t);
+          solve3(S.u.f.P[pa], S.u.f.P[pb], S.u.f.P[pc], S.u.f.v[t]);
+        }
+      __syncwarp();
+      // room for the planes that still have a vertex
+      int mf = 0;
+      for (int k0 = 6; k0 < np; k0 += 32)
+        mf += __popc(__ballot_sync(full, k0 + lane < np && S.u.f.start[k0 + lane] < 64));
+      int room = 0;
+      if (lane == 0) room = half_room(H, i, mf);
+      room = __shfl_sync(full, room, 0);
+      // faces: lane per plane, its vertices from one to the next
+      for (int k0 = 6; k0 < np; k0 += 32) {
+        const int k = k0 + lane;
+        double area = 0.0, fc[3] = {0.0, 0.0, 0.0};
+        bool keep = false;
+        const int t0 = k < np ? S.u.f.start[k] : 64;
+        if (t0 < 64) {
+          const double* pk = S.u.f.P[k];
+          const double n0 = fabs(pk[0]), n1 = fabs(pk[1]), n2 = fabs(pk[2]);
+          const int ax = n0 >= n1 ? (n0 >= n2 ? 0 : 2) : (n1 >= n2 ? 1 : 2);
+          const int cu = ax == 2 ? 0 : ax + 1, cv = ax == 0 ? 2 : ax - 1;
+          const double ou = S.u.f.v[t0][cu], ov = S.u.f.v[t0][cv];
+          double e1u = 0.0, e1v = 0.0, A = 0.0, Cu = 0.0, Cv = 0.0;
+          int t = t0, m = 0;
+          bool ok = true;
+          for (;;) {
+            // the vertex (k, x, y): its successor on the face is (k, y, .)
+            const unsigned tr = S.u.f.tri[t];
+            const int p0 = tr & 255, p1 = (tr >> 8) & 255, p2 = (tr >> 16) & 255;
+            const int y = p0 == k ? p2 : (p1 == k ? p0 : p1);
+            m++;
+            const int tn = S.u.f.next[k][y];
+            if (tn == t0) break;
+            // the table is not cleared: check that this entry is of this cell
+            bool good = m < MAXFV && tn < 64 && (((tn < 32 ? L[0] : L[1]) >> (tn & 31)) & 1u);
+            if (good) {
+              const unsigned tq = S.u.f.tri[tn];
+              const int g0 = tq & 255, g1 = (tq >> 8) & 255, g2 = (tq >> 16) & 255;
+              good = (g0 == k && g1 == y) || (g1 == k && g2 == y) || (g2 == k && g0 == y);
+            }
+            if (!good) {
+              ok = false;
+              break;
+            }
+            const double e2u = S.u.f.v[tn][cu] - ou, e2v = S.u.f.v[tn][cv] - ov;
+            const double at = e1u * e2v - e1v * e2u;
+            A += at;
+            Cu += at * (e1u + e2u);
+            Cv += at * (e1v + e2v);
+            e1u = e2u;
+            e1v = e2v;
+            t = tn;
+          }
+          if (!ok) rc = -1;
+          if (ok && m >= 3) {
+            // one division for both 1 / n_ax and 1 / (3 A)
+            const double nax = pk[ax];
+            const double A3 = A != 0.0 ? 3.0 * A : 1.0;
+            const double inv = 1.0 / (nax * A3);
+            const double in = inv * A3, third = inv * nax, ia = fabs(in);
+            const double a2 = 0.5 * fabs(A);             // area in the projection
+            area = a2 * ia * sqrt(2.0 * pk[3]);          // |n|^2 = 2 h
+            const double u = ou + Cu * third, v = ov + Cv * third;
+            const double z = (pk[3] - pk[cu] * u - pk[cv] * v) * in;
+            fc[0] = ax == 0 ? z : (cu == 0 ? u : v);
+            fc[1] = ax == 1 ? z : (cu == 1 ? u : v);
+            fc[2] = ax == 2 ? z : (cu == 2 ? u : v);
+            // pyramid with apex at the generator: height times area / 3 (the
+            // height is h / |n|), centroid 3/4 of the way to the face
+            const double vp = pk[3] * a2 * ia * (1.0 / 3.0);
+            sum[0] += vp;
+            for (int d = 0; d < 3; d++) sum[1 + d] += vp * 0.75 * fc[d];
+            keep = area > thr_area;
+          }
+        }
+        const unsigned km = __ballot_sync(full, keep);
+        if (keep) {
+          const int f = nf + __popc(km & ((1u << lane) - 1u));
+          if (room >= 0) {
+            HalfFace& o = H.f[room + f];
+            const int sh = S.ps[k];
+            o.j = S.pj[k];
+            for (int d = 0; d < 3; d++) o.s[d] = (signed char)shift_of(sh, d);
+            o.s[3] = 0;
+            o.area = area;
+            for (int d = 0; d < 3; d++) o.cen[d] = fc[d];
+          }
+        }
+        nf += __popc(km);
+      }
+      if (__any_sync(full, rc != 0)) rc = -1;
+      if (nf > MAXHF) rc = -1;
+    }
+    // the four sums over the lanes: two levels that halve the components a
+    // lane carries, then three; lanes 8 q.. hold component q
+    {
+      const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0;
+      const double s0 = (b4 ? sum[2] : sum[0]) + __shfl_xor_sync(full, b4 ? sum[0] : sum[2], 16);
+      const double s1 = (b4 ? sum[3] : sum[1]) + __shfl_xor_sync(full, b4 ? sum[1] : sum[3], 16);
+      double t = (b3 ? s1 : s0) + __shfl_xor_sync(full, b3 ? s0 : s1, 8);
+      t += __shfl_xor_sync(full, t, 4);
+      t += __shfl_xor_sync(full, t, 2);
+      t += __shfl_xor_sync(full, t, 1);
+      const double Vt = __shfl_sync(full, t, 0);
+      const int comp = lane >> 3;
+      if (rc == 0) {
+        if (lane == 0) {
+          nhf[i] = nf;
+          vol[i] = t;
+        } else if ((lane & 7) == 0) {
+          const double r = comp == 1 ? ri[0] : (comp == 2 ? ri[1] : ri[2]);
+          com[(size_t)i * 3 + comp - 1] = r + (Vt > 0.0 ? t / Vt : 0.0);
+        }
+      } else if (lane == 0) {
+        left[atomicAdd(nleft, 1)] = i;
+      }
+    }
+    __syncwarp();
+  }
+}
+
+__global__ void __launch_bounds__(32 * WARPS) k_cells3(Grid G, HalfList H, int* nhf, double* vol, double* com,
+                                                      int* err, const int* list, const int* nlist,
+                                                      double thr_area) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   Cell3& C = reinterpret_cast<Cell3*>(smem)[w];
   const double hcell = fmin(G.bs[0], fmin(G.bs[1], G.bs[2]));
   const double eps = 1e-12 * hcell;
-  for (int i = blockIdx.x * WARPS + w; i < G.n; i += gridDim.x * WARPS) {
+  // the cells that k_cells3_fast left
+  const int count = *nlist;
+  for (int idx = blockIdx.x * WARPS + w; idx < count; idx += gridDim.x * WARPS) {
+    const int i = list[idx];
     const double ri[3] = {G.pts[(size_t)i * 3], G.pts[(size_t)i * 3 + 1], G.pts[(size_t)i * 3 + 2]};
     // the initial cell: the box of the periodic domain around the generator
     if (lane < 6) {
@@ -521,6 +1115,9 @@ __global__ void __launch_bounds__(32 * WARPS) k_cells3(Grid G, HalfFace* hf, int
     int nf = 0;
     double V = 0.0, M[3] = {0.0, 0.0, 0.0};
     if (rc == 0) {
+      int room = 0;
+      if (lane == 0) room = half_room(H, i, MAXHF);
+      room = __shfl_sync(0xffffffffu, room, 0);
       for (int k0 = 6; k0 < C.np; k0 += 32) {
         const int k = k0 + lane;
         double area = 0.0, fc[3] = {0.0, 0.0, 0.0};
@@ -589,8 +1186,8 @@ __global__ void __launch_bounds__(32 * WARPS) k_cells3(Grid G, HalfFace* hf, int
         const unsigned km = __ballot_sync(0xffffffffu, keep);
         if (keep) {
           const int f = nf + __popc(km & ((1u << lane) - 1u));
-          if (f < MAXHF) {
-            HalfFace& o = hf[(size_t)i * MAXHF + f];
+          if (f < MAXHF && room >= 0) {
+            HalfFace& o = H.f[room + f];
             o.j = C.pj[k];
             for (int d = 0; d < 4; d++) o.s[d] = C.ps[k][d];
             o.area = area;
@@ -675,7 +1272,7 @@ __device__ int cut2(Line2* L, int& nl, const Line2& c, double eps, double& R2) {
   return 1;
 }
 
-__global__ void k_cells2(Grid G, HalfFace* hf, int* nhf, double* vol, double* com, int* err, double thr_len) {
+__global__ void k_cells2(Grid G, HalfList H, int* nhf, double* vol, double* com, int* err, double thr_len) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= G.n) return;
   const double ri[2] = {G.pts[(size_t)i * 2], G.pts[(size_t)i * 2 + 1]};
@@ -759,7 +1356,7 @@ __global__ void k_cells2(Grid G, HalfFace* hf, int* nhf, double* vol, double* co
         rc = E_CAPACITY;
         break;
       }
-      HalfFace& o = hf[(size_t)i * 32 + nf];
+      HalfFace& o = H.f[(size_t)i * 32 + nf];
       o.j = L[k].j;
       o.s[0] = L[k].s[0];
       o.s[1] = L[k].s[1];
@@ -772,6 +1369,7 @@ __global__ void k_cells2(Grid G, HalfFace* hf, int* nhf, double* vol, double* co
       nf++;
     }
   }
+  H.first[i] = i * 32;
   nhf[i] = rc == 0 ? nf : 0;
   vol[i] = V;
   com[(size_t)i * 2] = ri[0] + (V > 0.0 ? M[0] / V : 0.0);
@@ -789,55 +1387,82 @@ __device__ __forceinline__ bool keep_face(int i, const HalfFace& f, int dim) {
   return false;
 }
 
-__global__ void k_keep_count(int n, int dim, int slots, const HalfFace* hf, const int* nhf, int* keep) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// Sixteen lanes share a cell in the face-list kernels (a 3D cell has about 15
+// half-faces of 40 bytes, so a thread per cell reads them one behind the
+// other, each from its own sector).
+constexpr int FLANES = 16;
+
+__global__ void k_keep_count(int n, int dim, const HalfFace* hf, const int* first, const int* nhf, int* keep) {
+  const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / FLANES), l = threadIdx.x % FLANES;
   int c = 0;
-  for (int f = 0; f < nhf[i]; f++) c += keep_face(i, hf[(size_t)i * slots + f], dim) ? 1 : 0;
-  keep[i] = c;
+  if (i < n)
+    for (int f = l; f < nhf[i]; f += FLANES) c += keep_face(i, hf[(size_t)first[i] + f], dim) ? 1 : 0;
+#pragma unroll
+  for (int o = FLANES / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  if (i < n && l == 0) keep[i] = c;
 }
 
-__global__ void k_emit(int n, int dim, int slots, const double* pts, const HalfFace* hf, const int* nhf,
+__global__ void k_emit(int n, int dim, const double* pts, const HalfFace* hf, const int* first, const int* nhf,
                        const int* off, int32_t* cells, int8_t* shift, double* area, double* cen) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int o = off[i];
-  for (int f = 0; f < nhf[i]; f++) {
-    const HalfFace& h = hf[(size_t)i * slots + f];
-    if (!keep_face(i, h, dim)) continue;
-    cells[2 * (size_t)o] = i;
-    cells[2 * (size_t)o + 1] = h.j;
-    for (int d = 0; d < dim; d++) {
-      shift[(size_t)o * dim + d] = h.s[d];
-      cen[(size_t)o * dim + d] = pts[(size_t)i * dim + d] + h.cen[d];
+  const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / FLANES), l = threadIdx.x % FLANES;
+  const int base = (threadIdx.x & 31) / FLANES * FLANES;   // the group's first lane
+  const int m = i < n ? nhf[i] : 0;
+  int o = i < n ? off[i] : 0;
+  // (the groups of a warp run as many rounds as the longest list)
+  for (int f0 = 0; __any_sync(0xffffffffu, f0 < m); f0 += FLANES) {
+    const int f = f0 + l;
+    const HalfFace* h = hf + (i < n ? first[i] : 0) + f;
+    const bool keep = f < m && keep_face(i, *h, dim);
+    const unsigned k = (__ballot_sync(0xffffffffu, keep) >> base) & ((1u << FLANES) - 1u);
+    if (keep) {
+      const size_t at = (size_t)(o + __popc(k & ((1u << l) - 1u)));
+      cells[2 * at] = i;
+      cells[2 * at + 1] = h->j;
+      for (int d = 0; d < dim; d++) {
+        shift[at * dim + d] = h->s[d];
+        cen[at * dim + d] = pts[(size_t)i * dim + d] + h->cen[d];
+      }
+      area[at] = h->area;
     }
-    area[o] = h.area;
-    o++;
+    o += __popc(k);
   }
 }
 
 // every listed face against its mirror in the neighbour's list: count the
 // missing ones, the largest relative area mismatch (positive doubles order
-// like their bit patterns)
-__global__ void k_mirror(int n, int dim, int slots, const HalfFace* hf, const int* nhf,
+// like their bit patterns; one atomic per warp, and only where it would
+// change the maximum)
+__global__ void k_mirror(int n, int dim, const HalfFace* hf, const int* first, const int* nhf,
                          unsigned long long* missing, unsigned long long* maxrel_bits) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  for (int f = 0; f < nhf[i]; f++) {
-    const HalfFace& h = hf[(size_t)i * slots + f];
-    if (!keep_face(i, h, dim)) continue;
-    bool found = false;
-    for (int g = 0; g < nhf[h.j] && !found; g++) {
-      const HalfFace& m = hf[(size_t)h.j * slots + g];
-      bool same = m.j == i;
-      for (int d = 0; d < dim; d++) same = same && m.s[d] == -h.s[d];
-      if (same) {
-        found = true;
-        const double rel = fabs(m.area - h.area) / h.area;
-        atomicMax(maxrel_bits, (unsigned long long)__double_as_longlong(rel));
+  const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / FLANES), l = threadIdx.x % FLANES;
+  double rel = 0.0;
+  int miss = 0;
+  if (i < n)
+    for (int f = l; f < nhf[i]; f += FLANES) {
+      const HalfFace& h = hf[(size_t)first[i] + f];
+      if (!keep_face(i, h, dim)) continue;
+      const HalfFace* other = hf + first[h.j];
+      const int mo = nhf[h.j];
+      int g = 0;
+      for (; g < mo; g++) {
+        const HalfFace& m = other[g];
+        bool same = m.j == i;
+        for (int d = 0; d < dim; d++) same = same && m.s[d] == -h.s[d];
+        if (same) break;
       }
+      // (the FP64 division once, not at each lane's own round of the search)
+      if (g < mo)
+        rel = fmax(rel, fabs(other[g].area - h.area) / h.area);
+      else
+        miss++;
     }
-    if (!found) atomicAdd(missing, 1ull);
+  miss = __reduce_add_sync(0xffffffffu, miss);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) rel = fmax(rel, __shfl_xor_sync(0xffffffffu, rel, o));
+  if ((threadIdx.x & 31) == 0) {
+    if (miss) atomicAdd(missing, (unsigned long long)miss);
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(rel);
+    if (bits > *(volatile unsigned long long*)maxrel_bits) atomicMax(maxrel_bits, bits);
   }
 }
 
@@ -858,17 +1483,34 @@ namespace amm {
 namespace vor {
 
 // Device scratch and outputs of a build, grown on demand and kept between
-// builds by a caller that tessellates repeatedly (amm_retessellate).
+// builds by a caller that tessellates repeatedly (amm_retessellate).  Three
+// allocations: everything sized by the cells and bins, the half-face list, the
+// faces.
 struct TessWork {
   int64_t cap_n = 0, cap_bins = 0, cap_hf = 0, cap_f = 0;
+  int cap_dim = 0;
+  char *cell_ws = nullptr, *face_ws = nullptr;
   int *binof = nullptr, *count = nullptr, *start = nullptr, *cursor = nullptr, *bin_pts = nullptr;
-  int *err = nullptr, *nhf = nullptr, *keep = nullptr, *off = nullptr;
+  int *nhf = nullptr, *keep = nullptr, *off = nullptr, *left = nullptr, *part = nullptr, *first = nullptr;
+  int* err = nullptr;                  // error, cells left to k_cells3, half-faces taken
+  unsigned long long* chk = nullptr;   // missing mirrors, largest area mismatch
   HalfFace* hf = nullptr;
-  unsigned long long* chk = nullptr;
   double *vol = nullptr, *com = nullptr;
   int32_t* cells = nullptr;
   int8_t* shift = nullptr;
   double *area = nullptr, *cen = nullptr;
+};
+
+// lays arrays out one behind the other, 256 bytes aligned; with a null base
+// only the size is counted
+struct Layout {
+  char* base;
+  size_t bytes = 0;
+  template <typename T>
+  void operator()(T*& p, int64_t count) {
+    p = base ? reinterpret_cast<T*>(base + bytes) : nullptr;
+    bytes += (sizeof(T) * (size_t)std::max<int64_t>(count, 1) + 255) / 256 * 256;
+  }
 };
 
 TessWork* work_new() { return new TessWork(); }
@@ -883,8 +1525,7 @@ void work_faces(const TessWork* w, const int32_t** cells, const int8_t** shift, 
 
 void work_free(TessWork* w) {
   if (!w) return;
-  void* p[] = {w->binof, w->count, w->start, w->cursor, w->bin_pts, w->err, w->nhf, w->keep, w->off, w->hf,
-               w->chk,   w->vol,   w->com,   w->cells,  w->shift,   w->area, w->cen};
+  void* p[] = {w->cell_ws, w->hf, w->face_ws};
   for (void* q : p)
     if (q) cudaFree(q);
   delete w;
@@ -905,17 +1546,6 @@ const char* tess_msg(int rc) {
     case -7: return "too many generators in 32 bins of the search grid";
     default: return "tessellation failed";
   }
-}
-
-template <typename T>
-cudaError_t grow(T** p, int64_t& cap, int64_t need, int64_t alloc) {
-  if (need <= cap && *p) return cudaSuccess;
-  if (*p) cudaFree(*p);
-  *p = nullptr;
-  cap = 0;
-  cudaError_t e = cudaMalloc((void**)p, sizeof(T) * (size_t)std::max<int64_t>(alloc, 1));
-  if (e == cudaSuccess) cap = alloc;
-  return e;
 }
 
 }  // namespace
@@ -944,7 +1574,6 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
     }
   }
   const int nbins = G.nb[0] * G.nb[1] * G.nb[2];
-  const int slots = dim == 3 ? MAXHF : 32;
   int rc = AMM_OK;
   auto cu = [&](cudaError_t e, const char* where) {
     if (e != cudaSuccess && rc == AMM_OK) {
@@ -953,73 +1582,100 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
     }
     return rc == AMM_OK;
   };
-  // per-cell and per-bin scratch (sizes fixed by n, grown only)
-  if (n > w->cap_n || !w->binof) {
-    const int64_t m = n;
-    void* p[] = {w->binof, w->bin_pts, w->nhf, w->keep, w->off, w->vol, w->com};
-    for (void* q : p)
-      if (q) cudaFree(q);
-    w->binof = w->bin_pts = w->nhf = w->keep = w->off = nullptr;
-    w->vol = w->com = nullptr;
-    w->cap_n = 0;
-    cu(cudaMalloc(&w->binof, sizeof(int) * m), "alloc");
-    cu(cudaMalloc(&w->bin_pts, sizeof(int) * m), "alloc");
-    cu(cudaMalloc(&w->nhf, sizeof(int) * m), "alloc");
-    cu(cudaMalloc(&w->keep, sizeof(int) * m), "alloc");
-    cu(cudaMalloc(&w->off, sizeof(int) * (m + 1)), "alloc");
-    cu(cudaMalloc(&w->vol, sizeof(double) * m), "alloc");
-    cu(cudaMalloc(&w->com, sizeof(double) * m * 3), "alloc");
-    if (rc == AMM_OK) w->cap_n = m;
+  // per-cell and per-bin arrays (sizes fixed by n, grown only)
+  if (n > w->cap_n || nbins > w->cap_bins || dim != w->cap_dim || !w->cell_ws) {
+    if (w->cell_ws) cudaFree(w->cell_ws);
+    w->cell_ws = nullptr;
+    w->cap_n = w->cap_bins = 0;
+    for (int pass = 0; pass < 2; pass++) {   // count, then place
+      Layout at{w->cell_ws};
+      at(w->binof, n);
+      at(w->bin_pts, n);
+      at(w->nhf, n);
+      at(w->keep, n);
+      at(w->off, n + 1);
+      at(w->left, n);
+      at(w->first, n);
+      at(w->vol, n);
+      at(w->com, 3 * n);
+      at(w->count, nbins);
+      at(w->start, nbins + 1);
+      at(w->cursor, nbins);
+      at(w->part, std::max(scan_scratch(n), scan_scratch(nbins)));
+      at(w->err, 4);
+      at(w->chk, 2);
+      if (pass == 0 && !cu(cudaMalloc(&w->cell_ws, at.bytes), "alloc")) return rc;
+    }
+    w->cap_n = n;
+    w->cap_bins = nbins;
+    w->cap_dim = dim;
   }
-  if (nbins > w->cap_bins || !w->count) {
-    void* p[] = {w->count, w->start, w->cursor};
-    for (void* q : p)
-      if (q) cudaFree(q);
-    w->count = w->start = w->cursor = nullptr;
-    w->cap_bins = 0;
-    cu(cudaMalloc(&w->count, sizeof(int) * nbins), "alloc");
-    cu(cudaMalloc(&w->start, sizeof(int) * (nbins + 1)), "alloc");
-    cu(cudaMalloc(&w->cursor, sizeof(int) * nbins), "alloc");
-    if (rc == AMM_OK) w->cap_bins = nbins;
-  }
-  if (!w->err) cu(cudaMalloc(&w->err, sizeof(int)), "alloc");
-  if (!w->chk) cu(cudaMalloc(&w->chk, sizeof(unsigned long long) * 2), "alloc");
-  cu(grow(&w->hf, w->cap_hf, n * slots, n * slots), "alloc");
-  if (rc != AMM_OK) return rc;
+  // 3D: room for 18 half-faces per cell (15.5 on average among random
+  // generators); a build that needs more is repeated with that
+  const auto hf_room = [&](int64_t want) {
+    if (want <= w->cap_hf && w->hf) return true;
+    if (want > 0x7fffffffll - 64) {
+      g_tess_err = "more half-faces than the builder can index";
+      rc = AMM_ERR_NUMERIC;
+      return false;
+    }
+    if (w->hf) cudaFree(w->hf);
+    w->hf = nullptr;
+    w->cap_hf = 0;
+    if (cu(cudaMalloc((void**)&w->hf, sizeof(HalfFace) * (size_t)want), "alloc")) w->cap_hf = want;
+    return rc == AMM_OK;
+  };
+  if (!hf_room(dim == 3 ? std::min<int64_t>(18 * n + 1024, 0x7fffffffll - 64) : 32 * n)) return rc;
   const int nb256 = (int)((n + 255) / 256);
   G.pts = gen_d;
   cu(cudaMemsetAsync(w->count, 0, sizeof(int) * nbins, st), "memset");
-  cu(cudaMemsetAsync(w->err, 0, sizeof(int), st), "memset");
+  cu(cudaMemsetAsync(w->err, 0, 4 * sizeof(int), st), "memset");
   cu(cudaMemsetAsync(w->chk, 0, sizeof(unsigned long long) * 2, st), "memset");
   k_check_range<<<nb256, 256, 0, st>>>(G, w->err);
   k_bin_count<<<nb256, 256, 0, st>>>(G, w->binof, w->count);
-  k_scan<<<1, 1024, 0, st>>>(w->count, w->start, nbins);
+  cu(exclusive_scan(w->count, w->start, nbins, w->part, st), "scan");
   cu(cudaMemcpyAsync(w->cursor, w->start, sizeof(int) * nbins, cudaMemcpyDeviceToDevice, st), "copy");
   k_bin_fill<<<nb256, 256, 0, st>>>(G, w->binof, w->cursor, w->bin_pts);
   k_bin_sort<<<(nbins + 255) / 256, 256, 0, st>>>(w->start, w->bin_pts, nbins);
   G.bin_start = w->start;
   G.bin_pts = w->bin_pts;
   const double thr = 1e-12 * std::pow(hcell, dim - 1);
-  if (dim == 3) {
-    const size_t smem = sizeof(Cell3) * WARPS;
-    cu(cudaFuncSetAttribute(k_cells3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "attribute");
-    const int64_t blocks = std::min<int64_t>((n + WARPS - 1) / WARPS, 152 * 16);
-    k_cells3<<<(int)blocks, 32 * WARPS, smem, st>>>(G, w->hf, w->nhf, w->vol, w->com, w->err, thr);
-  } else {
-    k_cells2<<<nb256, 256, 0, st>>>(G, w->hf, w->nhf, w->vol, w->com, w->err, thr);
+  const int nbf = (int)((n * FLANES + 255) / 256);
+  int herr[4] = {0, 0, 0, 0};
+  for (;;) {
+    const HalfList H{w->hf, w->first, w->err + 2, (int)w->cap_hf};
+    if (dim == 3) {
+      const size_t smem = sizeof(Cell3) * WARPS, fsmem = sizeof(Fast3) * FWARPS;
+      cu(cudaFuncSetAttribute(k_cells3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "attribute");
+      cu(cudaFuncSetAttribute(k_cells3_fast, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem), "attribute");
+      // the ordinary cells, then whatever they left (often nothing)
+      const int64_t fblocks = std::min<int64_t>((n + FWARPS - 1) / FWARPS, 152 * 5);
+      const int64_t blocks = std::min<int64_t>((n + WARPS - 1) / WARPS, 152 * 4);
+      k_cells3_fast<<<(int)fblocks, 32 * FWARPS, fsmem, st>>>(G, H, w->nhf, w->vol, w->com, w->binof, w->left, w->err + 1,
+                                                            thr);
+      k_cells3<<<(int)blocks, 32 * WARPS, smem, st>>>(G, H, w->nhf, w->vol, w->com, w->err, w->left, w->err + 1, thr);
+    } else {
+      k_cells2<<<nb256, 256, 0, st>>>(G, H, w->nhf, w->vol, w->com, w->err, thr);
+    }
+    cu(cudaGetLastError(), "cells");
+    cu(cudaMemcpyAsync(herr, w->err, 3 * sizeof(int), cudaMemcpyDeviceToHost, st), "read");
+    // (the pass below reads the list: only where it holds every face)
+    cu(cudaStreamSynchronize(st), "sync");
+    if (rc != AMM_OK) return rc;
+    if (herr[0] != 0) {
+      g_tess_err = tess_msg(herr[0]);
+      return herr[0] == -5 ? AMM_ERR_INVALID_ARG : AMM_ERR_NUMERIC;
+    }
+    if (dim == 2 || (herr[2] >= 0 && herr[2] <= w->cap_hf)) break;
+    // (each warp's count is added whether or not it fits, so this is enough)
+    if (!hf_room(herr[2] < 0 ? 0x7fffffffll : (int64_t)herr[2] + 1024)) return rc;
+    cu(cudaMemsetAsync(w->err, 0, 4 * sizeof(int), st), "memset");
   }
-  k_keep_count<<<nb256, 256, 0, st>>>((int)n, dim, slots, w->hf, w->nhf, w->keep);
-  k_scan<<<1, 1024, 0, st>>>(w->keep, w->off, (int)n);
-  cu(cudaGetLastError(), "cells");
-  int herr[2] = {0, 0};
-  cu(cudaMemcpyAsync(&herr[0], w->err, sizeof(int), cudaMemcpyDeviceToHost, st), "read");
+  k_keep_count<<<nbf, 256, 0, st>>>((int)n, dim, w->hf, w->first, w->nhf, w->keep);
+  cu(exclusive_scan(w->keep, w->off, n, w->part, st), "scan");
   cu(cudaMemcpyAsync(&herr[1], w->off + n, sizeof(int), cudaMemcpyDeviceToHost, st), "read");
   cu(cudaStreamSynchronize(st), "sync");
   if (rc != AMM_OK) return rc;
-  if (herr[0] != 0) {
-    g_tess_err = tess_msg(herr[0]);
-    return herr[0] == -5 ? AMM_ERR_INVALID_ARG : AMM_ERR_NUMERIC;
-  }
   const int64_t nf = herr[1];
   if (nf < 1) {
     g_tess_err = "no faces";
@@ -1027,23 +1683,22 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
   }
   if (nf > w->cap_f || !w->cells) {
     const int64_t cap = nf + nf / 8;   // room for the next meshes of a moving run
-    void* p[] = {w->cells, w->shift, w->area, w->cen};
-    for (void* q : p)
-      if (q) cudaFree(q);
-    w->cells = nullptr;
-    w->shift = nullptr;
-    w->area = w->cen = nullptr;
+    if (w->face_ws) cudaFree(w->face_ws);
+    w->face_ws = nullptr;
     w->cap_f = 0;
-    cu(cudaMalloc(&w->cells, sizeof(int32_t) * 2 * cap), "alloc");
-    cu(cudaMalloc(&w->shift, (size_t)cap * 3), "alloc");
-    cu(cudaMalloc(&w->area, sizeof(double) * cap), "alloc");
-    cu(cudaMalloc(&w->cen, sizeof(double) * cap * 3), "alloc");
-    if (rc != AMM_OK) return rc;
+    for (int pass = 0; pass < 2; pass++) {
+      Layout at{w->face_ws};
+      at(w->cells, 2 * cap);
+      at(w->shift, 3 * cap);
+      at(w->area, cap);
+      at(w->cen, 3 * cap);
+      if (pass == 0 && !cu(cudaMalloc(&w->face_ws, at.bytes), "alloc")) return rc;
+    }
     w->cap_f = cap;
   }
-  k_emit<<<nb256, 256, 0, st>>>((int)n, dim, slots, gen_d, w->hf, w->nhf, w->off, w->cells, w->shift, w->area,
+  k_emit<<<nbf, 256, 0, st>>>((int)n, dim, gen_d, w->hf, w->first, w->nhf, w->off, w->cells, w->shift, w->area,
                                 w->cen);
-  if (check) k_mirror<<<nb256, 256, 0, st>>>((int)n, dim, slots, w->hf, w->nhf, w->chk, w->chk + 1);
+  if (check) k_mirror<<<nbf, 256, 0, st>>>((int)n, dim, w->hf, w->first, w->nhf, w->chk, w->chk + 1);
   cu(cudaGetLastError(), "faces");
   unsigned long long h[2] = {0, 0};
   if (check) cu(cudaMemcpyAsync(h, w->chk, sizeof h, cudaMemcpyDeviceToHost, st), "read");
