@@ -55,7 +55,7 @@ void free_ctx(amm_ctx* c) {
                   c->totals, c->stats,  c->closure, c->mlp,      c->defer_list, c->defer_count, c->scratch, c->counter,
                   c->ind_bin, c->ind_act, c->ind_list, c->ind_flist, c->ind_count, c->ind_fstamp, c->ind_cstamp,
                   c->ind_fdt, c->ind_hist, c->ind_slot_cell, c->ind_cell_slot, c->ind_leaf_off, c->ind_level_off,
-                  c->ind_rec, c->ind_rec32, c->ind_node, c->ind_loop, c->geo_ws, c->retess_ws};
+                  c->ind_rec, c->ind_rec32, c->ind_node, c->ind_loop, c->geo_ws, c->retess_ws, c->guard_mask};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 
@@ -430,6 +430,8 @@ int amm_create(amm_ctx** out, int dim, int64_t n, const double* gen, int64_t nf,
   CUB(dalloc(&c->csr, (size_t)2 * nf));
   CUB(dalloc(&c->ctiles, ct.size()));
   CUB(dalloc(&c->ftiles, ft.size()));
+  CUB(dalloc(&c->guard_mask, ft.size() * (amm::FACE_TILE / 32)));
+  CUB(cudaMemsetAsync(c->guard_mask, 0, sizeof(unsigned) * ft.size() * (amm::FACE_TILE / 32), c->stream));
   CUB(dalloc(&c->box_first_ctile, (size_t)nb + 1));
   CUB(cudaMalloc(&c->fgeo, rs * 4 * 2 * (size_t)nf));
   CUB(cudaMalloc(&c->igAB, rs * 4 * 4 * (size_t)nf));

@@ -86,6 +86,7 @@ struct GasC {
   real fan_rho;      // 2/(g-1)
   real fan_p;        // 2g/(g-1)
   real inv_gm1;      // 1/(g-1)
+  real sqrt_two_gp1, isqrt_two_gp1;   // (2/(g+1))^(+-1/2)
   GasC() = default;
   __host__ __device__ explicit GasC(double gamma) {
     g = (real)gamma;
@@ -102,6 +103,8 @@ struct GasC {
     fan_rho = (real)(2.0 / (gamma - 1.0));
     fan_p = (real)(2.0 * gamma / (gamma - 1.0));
     inv_gm1 = (real)(1.0 / (gamma - 1.0));
+    sqrt_two_gp1 = (real)sqrt(2.0 / (gamma + 1.0));
+    isqrt_two_gp1 = (real)sqrt(0.5 * (gamma + 1.0));
   }
 };
 
@@ -168,6 +171,8 @@ struct HydroView {
   unsigned char* kept;         // [n] 1 where the last update kept the advected entropy
   // learned proposal (FP32 learned form only)
   const void* mlp;
+  unsigned* guard_mask;        // FP32 forms: faces left to the flux kernel's FP64 pass, a bit each, by chunk and
+                               // warp (all zero between launches) [n_ftiles * FACE_TILE / 32]
   float* harvest;              // if set, the flux kernel records each face's Riemann inputs [nf][6]
 };
 
@@ -283,6 +288,7 @@ struct amm_ctx {
   void* mlp = nullptr;             // device copy of the proposal weights (MlpDevice)
   int2* defer_list = nullptr;      // learned form: faces past the proposal's gate [nf_cap] {face, box}
   unsigned* defer_count = nullptr; // and their number
+  unsigned* guard_mask = nullptr;  // [face tiles][FACE_TILE / 32]
   float* harvest = nullptr;        // set only during amm_harvest
   bool mlp_loaded = false;
   double* scratch = nullptr;       // layout conversions for getters/setters

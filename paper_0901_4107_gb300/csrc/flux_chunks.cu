@@ -28,6 +28,12 @@
 // extrapolates the two predicted records to its centroid, instead of
 // repeating the prediction on each of a cell's ~15 faces.
 //
+// The FP64 guard: a face whose FP32 Newton iteration falls towards vacuum or does
+// not converge is marked (a bit per face) and computed again, whole, by its
+// CTA after the loop.  Such faces are rare, and the FP64 solve's registers, spills
+// and code in the loop cost every face (11 M faces on a static mesh: 286 us
+// with the solve in the loop, 246 now; 2.05 M on a moving one: 81 us, 63).
+//
 // Learned form (LEARN): a face whose Riemann problem would take the proposal
 // (the linearised star pressure above PROPOSAL_GATE times the larger side
 // pressure) is not solved here; it is appended, warp by warp, to a list that
@@ -41,10 +47,13 @@
 
 namespace amm {
 
-// CTAs per SM each shape is compiled for (launch bounds, and so registers)
-template <int B>
+// CTAs per SM each shape is compiled for (launch bounds, and so registers).
+// The static mesh's kernel holds fewer values: 32 warps per SM (64 registers) run
+// it in 246 us for 11 M faces, 24 in 264; the moving mesh's spills there (2.05 M
+// faces: 73 us, 63 with 24 warps of 80 registers).
+template <int B, bool STATIC>
 constexpr int chunk_ctas_per_sm() {
-  return B == 256 ? 3 : 7;
+  return B == 256 ? (STATIC ? 4 : 3) : (STATIC ? 8 : 7);
 }
 
 // per warp: iteration histogram, statistics sums
@@ -70,6 +79,72 @@ __device__ __forceinline__ CellRec<float> load_rec256(const HydroView<float>& v,
   return r;
 }
 
+// the face k prepared from its records: the cells' half-step predicted records
+// on a static mesh (gradient kernel), else the face-frame prediction
+template <bool ENT, bool STATIC>
+__device__ __forceinline__ void chunk_prepare(const HydroView<float>& v, int k, bool valid, const int2& lr, float hdt,
+                                              FaceWork<float>& f) {
+  R4<float> G0, G1;
+  ldg256(v.fgeo + 2 * (size_t)k, G0, G1);
+  if constexpr (STATIC) {
+    const CellRec<float> pL = load_rec256<ENT>(v, v.cwp, v.Apw, lr.x);
+    const CellRec<float> pR = load_rec256<ENT>(v, v.cwp, v.Apw, lr.y);
+    float AL = 0.0f, AR = 0.0f;
+    if constexpr (ENT) {
+      AL = v.Aw[lr.x];
+      AR = v.Aw[lr.y];
+    }
+    face_prepare_pred<float, ENT>(v, k, valid, lr, G0, G1, pL, pR, AL, AR, f);
+  } else {
+    const CellRec<float> recL = load_rec256<ENT>(v, v.cw, v.Aw, lr.x);
+    const CellRec<float> recR = load_rec256<ENT>(v, v.cw, v.Aw, lr.y);
+    face_prepare_rec<float, ENT>(v, k, valid, hdt, hdt, lr, G0, G1, recL, recR, f);
+  }
+}
+
+// The chunk's faces that need the FP64 guard, by their warp: the whole face
+// again, with the solve in FP64, and its contributions (out of line: nothing
+// of it in the loop's registers).
+template <int B, bool ENT, bool STATIC>
+__device__ __forceinline__ void chunk_guard(const HydroView<float>& v, int c, unsigned todo, unsigned* hist, unsigned* red) {
+  constexpr int CPT = FACE_TILE / B, NM = ENT ? 6 : 5;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const Tile T = v.ftiles[c / CPT];
+  const int k = T.begin + (c % CPT) * B + (int)threadIdx.x;
+  const bool mine = (todo >> lane) & 1u;
+  FaceOut o;
+#pragma unroll
+  for (int a = 0; a < 6; a++) o.m[a] = 0u;
+  o.iters = 0u;
+  o.guard = o.vacuum = o.fail = o.fallback = false;
+  if (mine) {
+    FaceWork<float> f;
+    chunk_prepare<ENT, STATIC>(v, k, true, v.lr[k], (float)(0.5 * box_dt(v, T.box)), f);
+    face_finish_core<float, ENT, GUARD_INLINE>(v, f, false, 0.0f, o);
+    atomicAdd(hist + min(o.iters, 15u), 1u);
+    if (o.fail) atomicOr(v.box_status + T.box, (unsigned)ST_NEWTON_CAP);
+  }
+  if (v.fixed_acc) {
+#pragma unroll
+    for (int a = 0; a < NM; a++) {
+      const unsigned r = __reduce_max_sync(full, o.m[a]);
+      if (lane == 0 && r) atomicMax(v.fmax_bits + FMAX_STRIDE * T.box + a, r);
+    }
+  }
+  const unsigned it = __reduce_add_sync(full, o.iters), mx = __reduce_max_sync(full, o.iters);
+  const unsigned fa = __popc(__ballot_sync(full, o.fail)), fb = __popc(__ballot_sync(full, o.fallback));
+  if (lane == 0) {
+    red[0] += __popc(todo);
+    red[1] += it;
+    red[2] += __popc(todo);
+    red[4] += fa;
+    red[5] += fb;
+    red[6] = max(red[6], mx);
+  }
+  __syncwarp();
+}
+
 // face of this thread in chunk c of tile T (FACE_TILE / B chunks per tile);
 // faces past the tile's end take the tile's first face (in bounds; their
 // results are not stored)
@@ -81,7 +156,7 @@ __device__ __forceinline__ int chunk_face(int c, const Tile& T, bool& valid) {
 }
 
 template <int B, bool ENT, bool LEARN, bool STATIC>
-__global__ void __launch_bounds__(B, chunk_ctas_per_sm<B>()) k_flux_chunks(HydroView<float> v, int nchunks, int per_cta,
+__global__ void __launch_bounds__(B, chunk_ctas_per_sm<B, STATIC>()) k_flux_chunks(HydroView<float> v, int nchunks, int per_cta,
                                                                           FluxDefer defer) {
   constexpr int CPT = FACE_TILE / B;   // chunks per face tile
   __shared__ ChunkSmem<B> sm;
@@ -95,12 +170,12 @@ __global__ void __launch_bounds__(B, chunk_ctas_per_sm<B>()) k_flux_chunks(Hydro
   if (lane < 8) sm.red[warp][lane] = 0u;
   __syncwarp();
   const bool fixed = v.fixed_acc != 0;
-  // each thread's running maxima of |A F| per component (of the current box),
-  // reduced over the warp when the box changes
+  // the warp's running maxima of |A F| per component (of the current box)
   unsigned fm[NM];
 #pragma unroll
   for (int a = 0; a < NM; a++) fm[a] = 0u;
 
+  bool guarded = false;   // this warp has marked faces
   // tiles of chunks c0 and c0+1, cell indices of c0
   Tile T0 = v.ftiles[c0 / CPT];
   Tile T1 = (c0 + 1 < c1) ? v.ftiles[(c0 + 1) / CPT] : T0;
@@ -123,25 +198,7 @@ __global__ void __launch_bounds__(B, chunk_ctas_per_sm<B>()) k_flux_chunks(Hydro
       hdt = (float)(0.5 * box_dt(v, hbox));
     }
     FaceWork<float> f;
-    {
-      R4<float> G0, G1;
-      ldg256(v.fgeo + 2 * (size_t)k, G0, G1);
-      if constexpr (STATIC) {
-        // the cells' half-step predicted records (gradient kernel)
-        const CellRec<float> pL = load_rec256<ENT>(v, v.cwp, v.Apw, L0.x);
-        const CellRec<float> pR = load_rec256<ENT>(v, v.cwp, v.Apw, L0.y);
-        float AL = 0.0f, AR = 0.0f;
-        if constexpr (ENT) {
-          AL = v.Aw[L0.x];
-          AR = v.Aw[L0.y];
-        }
-        face_prepare_pred<float, ENT>(v, k, valid, L0, G0, G1, pL, pR, AL, AR, f);
-      } else {
-        const CellRec<float> recL = load_rec256<ENT>(v, v.cw, v.Aw, L0.x);
-        const CellRec<float> recR = load_rec256<ENT>(v, v.cw, v.Aw, L0.y);
-        face_prepare_rec<float, ENT>(v, k, valid, hdt, hdt, L0, G0, G1, recL, recR, f);
-      }
-    }
+    chunk_prepare<ENT, STATIC>(v, k, valid, L0, hdt, f);
     bool mine = valid;
     float cs[3];   // c_L, c_R and the linearised star pressure, for the gate and the solver
     if constexpr (LEARN) {
@@ -174,20 +231,19 @@ __global__ void __launch_bounds__(B, chunk_ctas_per_sm<B>()) k_flux_chunks(Hydro
       }
     }
     FaceOut o;
-    face_finish_core<float, ENT>(v, f, false, 0.0f, o, LEARN, cs);
-    if constexpr (STATIC) {
-#pragma unroll
-      for (int a = 0; a < NM; a++) fm[a] = max(fm[a], o.m[a]);
-    } else {
-      // the moving-mesh instantiation holds more live values: a warp
-      // reduction per chunk spills less than five private maxima (measured
-      // 4.6% faster at 64^3)
-#pragma unroll
-      for (int a = 0; a < NM; a++) {
-        const unsigned r = __reduce_max_sync(full, o.m[a]);
-        fm[a] = max(fm[a], r);
+    face_finish_core<float, ENT, GUARD_DEFER>(v, f, false, 0.0f, o, LEARN, cs);
+    {
+      const unsigned gb = __ballot_sync(full, o.guard);
+      if (gb) {
+        if (lane == 0) v.guard_mask[c * (B / 32) + warp] = gb;
+        guarded = true;
+        mine = mine && !o.guard;
       }
     }
+    // the warp's largest |A F| per component (a reduction per chunk: private
+    // running maxima cost five registers each)
+#pragma unroll
+    for (int a = 0; a < NM; a++) fm[a] = max(fm[a], __reduce_max_sync(full, o.m[a]));
     // Newton statistics of the warp: the iteration histogram (the lanes with
     // equal counts found by one match; the lowest of them adds their number,
     // so the lanes that write hold distinct bins), sums and flags
@@ -204,11 +260,10 @@ __global__ void __launch_bounds__(B, chunk_ctas_per_sm<B>()) k_flux_chunks(Hydro
       sm.red[warp][1] += sit;
       sm.red[warp][6] = max(sm.red[warp][6], smx);
     }
-    if (__any_sync(full, o.guard || o.vacuum || o.fail || o.fallback)) {
-      const unsigned g = __popc(__ballot_sync(full, o.guard)), va = __popc(__ballot_sync(full, o.vacuum));
+    if (__any_sync(full, o.vacuum || o.fail || o.fallback)) {
+      const unsigned va = __popc(__ballot_sync(full, o.vacuum));
       const unsigned fa = __popc(__ballot_sync(full, o.fail)), fb = __popc(__ballot_sync(full, o.fallback));
       if (lane == 0) {
-        sm.red[warp][2] += g;
         sm.red[warp][3] += va;
         sm.red[warp][4] += fa;
         sm.red[warp][5] += fb;
@@ -219,14 +274,24 @@ __global__ void __launch_bounds__(B, chunk_ctas_per_sm<B>()) k_flux_chunks(Hydro
     if (fixed && (!more1 || T1.box != T0.box)) {
 #pragma unroll
       for (int a = 0; a < NM; a++) {
-        const unsigned r = __reduce_max_sync(full, fm[a]);
-        if (lane == 0 && r) atomicMax(v.fmax_bits + FMAX_STRIDE * T0.box + a, r);
+        if (lane == 0 && fm[a]) atomicMax(v.fmax_bits + FMAX_STRIDE * T0.box + a, fm[a]);
         fm[a] = 0u;
       }
     }
     T0 = T1;
     T1 = T2;
     L0 = L1;
+  }
+  if (guarded) {
+    // the marked faces, chunk by chunk (the marks are this warp's own)
+    __syncwarp();
+#pragma unroll 1
+    for (int c = c0; c < c1; c++) {
+      const unsigned todo = v.guard_mask[c * (B / 32) + warp];
+      if (!todo) continue;
+      chunk_guard<B, ENT, STATIC>(v, c, todo, sm.hist[warp], sm.red[warp]);
+      if (lane == 0) v.guard_mask[c * (B / 32) + warp] = 0u;
+    }
   }
   // one set of global atomics per CTA for the statistics
   __syncthreads();

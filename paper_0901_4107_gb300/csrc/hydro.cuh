@@ -114,6 +114,49 @@ __device__ __forceinline__ T group_min(T x) {
   return x;
 }
 
+// Extrema and the limiter's maximum.  FP64 comparisons run on the narrow FP64
+// pipe (two of the three instructions a value takes there, besides its
+// difference), so the FP64 form compares in integers: doubles order like their
+// bits with the magnitude bits of negative ones flipped.  (91 k cells: gradients
+// 328 us with FP64 comparisons, 247 now.)
+template <typename real>
+struct Extrema;
+template <>
+struct Extrema<float> {
+  float mx, mn;
+  __device__ __forceinline__ void init(float x) { mx = mn = x; }
+  __device__ __forceinline__ void add(float x) {
+    mx = x > mx ? x : mx;
+    mn = x < mn ? x : mn;
+  }
+  __device__ __forceinline__ float max() const { return mx; }
+  __device__ __forceinline__ float min() const { return mn; }
+};
+template <>
+struct Extrema<double> {
+  long long mx, mn;
+  static __device__ __forceinline__ long long flip(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffll); }
+  __device__ __forceinline__ void init(double x) { mx = mn = flip(__double_as_longlong(x)); }
+  __device__ __forceinline__ void add(double x) {
+    const long long k = flip(__double_as_longlong(x));
+    mx = k > mx ? k : mx;
+    mn = k < mn ? k : mn;
+  }
+  __device__ __forceinline__ double max() const { return __longlong_as_double(flip(mx)); }
+  __device__ __forceinline__ double min() const { return __longlong_as_double(flip(mn)); }
+};
+
+// the larger of m >= 0 and dphi times the reciprocal of its own side, a value
+// that is not negative; a NaN (0 times infinity) is ignored
+__device__ __forceinline__ float limit_max(float m, float dphi, float rmx, float rmn) {
+  return fmaxf(m, dphi * (dphi > 0.0f ? rmx : rmn));
+}
+__device__ __forceinline__ double limit_max(double m, double dphi, double rmx, double rmn) {
+  const double x = dphi * (__double2hiint(dphi) >= 0 ? rmx : rmn);
+  const long long b = __double_as_longlong(x);
+  return (b > __double_as_longlong(m) && b <= 0x7ff0000000000000ll) ? x : m;
+}
+
 // Mesh velocity of cell i for the Courant step and the cold-flow criterion
 template <typename real>
 __device__ __forceinline__ void mesh_velocity(const HydroView<real>& v, int i, const R4<real>& Wi, real* w) {
@@ -158,11 +201,11 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
   const int q0 = valid ? v.csr_off[ii] : 0;
   const int q1 = valid ? v.csr_off[ii + 1] : 0;
   real g[NV][3];
-  real mx[NV], mn[NV];
+  Extrema<real> ex[NV];
 #pragma unroll
   for (int a = 0; a < NV; a++) {
     g[a][0] = g[a][1] = g[a][2] = (real)0;
-    mx[a] = mn[a] = phi_i[a];
+    ex[a].init(phi_i[a]);
   }
   // cold-flow criterion: largest 1/2 m_j |v_j - w_i|^2 over the cell and
   // its neighbours (start-of-step states)
@@ -214,8 +257,7 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
       g[a][0] += d * a4.x;
       g[a][1] += d * a4.y;
       g[a][2] += d * a4.z;
-      mx[a] = phi_j[a] > mx[a] ? phi_j[a] : mx[a];
-      mn[a] = phi_j[a] < mn[a] ? phi_j[a] : mn[a];
+      ex[a].add(phi_j[a]);
     }
   }
   const real invV = cg.x;
@@ -224,8 +266,8 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
     g[a][0] = group_sum<G>(g[a][0]) * invV;
     g[a][1] = group_sum<G>(g[a][1]) * invV;
     g[a][2] = group_sum<G>(g[a][2]) * invV;
-    mx[a] = group_max<G>(mx[a]);
-    mn[a] = group_min<G>(mn[a]);
+    ex[a].mx = group_max<G>(ex[a].mx);
+    ex[a].mn = group_min<G>(ex[a].mn);
   }
   if (v.limit) {
     // alpha = min(1, min over incidences of psi), psi = (max - phi_i) / dphi
@@ -238,8 +280,8 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
 #pragma unroll
     for (int a = 0; a < NV; a++) {
       bmax[a] = (real)0;
-      rmx[a] = (real)1 / (mx[a] - phi_i[a]);
-      rmn[a] = (real)-1 / (phi_i[a] - mn[a]);
+      rmx[a] = (real)1 / (ex[a].max() - phi_i[a]);
+      rmn[a] = (real)-1 / (phi_i[a] - ex[a].min());
     }
   #pragma unroll UNR
   for (int q = q0 + lane; q < q1; q += G) {
@@ -249,7 +291,7 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
 #pragma unroll
       for (int a = 0; a < NV; a++) {
         const real dphi = g[a][0] * fx + g[a][1] * fy + g[a][2] * fz;
-        bmax[a] = fmax(bmax[a], dphi * (dphi > (real)0 ? rmx[a] : rmn[a]));
+        bmax[a] = limit_max(bmax[a], dphi, rmx[a], rmn[a]);
       }
     }
 #pragma unroll
@@ -707,23 +749,39 @@ struct FaceOut {
   bool guard, vacuum, fail, fallback;
 };
 
+// The sampled state of a face's Riemann problem and how it was found.
+template <typename real>
+struct RiemannOut {
+  real rhoF, uF, pF, ps;
+  int side;
+  RiemannInfo info;
+};
+
 // Riemann solve, flux of the moving face and its stores (valid faces only);
 // the face's contributions to the reductions in `o` (zero for an invalid
 // face).  have_guess: start Newton from `guess` in place of the two-shock
 // estimate.  pre: the caller has the sides' sound speeds and the linearised
-// star pressure (cs = {c_L, c_R, p_pv}) already.
-template <typename real, bool ENT>
+// star pressure (cs = {c_L, c_R, p_pv}) already.  given: the caller has solved.
+// GUARD_DEFER: a face that needs the FP64 guard is not stored and contributes
+// only o.guard.
+template <typename real, bool ENT, GuardKind GUARD = GUARD_INLINE>
 __device__ __forceinline__ void face_finish_core(const HydroView<real>& v, const FaceWork<real>& f, bool have_guess,
-                                                 real guess, FaceOut& o, bool pre = false, const real* cs = nullptr) {
+                                                 real guess, FaceOut& o, bool pre = false, const real* cs = nullptr,
+                                                 const RiemannOut<real>* given = nullptr) {
   const GasC<real>& G = v.gas;
-  const bool valid = f.valid;
-  real rhoF, uF, pF, ps;
-  RiemannInfo info;
-  const int side =
-      pre ? riemann_sample_c(f.WppL[0], f.uL, f.WppL[4], f.WppR[0], f.uR, f.WppR[4], cs[0], cs[1], cs[2], G, v.tol,
-                             v.tol_r, v.maxit, have_guess, guess, rhoF, uF, pF, info, ps)
-          : riemann_sample(f.WppL[0], f.uL, f.WppL[4], f.WppR[0], f.uR, f.WppR[4], G, v.tol, v.tol_r, v.maxit,
-                           have_guess, guess, rhoF, uF, pF, info, ps);
+  RiemannOut<real> r;
+  if (given) {
+    r = *given;
+  } else {
+    r.side = pre ? riemann_sample_c<GUARD>(f.WppL[0], f.uL, f.WppL[4], f.WppR[0], f.uR, f.WppR[4], cs[0], cs[1], cs[2], G, v.tol,
+                                    v.tol_r, v.maxit, have_guess, guess, r.rhoF, r.uF, r.pF, r.info, r.ps)
+                 : riemann_sample<GUARD>(f.WppL[0], f.uL, f.WppL[4], f.WppR[0], f.uR, f.WppR[4], G, v.tol, v.tol_r, v.maxit,
+                                  have_guess, guess, r.rhoF, r.uF, r.pF, r.info, r.ps);
+  }
+  const RiemannInfo& info = r.info;
+  const bool valid = f.valid && !(GUARD == GUARD_DEFER && info.guard);
+  const real rhoF = r.rhoF, uF = r.uF, pF = r.pF, ps = r.ps;
+  const int side = r.side;
   const real* Wt = side ? f.WppR : f.WppL;
   const real ut = side ? f.uR : f.uL;
   real vlab[3];
@@ -773,7 +831,7 @@ __device__ __forceinline__ void face_finish_core(const HydroView<real>& v, const
     if constexpr (ENT) o.m[5] = __float_as_uint(fabsf((float)fS));
   }
   o.iters = valid ? (unsigned)info.iters : 0u;
-  o.guard = valid && info.guard;
+  o.guard = f.valid && info.guard;
   o.vacuum = valid && info.vacuum;
   o.fail = valid && info.fail;
   o.fallback = valid && f.fallback;
@@ -797,6 +855,64 @@ __device__ __forceinline__ void stats_add(DeviceStats* S, unsigned* box_status, 
   if (maxit) atomicMax(&S->newton_max, maxit);
 }
 
+// The FP64 form's Riemann problems of a CTA, solved in an order that keeps a
+// warp's lanes on one path.  What bounds the solve is the FP64 pipe, which
+// takes a warp's time for an instruction however few lanes are on: with the
+// faces in their own order each warp ran shocks and rarefactions of both sides
+// and as many iterations as its worst face (11.6 of 32 lanes on).  So the states
+// go through shared memory, ordered by the kind of solve (judged in FP32, on
+// the idle FP32 pipe); every face's arithmetic is the same wherever it runs.
+// 91 k cells, one step's fluxes: 2754 us in face order with pow; 2412 us with
+// pow64 and fewer divisions; 1540 us regrouped (21.7 lanes on).
+template <int B>
+__device__ __forceinline__ void solve_grouped(const HydroView<double>& v, const FaceWork<double>& f,
+                                              RiemannOut<double>& r) {
+  __shared__ double q[9][B];
+  __shared__ int total[SOLVE_KINDS], start[SOLVE_KINDS];
+  __shared__ short order[B];
+  const int t = (int)threadIdx.x;
+  const double rL = f.WppL[0], pL = f.WppL[4], rR = f.WppR[0], pR = f.WppR[4];
+  const double cL = sqrt(rn_mul(v.gas.g, pL) / rL), cR = sqrt(rn_mul(v.gas.g, pR) / rR);
+  const double ppv = linearised_pstar(rL, f.uL, pL, cL, rR, f.uR, pR, cR);
+  const int kind = solve_kind(rL, f.uL, pL, cL, rR, f.uR, pR, cR, ppv, GasC<float>(v.gamma));
+  if (t < SOLVE_KINDS) total[t] = 0;
+  q[0][t] = rL; q[1][t] = f.uL; q[2][t] = pL; q[3][t] = cL;
+  q[4][t] = rR; q[5][t] = f.uR; q[6][t] = pR; q[7][t] = cR; q[8][t] = ppv;
+  __syncthreads();
+  // counting sort (the order within a kind does not matter)
+  const int at = atomicAdd(&total[kind], 1);
+  __syncthreads();
+  if (t < SOLVE_KINDS) {
+    int s = 0;
+    for (int k = 0; k < t; k++) s += total[k];
+    start[t] = s;
+  }
+  __syncthreads();
+  order[start[kind] + at] = (short)t;
+  __syncthreads();
+  const int j = order[t];
+  RiemannOut<double> o;
+  o.side = riemann_sample_c(q[0][j], q[1][j], q[2][j], q[4][j], q[5][j], q[6][j], q[3][j], q[7][j], q[8][j], v.gas, v.tol,
+                            v.tol_r, v.maxit, false, 0.0, o.rhoF, o.uF, o.pF, o.info, o.ps);
+  // (only this thread read column j)
+  q[0][j] = o.rhoF;
+  q[1][j] = o.uF;
+  q[2][j] = o.pF;
+  q[3][j] = o.ps;
+  q[4][j] = __hiloint2double(o.info.iters, o.side | o.info.vacuum << 1 | o.info.fail << 2);
+  __syncthreads();
+  r.rhoF = q[0][t];
+  r.uF = q[1][t];
+  r.pF = q[2][t];
+  r.ps = q[3][t];
+  const int bits = __double2loint(q[4][t]);
+  r.side = bits & 1;
+  r.info.iters = __double2hiint(q[4][t]);
+  r.info.vacuum = (bits >> 1) & 1;
+  r.info.fail = bits >> 2;
+  r.info.guard = 0;
+}
+
 // Riemann solve, flux of the moving face, stores, and the CTA's reductions
 // (largest |A F| per component, Newton statistics).  All B threads call it.
 template <typename real, int B, bool ENT>
@@ -804,7 +920,13 @@ __device__ __forceinline__ void face_finish(const HydroView<real>& v, const Face
                                             bool have_guess, real guess) {
   const bool valid = f.valid;
   FaceOut o;
-  face_finish_core<real, ENT>(v, f, have_guess, guess, o);
+  if constexpr (sizeof(real) == 8) {
+    RiemannOut<double> r;
+    solve_grouped<B>(v, f, r);
+    face_finish_core<real, ENT>(v, f, false, guess, o, false, nullptr, &r);
+  } else {
+    face_finish_core<real, ENT>(v, f, have_guess, guess, o);
+  }
   if (sizeof(real) == 4 && v.fixed_acc) {
     // largest |A F| per component for the exact fixed-point sums
     constexpr int NM = ENT ? 6 : 5;
@@ -879,8 +1001,11 @@ __device__ __forceinline__ void flux_item(const HydroView<real>& v, int wi) {
   face_finish<real, B, ENT>(v, f, t.box, min(B, t.end - first), false, (real)0);
 }
 
+// (FP64: 16 warps per SM, 128 registers; with one CTA of 256 per SM and no
+// spills the barriers of the grouped solve leave the FP64 pipe idle: 1725 us
+// for 1540)
 template <typename real, int B, bool ENT>
-__global__ void __launch_bounds__(B, sizeof(real) == 4 ? 4 * FACE_TILE / B : FACE_TILE / B) k_flux(HydroView<real> v) {
+__global__ void __launch_bounds__(B, sizeof(real) == 4 ? 4 * FACE_TILE / B : 2 * FACE_TILE / B) k_flux(HydroView<real> v) {
   flux_item<real, B, ENT>(v, blockIdx.x);
 }
 
@@ -1484,6 +1609,7 @@ HydroView<real> make_view(amm_ctx* c, double cfl) {
   v.ekmax = (real*)c->ekmax;
   v.kept = c->kept;
   v.mlp = c->mlp;
+  v.guard_mask = c->guard_mask;
   v.harvest = c->harvest;
   return v;
 }
@@ -1545,7 +1671,16 @@ cudaError_t launch_flux(amm_ctx* c, double cfl) {
     return launch_flux_chunks(c, v, false, FluxDefer());
   } else {
     const bool ent = c->opt.entropy != 0;
-    if (b128 && ent)
+    // Few faces: CTAs of 64 spread them over all SMs, whose FP64 pipes are what
+    // bounds the solve; with many the larger CTAs group the faces' solves
+    // better.  (us for faces: 25 k 74 / 86 with 256, 49 k 112 / 141, 98 k 206 /
+    // 239, 715 k 2057 / 1540.)
+    const bool few = c->nf <= 152 * 768;
+    if (few && ent)
+      k_flux<real, 64, true><<<c->n_ftiles * 4, 64, 0, c->stream>>>(v);
+    else if (few)
+      k_flux<real, 64, false><<<c->n_ftiles * 4, 64, 0, c->stream>>>(v);
+    else if (b128 && ent)
       k_flux<real, 128, true><<<c->n_ftiles * 2, 128, 0, c->stream>>>(v);
     else if (b128)
       k_flux<real, 128, false><<<c->n_ftiles * 2, 128, 0, c->stream>>>(v);

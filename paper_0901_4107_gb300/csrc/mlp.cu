@@ -526,9 +526,9 @@ __global__ void k_riemann_pstar(double gamma, int64_t m, const float* st, double
     return;
   }
   RiemannInfo info{0, 0, 0, 0};
-  NewtonTail<double> nt;
+  double us;
   const double p0 = standard_guess(rL, uL, pL, cL, rR, uR, pR, cR, G);
-  const double p = newton_pstar(p0, rL, uL, pL, cL, rR, uR, pR, cR, G, tol, tol, maxit, info, nt);
+  const double p = newton_pstar(p0, rL, uL, pL, cL, rR, uR, pR, cR, G, tol, tol, maxit, info, us);
   pstar[i] = info.fail ? __int_as_float(0x7fc00000) : (float)p;
 }
 
@@ -547,9 +547,9 @@ __global__ void k_mlp_targets(double gamma, int64_t m, const float* st, double t
     return;
   }
   RiemannInfo info{0, 0, 0, 0};
-  NewtonTail<double> nt;
+  double us;
   const double p0 = standard_guess(rL, uL, pL, cL, rR, uR, pR, cR, G);
-  const double p = newton_pstar(p0, rL, uL, pL, cL, rR, uR, pR, cR, G, tol, tol, maxit, info, nt);
+  const double p = newton_pstar(p0, rL, uL, pL, cL, rR, uR, pR, cR, G, tol, tol, maxit, info, us);
   const GasC<float> Gf(gamma);
   const float cLf = sqrtf(Gf.g * s[2] / s[0]), cRf = sqrtf(Gf.g * s[5] / s[3]);
   const float ppv = linearised_pstar(s[0], s[1], s[2], cLf, s[3], s[4], s[5], cRf);

@@ -189,7 +189,7 @@ int amm_retessellate(amm_ctx* c) {
   c->ind_graph = nullptr;
   if (nf > c->nf_cap) {
     const int64_t cap = nf + nf / 8;
-    void** bufs[] = {(void**)&c->lr, (void**)&c->face_perm, (void**)&c->csr, &c->fgeo, &c->igAB, &c->flux, &c->fluxE, &c->fluxS, &c->machf, (void**)&c->ftiles,
+    void** bufs[] = {(void**)&c->lr, (void**)&c->face_perm, (void**)&c->csr, &c->fgeo, &c->igAB, &c->flux, &c->fluxE, &c->fluxS, &c->machf, (void**)&c->ftiles, (void**)&c->guard_mask,
                      (void**)&c->ind_flist, (void**)&c->ind_fstamp, (void**)&c->ind_fdt};
     const bool had_defer = c->defer_list != nullptr;
     if (had_defer) {
@@ -213,6 +213,9 @@ int amm_retessellate(amm_ctx* c) {
       cu(cudaMalloc(&c->machf, rs * cap), "alloc");
     }
     cu(cudaMalloc(&c->ftiles, sizeof(Tile) * ((cap + FACE_TILE - 1) / FACE_TILE)), "alloc");
+    const size_t guard_bytes = sizeof(unsigned) * ((cap + FACE_TILE - 1) / FACE_TILE) * (FACE_TILE / 32);
+    cu(cudaMalloc(&c->guard_mask, guard_bytes), "alloc");
+    if (c->guard_mask) cu(cudaMemsetAsync(c->guard_mask, 0, guard_bytes, st), "memset");
     if (had_defer) cu(cudaMalloc((void**)&c->defer_list, sizeof(int2) * cap), "alloc");
     if (c->ind_ready) {
       cu(cudaMalloc(&c->ind_flist, sizeof(int) * cap), "alloc");

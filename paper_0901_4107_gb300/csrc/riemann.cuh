@@ -26,11 +26,12 @@
 #include <float.h>
 
 #include "amm_internal.cuh"
+#include "pow64.cuh"
 
 namespace amm {
 
 
-__device__ __forceinline__ double xpow(double a, double b) { return pow(a, b); }
+__device__ __forceinline__ double xpow(double a, double b) { return pow64(a, b); }
 __device__ __forceinline__ float xpow(float a, float b) { return __powf(a, b); }
 __device__ __forceinline__ double xsqrt(double a) { return sqrt(a); }
 __device__ __forceinline__ float xsqrt(float a) { return sqrtf(a); }
@@ -56,12 +57,12 @@ __device__ __forceinline__ real rn_dot3(real ax, real ay, real az, real bx, real
   return rn_fma(az, bz, rn_fma(ay, by, rn_mul(ax, bx)));
 }
 
-// f_K(p) and f_K'(p)
-template <typename real>
-__device__ __forceinline__ void wave_curve(real p, real rhoK, real pK, real cK, const GasC<real>& G, real& f,
-                                           real& df) {
-  if constexpr (sizeof(real) == 4) {
-    // FP32: both branches, selected.  The sides of a warp's faces split
+// f_K(p) and f_K'(p), FP32
+__device__ __forceinline__ void wave_curve(float p, float rhoK, float pK, float cK, const GasC<float>& G, float& f,
+                                           float& df) {
+  using real = float;
+  {
+    // both branches, selected.  The sides of a warp's faces split
     // between shocks and rarefactions, so a branch would run both anyway;
     // unconditional, the per-side constants leave the Newton loop.
     const real A = G.two_gp1 / rhoK;
@@ -76,17 +77,43 @@ __device__ __forceinline__ void wave_curve(real p, real rhoK, real pK, real cK, 
     const bool shock = p > pK;
     f = shock ? fs : fr;
     df = shock ? dfs : dfr;
-  } else if (p > pK) {
-    const real A = G.two_gp1 / rhoK;
-    const real B = G.gm1_gp1 * pK;
-    const real q = xsqrt(A / (p + B));
-    f = (p - pK) * q;
-    df = q * ((real)1 - (real)0.5 * (p - pK) / (p + B));
+  }
+}
+
+// FP64: f_K(p) and f_K'(p).  Divisions and square roots cost about
+// ten FP64 instructions each, so the shock takes one reciprocal square root,
+// w = (rho (p + B))^(-1/2): q = sqrt(2/(gamma+1)) w and 1/(p + B) = rho w^2; the
+// rarefaction f' = (p/p_K)^z c_K / (gamma p) (rho_K c_K = gamma p_K / c_K), with
+// 1/p given (both sides need it) and 1/p_K formed once per solve.
+// (explicitly rounded: the persistent step kernel must round alike)
+struct WaveSide {
+  double rho, p, c, ip, B, two_c;   // state, 1/p, B, 2c/(gamma-1)
+};
+__device__ __forceinline__ WaveSide wave_side(double rho, double p, double c, const GasC<double>& G) {
+  WaveSide s;
+  s.rho = rho;
+  s.p = p;
+  s.c = c;
+  s.ip = 1.0 / p;
+  s.B = rn_mul(G.gm1_gp1, p);
+  s.two_c = rn_mul(G.two_gm1, c);
+  return s;
+}
+__device__ __forceinline__ void wave_curve(double p, double ip, const WaveSide& K, const GasC<double>& G, double& f,
+                                           double& df) {
+  const double d = rn_add(p, -K.p);
+  if (d > 0.0) {
+    const double w = rsqrt(rn_mul(K.rho, rn_add(p, K.B)));
+    const double q = rn_mul(G.sqrt_two_gp1, w);
+    const double h = rn_mul(rn_mul(w, w), K.rho);
+    const double dh = rn_mul(d, h);
+    f = rn_mul(d, q);
+    df = rn_mul(q, rn_fma(-0.5, dh, 1.0));
   } else {
-    const real pr = p / pK;
-    const real prz = xpow(pr, G.z);
-    f = G.two_gm1 * cK * (prz - (real)1);
-    df = prz / (pr * rhoK * cK);
+    const double pr = rn_mul(p, K.ip);
+    const double prz = pow64(pr, G.z);
+    f = rn_mul(K.two_c, rn_add(prz, -1.0));
+    df = rn_mul(rn_mul(prz, rn_mul(K.c, G.inv_g)), ip);
   }
 }
 
@@ -102,9 +129,17 @@ __device__ __forceinline__ real linearised_pstar(real rhoL, real uL, real pL, re
 template <typename real>
 __device__ __forceinline__ real two_shock_pstar(real rhoL, real uL, real pL, real rhoR, real uR, real pR, real ppv,
                                                 const GasC<real>& G) {
-  const real gL = xsqrt((G.two_gp1 / rhoL) / (ppv + G.gm1_gp1 * pL));
-  const real gR = xsqrt((G.two_gp1 / rhoR) / (ppv + G.gm1_gp1 * pR));
-  return (gL * pL + gR * pR - (uR - uL)) / (gL + gR);
+  if constexpr (sizeof(real) == 8) {
+    // one reciprocal square root per side (in units of sqrt(2/(gamma+1)))
+    const double gL = rsqrt(rn_mul(rhoL, rn_fma(G.gm1_gp1, pL, ppv)));
+    const double gR = rsqrt(rn_mul(rhoR, rn_fma(G.gm1_gp1, pR, ppv)));
+    const double du = rn_mul(rn_add(uR, -uL), G.isqrt_two_gp1);
+    return rn_add(rn_fma(gL, pL, rn_mul(gR, pR)), -du) / rn_add(gL, gR);
+  } else {
+    const real gL = xsqrt((G.two_gp1 / rhoL) / (ppv + G.gm1_gp1 * pL));
+    const real gR = xsqrt((G.two_gp1 / rhoR) / (ppv + G.gm1_gp1 * pR));
+    return (gL * pL + gR * pR - (uR - uL)) / (gL + gR);
+  }
 }
 
 // Standard starting value: the linearised (primitive-variable) estimate when
@@ -131,11 +166,11 @@ __device__ __forceinline__ real standard_guess_ppv(real rhoL, real uL, real pL, 
     const real ptr = xpow(num / den, G.inv_z);
     const real pts = have ? proposal : two_shock_pstar(rhoL, uL, pL, rhoR, uR, pR, ppv, G);
     p0 = pv ? ppv : (ppv < pmin ? ptr : pts);
-  } else if (pmax / pmin <= (real)2 && ppv >= pmin && ppv <= pmax) {
+  } else if (pmax <= (real)2 * pmin && ppv >= pmin && ppv <= pmax) {
     p0 = ppv;
   } else if (ppv < pmin) {
-    const real num = cL + cR - (real)0.5 * G.gm1 * du;
-    const real den = cL / xpow(pL, G.z) + cR / xpow(pR, G.z);
+    const real num = rn_add(rn_add(cL, cR), -rn_mul(rn_mul((real)0.5, G.gm1), du));
+    const real den = rn_fma(cL, xpow(pL, -G.z), rn_mul(cR, xpow(pR, -G.z)));
     p0 = xpow(num / den, G.inv_z);
   } else if (have) {
     p0 = proposal;
@@ -176,37 +211,74 @@ struct NewtonTail {
 // relative change of p cannot fall below a 1e-12 tolerance.
 constexpr double RESIDUAL_ULPS = 64.0;
 
+// The FP64 Newton iteration: p* from the iterate p; it and conv as in newton_pstar.
+__device__ __forceinline__ double newton_pstar64(double p, const WaveSide& KL, const WaveSide& KR, double du,
+                                                 const GasC<double>& G, double tol, int maxit, int& it, bool& conv,
+                                                 NewtonTail<double>& t) {
+  t.fL = t.dL = t.fR = t.dR = t.dp = 0.0;
+  while (it < maxit) {
+    const double ip = 1.0 / p;
+    wave_curve(p, ip, KL, G, t.fL, t.dL);
+    wave_curve(p, ip, KR, G, t.fR, t.dR);
+    t.dp = 0.0;
+    const double f = rn_add(rn_add(t.fL, t.fR), du);
+    const double small = rn_mul(RESIDUAL_ULPS * DBL_EPSILON, rn_add(rn_add(fabs(t.fL), fabs(t.fR)), fabs(du)));
+    if (fabs(f) <= small) {
+      conv = true;
+      break;
+    }
+    const double D = rn_add(t.dL, t.dR);
+    double pn = rn_add(p, -(f / D));
+    if (!(pn > 0.0)) pn = rn_mul(1e-3, p);
+    it++;
+    t.dp = rn_add(pn, -p);
+    // 2 |dp| / (p_new + p_old) < tol, without the division
+    if (rn_mul(2.0, fabs(t.dp)) < rn_mul(tol, rn_add(pn, p))) {
+      p = pn;
+      conv = true;
+      break;
+    }
+    p = pn;
+  }
+  return p;
+}
+
+// The FP32 forms' rare continuation in FP64: in place, or left to the caller
+// (info.guard set, the returned state unfinished), whose kernel then holds no
+// FP64 solve.
+enum GuardKind { GUARD_INLINE, GUARD_DEFER };
+struct GuardOut {
+  float p, us;
+  int iters, conv;
+};
+__device__ __forceinline__ GuardOut guard_solve(float p, float rhoL, float uL, float pL, float rhoR, float uR,
+                                                    float pR, float g, double tol, int maxit, int it) {
+  const GasC<double> G((double)g);
+  const double rL = rhoL, pLd = pL, rR = rhoR, pRd = pR;
+  NewtonTail<double> t;
+  bool done = false;
+  const double ps = newton_pstar64((double)p, wave_side(rL, pLd, sqrt(G.g * pLd / rL), G),
+                                   wave_side(rR, pRd, sqrt(G.g * pRd / rR), G), (double)uR - (double)uL, G, tol, maxit,
+                                   it, done, t);
+  GuardOut o;
+  o.p = (float)ps;
+  o.us = 0.5f * (uL + uR) + 0.5f * (((float)t.fR - (float)t.fL) + ((float)t.dR - (float)t.dL) * (float)t.dp);
+  o.iters = it;
+  o.conv = done;
+  return o;
+}
 // Newton iteration for p*; returns p* in `real`, with the FP64 guard in the
-// FP32 form.  iterations counted in info.
-template <typename real>
+// FP32 form, and the star velocity us.  iterations counted in info.
+template <GuardKind GUARD = GUARD_INLINE, typename real>
 __device__ __forceinline__ real newton_pstar(real p, real rhoL, real uL, real pL, real cL, real rhoR, real uR,
                                              real pR, real cR, const GasC<real>& G, double tol, real tol_r, int maxit,
-                                             RiemannInfo& info, NewtonTail<real>& tail) {
+                                             RiemannInfo& info, real& us) {
   const real du = uR - uL;
+  NewtonTail<real> tail;
   int it = 0;
   bool conv = false;
   if constexpr (sizeof(real) == 8) {
-    while (it < maxit) {
-      real fL, dL, fR, dR;
-      wave_curve(p, rhoL, pL, cL, G, fL, dL);
-      wave_curve(p, rhoR, pR, cR, G, fR, dR);
-      const real f = fL + fR + du;
-      if (fabs(f) <= RESIDUAL_ULPS * DBL_EPSILON * (fabs(fL) + fabs(fR) + fabs(du))) {
-        tail.fL = fL; tail.dL = dL; tail.fR = fR; tail.dR = dR; tail.dp = (real)0;
-        conv = true;
-        break;
-      }
-      real pn = p - f / (dL + dR);
-      if (!(pn > (real)0)) pn = (real)1e-3 * p;
-      it++;
-      const real ch = (real)2 * fabs(pn - p) / (pn + p);
-      tail.fL = fL; tail.dL = dL; tail.fR = fR; tail.dR = dR; tail.dp = pn - p;
-      p = pn;
-      if (ch < (real)tol) {
-        conv = true;
-        break;
-      }
-    }
+    p = newton_pstar64(p, wave_side(rhoL, pL, cL, G), wave_side(rhoR, pR, cR, G), du, G, tol, maxit, it, conv, tail);
   } else {
     constexpr int FLOAT_ITERS = 12;
     const float tol_f = (float)tol_r;   // the tolerance in FP32, converted once on the host
@@ -234,35 +306,24 @@ __device__ __forceinline__ real newton_pstar(real p, real rhoL, real uL, real pL
     }
     if (to64) {
       info.guard = 1;
-      const GasC<double> G64((double)G.g);
-      double pd = (double)p;
-      const double rL = rhoL, uLd = uL, pLd = pL, rR = rhoR, uRd = uR, pRd = pR;
-      const double cLd = sqrt(G64.g * pLd / rL), cRd = sqrt(G64.g * pRd / rR);
-      const double dud = uRd - uLd;
-      while (it < maxit) {
-        double fL, dL, fR, dR;
-        wave_curve(pd, rL, pLd, cLd, G64, fL, dL);
-        wave_curve(pd, rR, pRd, cRd, G64, fR, dR);
-        const double f = fL + fR + dud;
-        if (fabs(f) <= RESIDUAL_ULPS * DBL_EPSILON * (fabs(fL) + fabs(fR) + fabs(dud))) {
-          tail.fL = (real)fL; tail.dL = (real)dL; tail.fR = (real)fR; tail.dR = (real)dR; tail.dp = (real)0;
-          conv = true;
-          break;
-        }
-        double pn = pd - f / (dL + dR);
-        if (!(pn > 0.0)) pn = 1e-3 * pd;
-        it++;
-        const double ch = 2.0 * fabs(pn - pd) / (pn + pd);
-        tail.fL = (real)fL; tail.dL = (real)dL; tail.fR = (real)fR; tail.dR = (real)dR; tail.dp = (real)(pn - pd);
-        pd = pn;
-        if (ch < tol) {
-          conv = true;
-          break;
-        }
+      if constexpr (GUARD == GUARD_DEFER) {
+        info.iters = it;
+        info.fail = 0;
+        us = (real)0;
+        return p;
       }
-      p = (real)pd;
+      const GuardOut o = guard_solve(p, rhoL, uL, pL, rhoR, uR, pR, G.g, tol, maxit, it);
+      info.iters = o.iters;
+      info.fail = o.conv ? 0 : 1;
+      us = o.us;
+      return o.p;
     }
   }
+  if constexpr (sizeof(real) == 8)
+    us = rn_mul(0.5, rn_add(rn_add(uL, uR),
+                            rn_fma(rn_add(tail.dR, -tail.dL), tail.dp, rn_add(tail.fR, -tail.fL))));
+  else
+    us = (real)0.5 * (uL + uR) + (real)0.5 * ((tail.fR - tail.fL) + (tail.dR - tail.dL) * tail.dp);
   info.iters = it;
   info.fail = conv ? 0 : 1;
   return p;
@@ -274,7 +335,7 @@ __device__ __forceinline__ real newton_pstar(real p, real rhoL, real uL, real pL
 // (0 when vacuum is generated).
 // cL, cR: the sides' sound speeds; ppv: the linearised star pressure (the
 // caller may have formed them already, for the proposal's gate).
-template <typename real>
+template <GuardKind GUARD = GUARD_INLINE, typename real>
 __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, real rhoR, real uR, real pR, real cL,
                                                 real cR, real ppv, const GasC<real>& G, double tol, real tol_r,
                                                 int maxit, bool have_guess, real guess, real& rhoF, real& uF, real& pF,
@@ -317,10 +378,9 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
     return 0;
   }
   const real p0 = standard_guess_ppv(rhoL, uL, pL, cL, rhoR, uR, pR, cR, ppv, G, have_guess, guess);
-  NewtonTail<real> nt;
-  const real ps = newton_pstar(p0, rhoL, uL, pL, cL, rhoR, uR, pR, cR, G, tol, tol_r, maxit, info, nt);
+  real us;
+  const real ps = newton_pstar<GUARD>(p0, rhoL, uL, pL, cL, rhoR, uR, pR, cR, G, tol, tol_r, maxit, info, us);
   pstar = ps;
-  const real us = (real)0.5 * (uL + uR) + (real)0.5 * ((nt.fR - nt.fL) + (nt.dR - nt.dL) * nt.dp);
   // the side the face sees (the contact's upwind side): s = +1 left, -1
   // right; the right side's formulas are the left side's with the velocity
   // signs flipped (products with s are exact), so one path serves both
@@ -359,9 +419,11 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
     if ((real)0 <= s * (uK - s * cK)) {
       rhoF = rhoK; uF = uK; pF = pK;
     } else {
-      const real tail = us - s * cK * xpow(r, G.z);
+      // r^(1/gamma) = r / (r^z)^2
+      const real rz = xpow(r, G.z);
+      const real tail = us - s * cK * rz;
       if ((real)0 > s * tail) {
-        rhoF = rhoK * xpow(r, G.inv_g); uF = us; pF = ps;
+        rhoF = rhoK * (r / rn_mul(rz, rz)); uF = us; pF = ps;
       } else {
         const real c = G.two_gp1 * cK + s * G.gm1_gp1 * uK;
         const real q = c / cK;
@@ -374,13 +436,34 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
   return side;
 }
 
-template <typename real>
+// Which way the FP64 solve of these states will go, judged in FP32: 0 for two
+// rarefactions (the standard guess is then the root itself), else one plus the
+// waves' kinds and whether the guess is far off (more iterations).  Only the
+// grouping of faces into warps uses it.
+constexpr int SOLVE_KINDS = 8;
+__device__ __forceinline__ int solve_kind(double rL, double uL, double pL, double cL, double rR, double uR, double pR,
+                                          double cR, double ppv, const GasC<float>& G) {
+  const float rl = (float)rL, pl = (float)pL, cl = (float)cL, rr = (float)rR, pr = (float)pR, cr = (float)cR;
+  const float du = (float)(uR - uL);
+  const float p0 = standard_guess_ppv<float>(rl, 0.0f, pl, cl, rr, du, pr, cr, (float)ppv, G);
+  float fL, dL, fR, dR;
+  wave_curve(p0, rl, pl, cl, G, fL, dL);
+  wave_curve(p0, rr, pr, cr, G, fR, dR);
+  const float dp = -(fL + fR + du) / (dL + dR);
+  const float p = p0 + dp;
+  if (p <= pl && p <= pr) return 0;
+  const int far = fabsf(dp) > 3e-4f * p0 ? 1 : 0;
+  // left shock, both, right shock: neighbours in this order share a branch
+  return p <= pr ? 1 + far : (p <= pl ? 6 + far : 3 + far);
+}
+
+template <GuardKind GUARD = GUARD_INLINE, typename real>
 __device__ __forceinline__ int riemann_sample(real rhoL, real uL, real pL, real rhoR, real uR, real pR,
                                               const GasC<real>& G, double tol, real tol_r, int maxit, bool have_guess,
                                               real guess, real& rhoF, real& uF, real& pF, RiemannInfo& info,
                                               real& pstar) {
   const real cL = xsqrt(G.g * pL / rhoL), cR = xsqrt(G.g * pR / rhoR);
-  return riemann_sample_c(rhoL, uL, pL, rhoR, uR, pR, cL, cR, linearised_pstar(rhoL, uL, pL, cL, rhoR, uR, pR, cR), G,
+  return riemann_sample_c<GUARD>(rhoL, uL, pL, rhoR, uR, pR, cL, cR, linearised_pstar(rhoL, uL, pL, cL, rhoR, uR, pR, cR), G,
                           tol, tol_r, maxit, have_guess, guess, rhoF, uF, pF, info, pstar);
 }
 
