@@ -146,6 +146,30 @@ struct Extrema<double> {
   __device__ __forceinline__ double min() const { return __longlong_as_double(flip(mn)); }
 };
 
+// x[a] = 1 / x[a] for values that the G lanes of a group all hold.  FP64: lane l
+// divides for a = l, l + G, ..., since a division is some ten instructions of the
+// narrow FP64 pipe for every lane's copy of it (15 per cell were 45% of the
+// gradients' FP64 work; 91 k cells, two lanes: 247 -> 235 us).
+template <int G, int N>
+__device__ __forceinline__ void group_reciprocals(float* x, int) {
+#pragma unroll
+  for (int a = 0; a < N; a++) x[a] = 1.0f / x[a];
+}
+template <int G, int N>
+__device__ __forceinline__ void group_reciprocals(double* x, int lane) {
+#pragma unroll
+  for (int b = 0; b < N; b += G) {
+    double mine = x[b];
+#pragma unroll
+    for (int l = 1; l < G; l++)
+      if (b + l < N && lane == l) mine = x[b + l];
+    mine = 1.0 / mine;
+#pragma unroll
+    for (int l = 0; l < G; l++)
+      if (b + l < N) x[b + l] = G > 1 ? __shfl_sync(0xffffffffu, mine, l, G) : mine;
+  }
+}
+
 // the larger of m >= 0 and dphi times the reciprocal of its own side, a value
 // that is not negative; a NaN (0 times infinity) is ignored
 __device__ __forceinline__ float limit_max(float m, float dphi, float rmx, float rmn) {
@@ -276,12 +300,18 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
     // two reciprocals once per cell and variable, one product per incidence.
     // (An extremal cell's reciprocal is infinite, so a dphi towards it gives
     // alpha = 0; a dphi of 0 gives NaN, which fmax ignores.)
-    real bmax[NV], rmx[NV], rmn[NV];
+    real bmax[NV], rmx[NV], rmn[NV], r[2 * NV];
 #pragma unroll
     for (int a = 0; a < NV; a++) {
       bmax[a] = (real)0;
-      rmx[a] = (real)1 / (ex[a].max() - phi_i[a]);
-      rmn[a] = (real)-1 / (phi_i[a] - ex[a].min());
+      r[2 * a] = ex[a].max() - phi_i[a];
+      r[2 * a + 1] = phi_i[a] - ex[a].min();
+    }
+    group_reciprocals<G, 2 * NV>(r, lane);
+#pragma unroll
+    for (int a = 0; a < NV; a++) {
+      rmx[a] = r[2 * a];
+      rmn[a] = -r[2 * a + 1];
     }
   #pragma unroll UNR
   for (int q = q0 + lane; q < q1; q += G) {
@@ -295,8 +325,11 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
       }
     }
 #pragma unroll
+    for (int a = 0; a < NV; a++) bmax[a] = fmax((real)1, group_max<G>(bmax[a]));
+    group_reciprocals<G, NV>(bmax, lane);
+#pragma unroll
     for (int a = 0; a < NV; a++) {
-      const real al = (real)1 / fmax((real)1, group_max<G>(bmax[a]));
+      const real al = bmax[a];
       g[a][0] *= al;
       g[a][1] *= al;
       g[a][2] *= al;
