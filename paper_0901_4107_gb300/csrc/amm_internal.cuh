@@ -210,7 +210,6 @@ struct IndView {
   double* fdt;                      // [nf] the active face's step
   unsigned* hist;                   // [64] cells per bin
   // pyramid: cells in leaf-bucket order
-  const int* slot_cell;             // [n] slot -> cell
   const int* cell_slot;             // [n] cell -> slot
   const int* leaf_off;              // [leaf buckets + 1]
   DeviceStats* stats;               // status bits (the loop stops on a failure)
@@ -322,7 +321,6 @@ struct amm_ctx {
   int* ind_cstamp = nullptr;
   double* ind_fdt = nullptr;
   unsigned* ind_hist = nullptr;
-  int* ind_slot_cell = nullptr;
   int* ind_cell_slot = nullptr;
   int* ind_leaf_off = nullptr;
   int* ind_level_off = nullptr;

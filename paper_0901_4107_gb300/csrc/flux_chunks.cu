@@ -103,8 +103,7 @@ __device__ __forceinline__ void chunk_prepare(const HydroView<float>& v, int k, 
 }
 
 // The chunk's faces that need the FP64 guard, by their warp: the whole face
-// again, with the solve in FP64, and its contributions (out of line: nothing
-// of it in the loop's registers).
+// again, with the solve in FP64, and its contributions.
 template <int B, bool ENT, bool STATIC>
 __device__ __forceinline__ void chunk_guard(const HydroView<float>& v, int c, unsigned todo, unsigned* hist, unsigned* red) {
   constexpr int CPT = FACE_TILE / B, NM = ENT ? 6 : 5;

@@ -953,12 +953,14 @@ __device__ __forceinline__ void face_finish(const HydroView<real>& v, const Face
                                             bool have_guess, real guess) {
   const bool valid = f.valid;
   FaceOut o;
-  if constexpr (sizeof(real) == 8) {
+  if constexpr (sizeof(real) == 8 && B > 32) {
     RiemannOut<double> r;
     solve_grouped<B>(v, f, r);
     face_finish_core<real, ENT>(v, f, false, guess, o, false, nullptr, &r);
   } else {
-    face_finish_core<real, ENT>(v, f, have_guess, guess, o);
+    // (one warp of FP64 faces: the caller gives lanes l and l ^ 16 the same face)
+    constexpr GuardKind SOLVE = sizeof(real) == 8 ? SOLVE_PAIRED : GUARD_INLINE;
+    face_finish_core<real, ENT, SOLVE>(v, f, have_guess, guess, o);
   }
   if (sizeof(real) == 4 && v.fixed_acc) {
     // largest |A F| per component for the exact fixed-point sums

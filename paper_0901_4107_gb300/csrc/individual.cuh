@@ -90,39 +90,63 @@ __global__ void k_ind_activate(HydroView<real> v, IndView d) {
 }
 
 // ------------------------------------------------------------ the pyramid
-static __global__ void k_ind_leaf(IndView d) {
-  const int nb = d.level_off[d.levels - 1];
-  const int leaves = (d.dim == 3) ? (1 << (3 * (d.levels - 1))) : (1 << (2 * (d.levels - 1)));
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= leaves) return;
+// coordinates of bucket b of a level
+__device__ __forceinline__ void bucket_coords(int dim, int l, int b, int& ix, int& iy, int& iz) {
+  const int m = (1 << l) - 1;
+  if (dim == 3) {
+    ix = b >> (2 * l); iy = (b >> l) & m; iz = b & m;
+  } else {
+    ix = b >> l; iy = b & m; iz = 0;
+  }
+}
+
+// The two finest levels: a warp per bucket of the second finest, its lanes shared
+// out among the 2^dim leaf buckets in it, so that the records of a leaf are read at
+// once instead of one behind the other (a thread per leaf took 20 us a tick,
+// 4.5 now).
+static __global__ void __launch_bounds__(256) k_ind_leaf(IndView d) {
+  const int l = d.levels - 2, side = 1 << l, cs = 2 * side;
+  const int per = 1 << (d.dim * l);
+  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (b >= per) return;
+  const int lanes = 32 >> d.dim, q = lane / lanes;
+  int ix, iy, iz;
+  bucket_coords(d.dim, l, b, ix, iy, iz);
+  const int jx = 2 * ix + (q & 1), jy = 2 * iy + ((q >> 1) & 1), jz = 2 * iz + ((q >> 2) & 1);
+  const int leaf = (d.dim == 3) ? (jx * cs + jy) * cs + jz : jx * cs + jy;
   // FP32 records, the maximum raised by 1e-5 to cover their rounding (the
   // bounds are used in FP32 only); an empty bucket keeps -1 and a valid slot
   float m = -1.0f;
-  int arg = d.leaf_off[b];
-  for (int s = d.leaf_off[b]; s < d.leaf_off[b + 1]; s++) {
+  const int s0 = d.leaf_off[leaf], s1 = d.leaf_off[leaf + 1];
+  int arg = min(s0, d.n - 1);
+  for (int s = s0 + lane % lanes; s < s1; s += lanes) {
     const float4 a = d.rec32[2 * (size_t)s], c = d.rec32[2 * (size_t)s + 1];
     if (a.w + c.w > m) {
       m = a.w + c.w;
       arg = s;
     }
   }
-  if (arg >= d.n) arg = d.n - 1;
-  d.node[nb + b] = make_float2(m >= 0.0f ? m * (1.0f + 1e-5f) : -1.0f, __int_as_float(arg));
+  if (m >= 0.0f) m *= 1.0f + 1e-5f;
+  for (int o = 1; o < 32; o <<= 1) {
+    if (o == lanes && lane % lanes == 0) d.node[d.level_off[l + 1] + leaf] = make_float2(m, __int_as_float(arg));
+    const float mo = __shfl_xor_sync(0xffffffffu, m, o);
+    const int ao = __shfl_xor_sync(0xffffffffu, arg, o);
+    if (mo > m || (mo == m && ao < arg)) {
+      m = mo;
+      arg = ao;
+    }
+  }
+  if (lane == 0) d.node[d.level_off[l] + b] = make_float2(m, __int_as_float(arg));
 }
 
 // all coarser levels by one CTA, finest first
 static __global__ void __launch_bounds__(1024) k_ind_up(IndView d) {
   const int ch = (d.dim == 3) ? 8 : 4;
-  for (int l = d.levels - 2; l >= 0; l--) {
-    const int per = (d.dim == 3) ? (1 << l) * (1 << l) * (1 << l) : (1 << l) * (1 << l);
-    const int side = 1 << l;
+  for (int l = d.levels - 3; l >= 0; l--) {
+    const int per = 1 << (d.dim * l), side = 1 << l;
     for (int b = threadIdx.x; b < per; b += blockDim.x) {
       int ix, iy, iz;
-      if (d.dim == 3) {
-        ix = b / (side * side); iy = (b / side) % side; iz = b % side;
-      } else {
-        ix = b / side; iy = b % side; iz = 0;
-      }
+      bucket_coords(d.dim, l, b, ix, iy, iz);
       const int cs = side * 2;
       float2 m = make_float2(-2.0f, 0.0f);
       for (int q = 0; q < ch; q++) {
@@ -138,13 +162,17 @@ static __global__ void __launch_bounds__(1024) k_ind_up(IndView d) {
 }
 
 // ---------------------------------------------------- gradients of active cells
+// The active cells' gradients by CTAs of BINS_WARPS warps, G lanes per cell.  The
+// warps of a round are numbered across the CTAs first, so that few cells spread
+// over all SMs' FP64 pipes.
+constexpr int BINS_WARPS = 4;
 template <typename real, int G>
-__global__ void __launch_bounds__(CELL_TILE) k_ind_grad(HydroView<real> v, IndView d) {
-  constexpr int CELLS = CELL_TILE / G;
+__device__ __forceinline__ void ind_grad(const HydroView<real>& v, const IndView& d, int cta, int ctas) {
+  constexpr int CELLS = 32 / G;
   const int count = d.count[0];
   const int lane = (int)threadIdx.x % G;
-  for (int blk = blockIdx.x; blk * CELLS < count; blk += gridDim.x) {
-    const int idx = blk * CELLS + (int)threadIdx.x / G;
+  for (int w = ((int)threadIdx.x >> 5) * ctas + cta; w * CELLS < count; w += ctas * BINS_WARPS) {
+    const int idx = w * CELLS + ((int)threadIdx.x & 31) / G;
     const bool valid = idx < count;
     const int i = d.list[valid ? idx : 0];
     R4<real> Wi, cg;
@@ -182,13 +210,13 @@ __device__ __forceinline__ double pair_tau(const IndView& d, int s, double xi, d
   return sig > 0.0 ? r / sig : INFINITY;
 }
 
+// the warp's minimum of non-negative values (which order like their bits: no
+// FP64 comparisons)
 __device__ __forceinline__ double warp_min_d(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double y = __shfl_xor_sync(0xffffffffu, x, o);
-    x = y < x ? y : x;
-  }
-  return x;
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned h = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned l = __reduce_min_sync(0xffffffffu, hi == h ? lo : 0xffffffffu);
+  return __hiloint2double((int)h, (int)l);
 }
 
 // FP32 bounds of a pair's value r / sig, from the FP32 records, with margins
@@ -232,202 +260,255 @@ __device__ __forceinline__ void pair_tau_bounds(const IndView& d, int s, float x
 // tau_i = min_j r_ij / (c_i + c_j - v_ij . r_ij / r_ij) by a walk of the
 // pyramid.  A bucket cannot hold a pair below gap / (c_i + |v_i| + max_j
 // (c_j + |v_j|)) (r >= gap, signal speed <= c_i + c_j + |v_i - v_j|); the walk
-// skips buckets whose bound is not below the current minimum and opens the
-// others smallest bound first (the children of a bucket are pushed in order).
+// skips buckets whose bound is not below the current one and opens the others.
 // The bounds and a first screen of the pairs run in FP32 with conservative
 // margins; every pair that passes the screen is evaluated exactly in FP64, so
-// the minimum is the FP64 minimum over all pairs.  It starts from the pairs
-// with the fastest cell of every bucket of a coarse level (any pair value
-// bounds the minimum).  The lanes split a bucket's children, a leaf's cells
-// and the seeds; the stack is per warp in shared memory.
-constexpr int BINS_WARPS = 4;
+// the minimum is the FP64 minimum over all pairs, in whatever order it is
+// found.  It starts from the pairs with the fastest cell of every bucket of a
+// coarse level (any pair value bounds the minimum) and the cells of the 3^dim
+// buckets around the cell.
+//
+// What bounds it is the latency of one warp's chain, for most ticks start few
+// cells: so a step of the walk opens as many buckets as their children fill the
+// lanes (32 / 2^dim), from the top of a stack; the buckets to scan are gathered
+// and their cells spread over the lanes; and the pairs that pass the screen are
+// listed and evaluated together at the end.  (With one bucket opened per step,
+// a lane per bucket scanned, FP64 pairs at once and 64 cells a bucket: 92 us for a few
+// cells, 1.5 ms for 32768; 25 us and 0.34 ms now.)
+constexpr int WALK_STACK = 256;   // a step pops 32 / 2^dim buckets and pushes at most 32, over at most 9 levels
+constexpr int WALK_PENDING = 64;
+
+struct WalkShared {
+  unsigned node[WALK_STACK];
+  float lb[WALK_STACK];
+  int base[33], off[33];          // a scan's runs of slots
+  int leaf[32];                   // buckets to scan
+  int pending[WALK_PENDING];      // pairs to evaluate exactly
+};
+
+// the cell the walk is for, and its bounds
+struct WalkCell {
+  int self;                       // its slot
+  double xi, yi, zi, ci, vx, vy, vz;
+  float xf, yf, zf, cf, vxf, vyf, vzf, eps;
+  double cur;                     // the minimum so far, exact
+  float curf;                     // an upper bound of the minimum
+  int npend;
+};
+
+__device__ __forceinline__ void walk_flush(const IndView& d, WalkShared& S, WalkCell& C, int lane) {
+  __syncwarp();
+  double t = INFINITY;
+  for (int q = lane; q < C.npend; q += 32) {
+    const double ts = pair_tau(d, S.pending[q], C.xi, C.yi, C.zi, C.ci, C.vx, C.vy, C.vz);
+    t = ts < t ? ts : t;
+  }
+  t = warp_min_d(t);
+  C.npend = 0;
+  if (t < C.cur) {
+    C.cur = t;
+    C.curf = fminf(C.curf, (float)t * (1.0f + 1e-5f));
+  }
+  __syncwarp();
+}
+
+// The cells of the lanes' runs [s0, s1) of slots, SCAN_PER a lane at a time: their
+// upper bounds tighten curf, then those whose lower bound stays below it are listed.
+constexpr int SCAN_PER = 8;
+__device__ __forceinline__ void walk_scan(const IndView& d, WalkShared& S, WalkCell& C, int lane, int s0, int s1) {
+  const int cnt = s1 - s0;
+  int pre = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, pre, o);
+    if (lane >= o) pre += y;
+  }
+  __syncwarp();
+  S.base[lane] = s0;
+  S.off[lane] = pre - cnt;
+  const int total = __shfl_sync(0xffffffffu, pre, 31);
+  __syncwarp();
+  for (int q0 = 0; q0 < total; q0 += 32 * SCAN_PER) {
+    float lo[SCAN_PER], hmin = INFINITY;
+    int slot[SCAN_PER];
+#pragma unroll
+    for (int u = 0; u < SCAN_PER; u++) {
+      const int q = q0 + 32 * u + lane;
+      int r = 0;   // the last run that starts at or before q
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        if (S.off[r + o] <= q) r += o;
+      const int s = q < total ? S.base[r] + (q - S.off[r]) : C.self;
+      float hi;
+      pair_tau_bounds(d, s, C.xf, C.yf, C.zf, C.cf, C.vxf, C.vyf, C.vzf, C.eps, lo[u], hi);
+      if (s == C.self) lo[u] = hi = INFINITY;
+      hmin = fminf(hmin, hi);
+      slot[u] = s;
+    }
+    C.curf = fminf(C.curf, __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(hmin))));
+#pragma unroll
+    for (int u = 0; u < SCAN_PER; u++) {
+      const bool need = lo[u] < C.curf;
+      const unsigned m = __ballot_sync(0xffffffffu, need);
+      if (m == 0u) continue;
+      if (C.npend + __popc(m) > WALK_PENDING) walk_flush(d, S, C, lane);
+      if (need) S.pending[C.npend + __popc(m & ((1u << lane) - 1u))] = slot[u];
+      C.npend += __popc(m);
+    }
+  }
+}
+
+// first node of a pyramid level
+__device__ __forceinline__ int level_start(int l, int dim) { return dim == 3 ? ((1 << (3 * l)) - 1) / 7 : ((1 << (2 * l)) - 1) / 3; }
 
 template <typename real>
-__global__ void __launch_bounds__(32 * BINS_WARPS) k_ind_bins(HydroView<real> v, IndView d) {
-  __shared__ unsigned s_node[BINS_WARPS][64];
-  __shared__ float s_lb[BINS_WARPS][64];
+__device__ __forceinline__ void ind_bins(const HydroView<real>& v, const IndView& d, int cta, int ctas) {
+  __shared__ WalkShared shared[BINS_WARPS];
+  const unsigned full = 0xffffffffu;
   const int lane = (int)threadIdx.x & 31, w = (int)threadIdx.x >> 5;
+  WalkShared& S = shared[w];
   const int count = d.count[0];
   const long long tick = d.loop->tick;
-  const float eps = 1e-6f * (float)fmax(d.box[0], fmax(d.box[1], d.box[2]));
-  for (int idx = blockIdx.x * BINS_WARPS + w; idx < count; idx += gridDim.x * BINS_WARPS) {
+  const float bx = (float)d.box[0], by = (float)d.box[1], bz = (float)d.box[2];
+  for (int idx = w * ctas + cta; idx < count; idx += ctas * BINS_WARPS) {
     const int i = d.list[idx];
     // the cell's position, sound speed, velocity and speed in FP64: the walk
     // record the activation kernel wrote (one thread per cell), rather than
     // every lane of this warp repeating the FP64 square roots on the narrow
     // FP64 pipe
-    double ci, si, vx, vy, vz, xi = 0.0, yi = 0.0, zi = 0.0;
+    WalkCell C;
+    double si;
     if (d.signal) {
       const int slot = d.cell_slot[i];
+      C.self = slot;
       const double4 ra = d.rec[2 * (size_t)slot], rb = d.rec[2 * (size_t)slot + 1];
-      xi = ra.x; yi = ra.y; zi = ra.z; ci = ra.w;
-      vx = rb.x; vy = rb.y; vz = rb.z; si = rb.w;
+      C.xi = ra.x; C.yi = ra.y; C.zi = ra.z; C.ci = ra.w;
+      C.vx = rb.x; C.vy = rb.y; C.vz = rb.z; si = rb.w;
     } else {
       const R4<real> wi = v.cw[2 * (size_t)i];
       const double rho = (double)wi.x, P = (double)v.cw[2 * (size_t)i + 1].x;
-      vx = (double)wi.y; vy = (double)wi.z; vz = (double)wi.w;
-      ci = sqrt(d.gamma * P / rho);
-      si = sqrt(vx * vx + vy * vy + vz * vz);
+      C.vx = (double)wi.y; C.vy = (double)wi.z; C.vz = (double)wi.w;
+      C.xi = C.yi = C.zi = 0.0;
+      C.ci = sqrt(d.gamma * P / rho);
+      si = sqrt(C.vx * C.vx + C.vy * C.vy + C.vz * C.vz);
     }
-    double cur = (double)v.crad[i] / (ci + si);           // R_i / (c_i + |v_i|)
+    double cur = (double)v.crad[i] / (C.ci + si);           // R_i / (c_i + |v_i|)
     if (d.signal) {
-      const float xf = (float)xi, yf = (float)yi, zf = (float)zi;
-      const float cf = (float)ci, vxf = (float)vx, vyf = (float)vy, vzf = (float)vz;
-      const float minef = (float)(ci + si);
-      const float bx = (float)d.box[0], by = (float)d.box[1], bz = (float)d.box[2];
+      C.cur = cur;
+      C.npend = 0;
+      C.xf = (float)C.xi; C.yf = (float)C.yi; C.zf = (float)C.zi;
+      C.cf = (float)C.ci; C.vxf = (float)C.vx; C.vyf = (float)C.vy; C.vzf = (float)C.vz;
+      C.eps = 1e-6f * fmaxf(bx, fmaxf(by, bz));
+      const float minef = (float)(C.ci + si);
       // the pruning bound curf >= the FP64 minimum: the local term, and upper
       // bounds of the pairs with the fastest cell of each coarse bucket
-      float curf = (float)cur * (1.0f + 1e-5f);
+      C.curf = (float)cur * (1.0f + 1e-5f);
+      const int leaf = d.levels - 1;
+      const int ls = leaf < 2 ? leaf : 2;
       {
-        const int ls = d.levels - 1 < 2 ? d.levels - 1 : 2;
+        const int n0 = level_start(ls, d.dim), n1 = level_start(ls + 1, d.dim);
         float t = INFINITY;
-        for (int b = d.level_off[ls] + lane; b < d.level_off[ls + 1]; b += 32) {
+        for (int b = n0 + lane; b < n1; b += 32) {
           const int s = __float_as_int(d.node[b].y);
-          if (d.slot_cell[s] != i) {
+          if (s != C.self) {
             float lo, hi;
-            pair_tau_bounds(d, s, xf, yf, zf, cf, vxf, vyf, vzf, eps, lo, hi);
+            pair_tau_bounds(d, s, C.xf, C.yf, C.zf, C.cf, C.vxf, C.vyf, C.vzf, C.eps, lo, hi);
             t = hi < t ? hi : t;
           }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t = fminf(t, __shfl_xor_sync(0xffffffffu, t, o));
-        curf = t < curf ? t : curf;
+        C.curf = fminf(C.curf, __uint_as_float(__reduce_min_sync(full, __float_as_uint(t))));
       }
-      const int leaf = d.levels - 1;
-      const int nch = (d.dim == 3) ? 8 : 4;
+      const int lnch = d.dim;                    // log2 of the children per bucket
+      const int nch = 1 << lnch;
       // the cell's own leaf bucket and its 3^dim - 1 neighbours first (lane q
       // takes neighbour q), so the walk below starts from a tight bound and
       // skips them
       const int lside = 1 << leaf;
-      const int lx = min(lside - 1, max(0, (int)floorf(xf / bx * (float)lside)));
-      const int ly = min(lside - 1, max(0, (int)floorf(yf / by * (float)lside)));
-      const int lz = (d.dim == 3) ? min(lside - 1, max(0, (int)floorf(zf / bz * (float)lside))) : 0;
+      const int lx = min(lside - 1, max(0, (int)floorf(C.xf / bx * (float)lside)));
+      const int ly = min(lside - 1, max(0, (int)floorf(C.yf / by * (float)lside)));
+      const int lz = (d.dim == 3) ? min(lside - 1, max(0, (int)floorf(C.zf / bz * (float)lside))) : 0;
       {
         const int nnb = (d.dim == 3) ? 27 : 9;
         int s0 = 0, s1 = 0;
         if (lane < nnb) {
           const int qx = lane % 3 - 1, qy = (lane / 3) % 3 - 1, qz = (d.dim == 3) ? lane / 9 - 1 : 0;
-          const int jx = (lx + qx + lside) % lside, jy = (ly + qy + lside) % lside, jz = (lz + qz + lside) % lside;
+          const int jx = (lx + qx + lside) & (lside - 1), jy = (ly + qy + lside) & (lside - 1),
+                    jz = (lz + qz + lside) & (lside - 1);
           const int b = (d.dim == 3) ? (jx * lside + jy) * lside + jz : jx * lside + jy;
           s0 = d.leaf_off[b];
           s1 = d.leaf_off[b + 1];
         }
-        float hmin = INFINITY;
-        for (int s = s0; s < s1; s++) {
-          if (d.slot_cell[s] == i) continue;
-          float lo, hi;
-          pair_tau_bounds(d, s, xf, yf, zf, cf, vxf, vyf, vzf, eps, lo, hi);
-          hmin = hi < hmin ? hi : hmin;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) hmin = fminf(hmin, __shfl_xor_sync(0xffffffffu, hmin, o));
-        curf = hmin < curf ? hmin : curf;
-        double t = INFINITY;
-        for (int s = s0; s < s1; s++) {
-          if (d.slot_cell[s] == i) continue;
-          float lo, hi;
-          pair_tau_bounds(d, s, xf, yf, zf, cf, vxf, vyf, vzf, eps, lo, hi);
-          if (lo < curf) {
-            const double ts = pair_tau(d, s, xi, yi, zi, ci, vx, vy, vz);
-            t = ts < t ? ts : t;
-          }
-        }
-        t = warp_min_d(t);
-        if (t < cur) {
-          cur = t;
-          const float cu = (float)cur * (1.0f + 1e-5f);
-          curf = cu < curf ? cu : curf;
-        }
+        walk_scan(d, S, C, lane, s0, s1);
       }
-      int sp = 1;
+      // the walk from the root; leaves to scan are gathered until 32 are there
+      // or the stack is empty
+      int sp = 1, nleaf = 0;
       if (lane == 0) {
-        s_node[w][0] = 0u;                                 // level 0, bucket 0
-        s_lb[w][0] = 0.0f;
+        S.node[0] = 0u;                          // level 0, bucket 0
+        S.lb[0] = 0.0f;
       }
       __syncwarp();
-      while (sp > 0) {
-        sp--;
-        const unsigned e = s_node[w][sp];
-        const float lbe = s_lb[w][sp];
-        __syncwarp();
-        if (!(lbe < curf)) continue;
-        const int l = (int)(e >> 27);
-        const int ix = (int)((e >> 18) & 511u), iy = (int)((e >> 9) & 511u), iz = (int)(e & 511u);
-        const int side = 1 << l;
-        if (l == leaf) {
-          const int b = (d.dim == 3) ? (ix * side + iy) * side + iz : ix * side + iy;
-          // first the FP32 upper bounds tighten curf, then only the pairs
-          // whose lower bound stays below it are evaluated in FP64
-          const int s0 = d.leaf_off[b], s1 = d.leaf_off[b + 1];
-          float hmin = INFINITY;
-          for (int s = s0 + lane; s < s1; s += 32) {
-            if (d.slot_cell[s] == i) continue;
-            float lo, hi;
-            pair_tau_bounds(d, s, xf, yf, zf, cf, vxf, vyf, vzf, eps, lo, hi);
-            hmin = hi < hmin ? hi : hmin;
+      while (sp > 0 || nleaf > 0) {
+        if (sp == 0 || nleaf > 32 - nch) {
+          int s0 = 0, s1 = 0;
+          if (lane < nleaf) {
+            s0 = d.leaf_off[S.leaf[lane]];
+            s1 = d.leaf_off[S.leaf[lane] + 1];
           }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) hmin = fminf(hmin, __shfl_xor_sync(0xffffffffu, hmin, o));
-          curf = hmin < curf ? hmin : curf;
-          double t = INFINITY;
-          for (int s = s0 + lane; s < s1; s += 32) {
-            if (d.slot_cell[s] == i) continue;
-            float lo, hi;
-            pair_tau_bounds(d, s, xf, yf, zf, cf, vxf, vyf, vzf, eps, lo, hi);
-            if (lo < curf) {
-              const double ts = pair_tau(d, s, xi, yi, zi, ci, vx, vy, vz);
-              t = ts < t ? ts : t;
-            }
-          }
-          t = warp_min_d(t);
-          if (t < cur) {
-            cur = t;
-            const float cu = (float)cur * (1.0f + 1e-5f);
-            curf = cu < curf ? cu : curf;
-          }
+          nleaf = 0;
+          walk_scan(d, S, C, lane, s0, s1);
           continue;
         }
-        // lane q < nch takes child q: its bound, then its rank among the
-        // surviving children (larger bound deeper in the stack)
-        const int cside = side * 2;
-        bool ok = false;
+        // open up to 32 / nch buckets from the top (as many as leave room for
+        // their leaves); lane q takes child q % nch of the q / nch-th
+        const int take = min(sp, min(32, 32 - nleaf) >> lnch);
+        sp -= take;
+        const int par = lane >> lnch, ch = lane & (nch - 1);
+        bool ok = false, isleaf = false;
         float lb = 0.0f;
         unsigned ce = 0u;
-        if (lane < nch) {
-          const unsigned jx = 2u * ix + (lane & 1), jy = 2u * iy + ((lane >> 1) & 1), jz = 2u * iz + ((lane >> 2) & 1);
-          const int cb = (d.dim == 3) ? ((int)jx * cside + (int)jy) * cside + (int)jz : (int)jx * cside + (int)jy;
-          const float fast = d.node[d.level_off[l + 1] + cb].x;
+        int cb = 0;
+        if (par < take && S.lb[sp + par] < C.curf) {
+          const unsigned e = S.node[sp + par];
+          const int l = (int)(e >> 27) + 1;      // the children's level
+          const unsigned jx = 2u * ((e >> 18) & 511u) + (ch & 1), jy = 2u * ((e >> 9) & 511u) + ((ch >> 1) & 1),
+                         jz = 2u * (e & 511u) + ((ch >> 2) & 1);
+          const int cside = 1 << l;
+          cb = (d.dim == 3) ? ((int)jx * cside + (int)jy) * cside + (int)jz : (int)jx * cside + (int)jy;
+          const float fast = d.node[level_start(l, d.dim) + cb].x;
+          isleaf = l == leaf;
           bool near = false;
-          if (l + 1 == leaf) {
+          if (isleaf) {
             // a leaf of the neighbourhood scanned above (periodic distance <= 1)
             const int ax = abs((int)jx - lx), ay = abs((int)jy - ly), az = abs((int)jz - lz);
             near = min(ax, lside - ax) <= 1 && min(ay, lside - ay) <= 1 && min(az, lside - az) <= 1;
           }
           if (fast >= 0.0f && !near) {
-            const float hx = bx / (float)cside, hy = by / (float)cside, hz = bz / (float)cside;
-            const float gx = interval_gap(xf, (float)jx * hx, hx, bx);
-            const float gy = interval_gap(yf, (float)jy * hy, hy, by);
-            const float gz = (d.dim == 3) ? interval_gap(zf, (float)jz * hz, hz, bz) : 0.0f;
-            const float gap = fmaxf(sqrtf(gx * gx + gy * gy + gz * gz) - eps, 0.0f);
+            const float inv = __int_as_float((127 - l) << 23);   // 1 / cside
+            const float hx = bx * inv, hy = by * inv, hz = bz * inv;
+            const float gx = interval_gap(C.xf, (float)jx * hx, hx, bx);
+            const float gy = interval_gap(C.yf, (float)jy * hy, hy, by);
+            const float gz = (d.dim == 3) ? interval_gap(C.zf, (float)jz * hz, hz, bz) : 0.0f;
+            const float gap = fmaxf(sqrtf(gx * gx + gy * gy + gz * gz) - C.eps, 0.0f);
             lb = gap / ((minef + fast) * (1.0f + 1e-5f));
-            ok = lb < curf;
-            ce = ((unsigned)(l + 1) << 27) | (jx << 18) | (jy << 9) | jz;
+            ok = lb < C.curf;
+            ce = ((unsigned)l << 27) | (jx << 18) | (jy << 9) | jz;
           }
         }
-        const unsigned okm = __ballot_sync(0xffffffffu, ok);
-        int rank = 0;
-        for (int q = 0; q < nch; q++) {
-          const float lq = __shfl_sync(0xffffffffu, lb, q);
-          if (((okm >> q) & 1u) && (lq > lb || (lq == lb && q < lane))) rank++;
+        __syncwarp();                            // (the popped entries are read)
+        const unsigned lm = __ballot_sync(full, ok && isleaf), nm = __ballot_sync(full, ok && !isleaf);
+        const unsigned below = (1u << lane) - 1u;
+        if (ok && isleaf) S.leaf[nleaf + __popc(lm & below)] = cb;
+        if (ok && !isleaf) {
+          S.node[sp + __popc(nm & below)] = ce;
+          S.lb[sp + __popc(nm & below)] = lb;
         }
-        const int nok = __popc(okm);
-        if (ok && sp + rank < 64) {
-          s_node[w][sp + rank] = ce;
-          s_lb[w][sp + rank] = lb;
-        }
+        nleaf += __popc(lm);
+        sp += __popc(nm);
         __syncwarp();
-        sp = sp + nok < 64 ? sp + nok : 64;
       }
+      walk_flush(d, S, C, lane);
+      cur = C.cur;
     }
     if (lane == 0) {
       const double dti = d.cfl * cur;
@@ -483,14 +564,42 @@ __global__ void k_ind_faces(HydroView<real> v, IndView d) {
 }
 
 // ---------------------------------------------------- fluxes of active faces
+// Gradients and bins of the active cells need nothing of one another: odd CTAs take
+// the ones, even CTAs the others, so that the two chains of a tick with few cells
+// overlap.  Few cells get 16 lanes each for their gradients, about an incidence a
+// lane; many get 4.  (Two kernels, the gradients with 4 lanes in CTAs of 256: 25 + 92 us
+// a tick for some 70 cells, 24 now, and 1.6 -> 0.52 ms for 32768 cells.)
+template <typename real>
+__global__ void __launch_bounds__(32 * BINS_WARPS, 4) k_ind_cells(HydroView<real> v, IndView d, int few) {
+  const int cta = (int)blockIdx.x >> 1, ctas = (int)gridDim.x >> 1;
+  if ((blockIdx.x & 1) == 0)
+    ind_bins(v, d, cta, ctas);
+  else if (d.count[0] <= few)
+    ind_grad<real, 16>(v, d, cta, ctas);
+  else
+    ind_grad<real, 4>(v, d, cta, ctas);
+}
+
+// Runs for more than `above` active faces and at most `most`.  FP64 form: what
+// bounds the few faces of most ticks is the chain of one warp's FP64 instructions,
+// which cost the same however few lanes are on; so warps (B = 32) take few faces each,
+// down to one, with a lane for each side of a face, and the pipes of all SMs are used (70 us a tick
+// with CTAs of 128 for some 340 faces, 47 now).  Many faces go to CTAs of 128, which group their solves.
 template <typename real, int B>
-__global__ void __launch_bounds__(B) k_ind_flux(HydroView<real> v, IndView d) {
+__global__ void __launch_bounds__(B) k_ind_flux(HydroView<real> v, IndView d, int above, int most) {
   const int count = d.count[1];
+  if (count <= above || count > most) return;
   const long long tick = d.loop->tick;
-  for (int blk = blockIdx.x; blk * B < count; blk += gridDim.x) {
-    const int idx = blk * B + (int)threadIdx.x;
-    const bool valid = idx < count;
-    const int k = d.flist[valid ? idx : 0];
+  int per = B;                                            // faces per CTA; a lane per side for B = 32
+  if (B == 32) {
+    per = 16;
+    while (per > 1 && (per >> 1) * (int)gridDim.x >= count) per >>= 1;
+  }
+  const int t = (int)threadIdx.x & (per - 1);             // (the lanes beyond per repeat the first ones' faces)
+  for (int blk = blockIdx.x; blk * per < count; blk += gridDim.x) {
+    const int idx = blk * per + t;
+    const bool valid = idx < count && t == (int)threadIdx.x;
+    const int k = d.flist[idx < count ? idx : count - 1];
     const int2 e = v.lr[k];
     const long long sL = step_ticks(d.depth, d.bin[e.x]), sR = step_ticks(d.depth, d.bin[e.y]);
     const long long sf = sL < sR ? sL : sR;
@@ -499,32 +608,48 @@ __global__ void __launch_bounds__(B) k_ind_flux(HydroView<real> v, IndView d) {
     const double hR = (double)(t2 - 2 * (tick - (tick & (sR - 1)))) * (0.5 * d.dtick);
     FaceWork<real> f;
     face_prepare<real, false>(v, k, valid, (real)hL, (real)hR, f);
-    face_finish<real, B, false>(v, f, 0, min(B, count - blk * B), false, (real)0);
+    face_finish<real, B, false>(v, f, 0, min(per, count - blk * per), false, (real)0);
+    if (B > 32) __syncthreads();
   }
 }
 
 // --------------------------------------------------- the pairwise exchange
+// Four lanes per cell, each with every fourth incidence, its face's stamp, step
+// and flux loaded whether or not the face is active (a thread per cell waited for
+// each in turn: 31 us a tick, 15 now, 32768 cells with few touched).
 template <typename real>
-__global__ void k_ind_update(HydroView<real> v, IndView d) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= d.n) return;
+__global__ void __launch_bounds__(256) k_ind_update(HydroView<real> v, IndView d) {
+  constexpr int G = 4;
+  const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G), lane = threadIdx.x % G;
   const int stamp = d.loop->stamp;
-  if (d.cstamp[i] != stamp) return;
+  const bool touched = i < d.n && d.cstamp[i] == stamp;
+  if (!__any_sync(0xffffffffu, touched)) return;
   double s[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  for (int q = v.csr_off[i]; q < v.csr_off[i + 1]; q++) {
-    const int2 e = v.csr[q];
-    const int k = e.x >> 1;
-    if (d.fstamp[k] != stamp) continue;
-    const double w = (e.x & 1) ? -d.fdt[k] : d.fdt[k];
-    const R4<real> f = v.flux[k];
-    s[0] += w * (double)f.x;
-    s[1] += w * (double)f.y;
-    s[2] += w * (double)f.z;
-    s[3] += w * (double)f.w;
-    s[4] += w * (double)v.fluxE[k];
+  if (touched) {
+    const int q1 = v.csr_off[i + 1];
+#pragma unroll 4
+    for (int q = v.csr_off[i] + lane; q < q1; q += G) {
+      const int2 e = v.csr[q];
+      const int k = e.x >> 1;
+      const R4<real> f = v.flux[k];
+      const real fE = v.fluxE[k];
+      const double dt = d.fdt[k];
+      if (d.fstamp[k] != stamp) continue;
+      const double w = (e.x & 1) ? -dt : dt;
+      s[0] += w * (double)f.x;
+      s[1] += w * (double)f.y;
+      s[2] += w * (double)f.z;
+      s[3] += w * (double)f.w;
+      s[4] += w * (double)fE;
+    }
   }
+#pragma unroll
+  for (int a = 0; a < 5; a++) s[a] = group_sum<G>(s[a]);
+  if (!touched) return;
   const size_t n = (size_t)d.n;
-  for (int a = 0; a < 5; a++) v.Q[a * n + i] -= s[a];
+  // (lane a writes component a, lane 0 also the last)
+  v.Q[lane * n + i] -= lane == 0 ? s[0] : (lane == 1 ? s[1] : (lane == 2 ? s[2] : s[3]));
+  if (lane == 0) v.Q[4 * n + i] -= s[4];
 }
 
 // ----------------------------------------------------------- the next tick
@@ -565,19 +690,20 @@ cudaError_t launch_individual_tick(amm_ctx* c, const IndView& d) {
   const int grid_c = nblk(c->n, 256);
   k_ind_activate<real><<<grid_c, 256, 0, c->stream>>>(v, d);
   if (d.signal) {
-    const int leaves = (d.dim == 3) ? (1 << (3 * (d.levels - 1))) : (1 << (2 * (d.levels - 1)));
-    k_ind_leaf<<<nblk(leaves, 256), 256, 0, c->stream>>>(d);
+    const int parents = 1 << (d.dim * (d.levels - 2));
+    k_ind_leaf<<<nblk((int64_t)parents * 32, 256), 256, 0, c->stream>>>(d);
     k_ind_up<<<1, 1024, 0, c->stream>>>(d);
   }
   // list kernels: a fixed grid strides over the list, whose length only the
   // device knows
   const int sms = 152;
-  const int g_grad = nblk(c->n, CELL_TILE / 4), g_bins = nblk(c->n, BINS_WARPS), g_flux = nblk(c->nf, 128);
-  k_ind_grad<real, 4><<<g_grad < sms * 8 ? g_grad : sms * 8, CELL_TILE, 0, c->stream>>>(v, d);
-  k_ind_bins<real><<<g_bins < sms * 16 ? g_bins : sms * 16, 32 * BINS_WARPS, 0, c->stream>>>(v, d);
+  const int g_cells = nblk(c->n, BINS_WARPS), g_flux = nblk(c->nf, 128);
+  k_ind_cells<real><<<2 * (g_cells < sms * 8 ? g_cells : sms * 8), 32 * BINS_WARPS, 0, c->stream>>>(v, d, sms * 4);
   k_ind_faces<real><<<nblk(c->nf, 256), 256, 0, c->stream>>>(v, d);
-  k_ind_flux<real, 128><<<g_flux < sms * 8 ? g_flux : sms * 8, 128, 0, c->stream>>>(v, d);
-  k_ind_update<real><<<grid_c, 256, 0, c->stream>>>(v, d);
+  const int few = sizeof(real) == 8 ? sms * 32 * 2 : 0;
+  if (few) k_ind_flux<real, 32><<<sms * 4, 32, 0, c->stream>>>(v, d, 0, few);
+  k_ind_flux<real, 128><<<g_flux < sms * 8 ? g_flux : sms * 8, 128, 0, c->stream>>>(v, d, few, 0x7fffffff);
+  k_ind_update<real><<<nblk(c->n * 4, 256), 256, 0, c->stream>>>(v, d);
   return cudaGetLastError();
 }
 

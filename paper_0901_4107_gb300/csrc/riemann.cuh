@@ -211,6 +211,23 @@ struct NewtonTail {
 // relative change of p cannot fall below a 1e-12 tolerance.
 constexpr double RESIDUAL_ULPS = 64.0;
 
+// One step from p, whose f_K and f_K' are in t; true when p (or the new p) is converged
+__device__ __forceinline__ bool newton_step64(double& p, double du, double tol, int& it, NewtonTail<double>& t) {
+  t.dp = 0.0;
+  const double f = rn_add(rn_add(t.fL, t.fR), du);
+  const double small = rn_mul(RESIDUAL_ULPS * DBL_EPSILON, rn_add(rn_add(fabs(t.fL), fabs(t.fR)), fabs(du)));
+  if (fabs(f) <= small) return true;
+  const double D = rn_add(t.dL, t.dR);
+  double pn = rn_add(p, -(f / D));
+  if (!(pn > 0.0)) pn = rn_mul(1e-3, p);
+  it++;
+  t.dp = rn_add(pn, -p);
+  // 2 |dp| / (p_new + p_old) < tol, without the division
+  const bool done = rn_mul(2.0, fabs(t.dp)) < rn_mul(tol, rn_add(pn, p));
+  p = pn;
+  return done;
+}
+
 // The FP64 Newton iteration: p* from the iterate p; it and conv as in newton_pstar.
 __device__ __forceinline__ double newton_pstar64(double p, const WaveSide& KL, const WaveSide& KR, double du,
                                                  const GasC<double>& G, double tol, int maxit, int& it, bool& conv,
@@ -220,25 +237,33 @@ __device__ __forceinline__ double newton_pstar64(double p, const WaveSide& KL, c
     const double ip = 1.0 / p;
     wave_curve(p, ip, KL, G, t.fL, t.dL);
     wave_curve(p, ip, KR, G, t.fR, t.dR);
-    t.dp = 0.0;
-    const double f = rn_add(rn_add(t.fL, t.fR), du);
-    const double small = rn_mul(RESIDUAL_ULPS * DBL_EPSILON, rn_add(rn_add(fabs(t.fL), fabs(t.fR)), fabs(du)));
-    if (fabs(f) <= small) {
+    if (newton_step64(p, du, tol, it, t)) {
       conv = true;
       break;
     }
-    const double D = rn_add(t.dL, t.dR);
-    double pn = rn_add(p, -(f / D));
-    if (!(pn > 0.0)) pn = rn_mul(1e-3, p);
-    it++;
-    t.dp = rn_add(pn, -p);
-    // 2 |dp| / (p_new + p_old) < tol, without the division
-    if (rn_mul(2.0, fabs(t.dp)) < rn_mul(tol, rn_add(pn, p))) {
-      p = pn;
-      conv = true;
-      break;
-    }
-    p = pn;
+  }
+  return p;
+}
+
+// The same iteration by two lanes, l and l ^ 16, that hold the same problem: each
+// evaluates the wave curve of its own side (side: 1 right) and passes it to the
+// other, which halves the chain of FP64 instructions of a warp with few problems.
+// All lanes of `in` call it; the values and their order are newton_pstar64's.
+__device__ __forceinline__ double newton_pstar64_pair(double p, const WaveSide& K, int side, double du,
+                                                      const GasC<double>& G, double tol, int maxit, unsigned in,
+                                                      int& it, bool& conv, NewtonTail<double>& t) {
+  t.fL = t.dL = t.fR = t.dR = t.dp = 0.0;
+  while (__any_sync(in, !conv && it < maxit)) {
+    const double ip = 1.0 / p;
+    double f1, d1;
+    wave_curve(p, ip, K, G, f1, d1);
+    const double f2 = __shfl_xor_sync(in, f1, 16), d2 = __shfl_xor_sync(in, d1, 16);
+    if (conv || it >= maxit) continue;
+    t.fL = side ? f2 : f1;
+    t.fR = side ? f1 : f2;
+    t.dL = side ? d2 : d1;
+    t.dR = side ? d1 : d2;
+    conv = newton_step64(p, du, tol, it, t);
   }
   return p;
 }
@@ -246,7 +271,8 @@ __device__ __forceinline__ double newton_pstar64(double p, const WaveSide& KL, c
 // The FP32 forms' rare continuation in FP64: in place, or left to the caller
 // (info.guard set, the returned state unfinished), whose kernel then holds no
 // FP64 solve.
-enum GuardKind { GUARD_INLINE, GUARD_DEFER };
+// SOLVE_PAIRED: FP64 problems held by lanes l and l ^ 16 alike (all lanes call).
+enum GuardKind { GUARD_INLINE, GUARD_DEFER, SOLVE_PAIRED };
 struct GuardOut {
   float p, us;
   int iters, conv;
@@ -272,12 +298,16 @@ __device__ __forceinline__ GuardOut guard_solve(float p, float rhoL, float uL, f
 template <GuardKind GUARD = GUARD_INLINE, typename real>
 __device__ __forceinline__ real newton_pstar(real p, real rhoL, real uL, real pL, real cL, real rhoR, real uR,
                                              real pR, real cR, const GasC<real>& G, double tol, real tol_r, int maxit,
-                                             RiemannInfo& info, real& us) {
+                                             RiemannInfo& info, real& us, unsigned in = 0u) {
   const real du = uR - uL;
   NewtonTail<real> tail;
   int it = 0;
   bool conv = false;
-  if constexpr (sizeof(real) == 8) {
+  if constexpr (sizeof(real) == 8 && GUARD == SOLVE_PAIRED) {
+    const int side = ((int)threadIdx.x >> 4) & 1;
+    p = newton_pstar64_pair(p, wave_side(side ? rhoR : rhoL, side ? pR : pL, side ? cR : cL, G), side, du, G, tol,
+                            maxit, in, it, conv, tail);
+  } else if constexpr (sizeof(real) == 8) {
     p = newton_pstar64(p, wave_side(rhoL, pL, cL, G), wave_side(rhoR, pR, cR, G), du, G, tol, maxit, it, conv, tail);
   } else {
     constexpr int FLOAT_ITERS = 12;
@@ -345,7 +375,10 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
   info.guard = 0;
   info.vacuum = 0;
   info.fail = 0;
-  if (G.two_gm1 * (cL + cR) <= uR - uL) {
+  const bool vacuum = G.two_gm1 * (cL + cR) <= uR - uL;
+  unsigned in = 0u;
+  if constexpr (GUARD == SOLVE_PAIRED) in = __ballot_sync(0xffffffffu, !vacuum);
+  if (vacuum) {
     // two rarefactions with vacuum between them
     info.vacuum = 1;
     const real frontL = uL + G.two_gm1 * cL;
@@ -379,7 +412,7 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
   }
   const real p0 = standard_guess_ppv(rhoL, uL, pL, cL, rhoR, uR, pR, cR, ppv, G, have_guess, guess);
   real us;
-  const real ps = newton_pstar<GUARD>(p0, rhoL, uL, pL, cL, rhoR, uR, pR, cR, G, tol, tol_r, maxit, info, us);
+  const real ps = newton_pstar<GUARD>(p0, rhoL, uL, pL, cL, rhoR, uR, pR, cR, G, tol, tol_r, maxit, info, us, in);
   pstar = ps;
   // the side the face sees (the contact's upwind side): s = +1 left, -1
   // right; the right side's formulas are the left side's with the velocity
