@@ -74,12 +74,17 @@ void free_ctx(amm_ctx* c) {
 //   262 k         78 / 55        64 / 49        63 / 53        82 / 80
 //   1.4 M        331 / 217      271 / 192      281 / 236      398 / 369
 //   FP64, cells
-//     8.2 k (2D)  67 / 18        51 / 16        44 / 10        63 / 12
-//    91 k        344 / 68       328 / 61       414 / 76       608 / 78
+//     8.2 k (2D)  47 / 19        38 / 14        35 / 10        44 / 12
+//    13.8 k       86 / 29        60 / 20        67 / 21        76 / 18
+//    33 k         86 / 29       102 / 28       118 / 35       150 / 41
+//    91 k        208 / 68       217 / 59       264 / 76       374 / 92
 void default_lanes(amm_ctx* c) {
-  const int64_t few = 40000;   // threads below which more lanes still pay in the update
+  const int64_t few = 40000;   // threads below which more lanes still pay (two warps for each of the chip's 608 FP64 pipes)
   c->update_lanes = 8 * c->n <= few ? 8 : (4 * c->n <= few ? 4 : 2);
-  c->grad_lanes = c->n <= (c->is_fp64() ? 30000 : 300000) ? 4 : 2;
+  if (c->is_fp64())
+    c->grad_lanes = 4 * c->n <= few ? 4 : (2 * c->n <= few ? 2 : 1);
+  else
+    c->grad_lanes = c->n <= 300000 ? 4 : 2;
 }
 
 template <typename F64, typename F32>

@@ -147,9 +147,8 @@ struct Extrema<double> {
 };
 
 // x[a] = 1 / x[a] for values that the G lanes of a group all hold.  FP64: lane l
-// divides for a = l, l + G, ..., since a division is some ten instructions of the
-// narrow FP64 pipe for every lane's copy of it (15 per cell were 45% of the
-// gradients' FP64 work; 91 k cells, two lanes: 247 -> 235 us).
+// divides for a = l, l + G, ..., rather than every lane for all 15 (91 k cells, two
+// lanes: gradients 247 -> 235 us, 216 with the divisions in fixed point).
 template <int G, int N>
 __device__ __forceinline__ void group_reciprocals(float* x, int) {
 #pragma unroll
@@ -163,7 +162,9 @@ __device__ __forceinline__ void group_reciprocals(double* x, int lane) {
 #pragma unroll
     for (int l = 1; l < G; l++)
       if (b + l < N && lane == l) mine = x[b + l];
-    mine = 1.0 / mine;
+    const bool zero = __double_as_longlong(mine) == 0ll;   // an extremal cell's difference
+    mine = recip64(zero ? 1.0 : mine);
+    mine = zero ? INFINITY : mine;
 #pragma unroll
     for (int l = 0; l < G; l++)
       if (b + l < N) x[b + l] = G > 1 ? __shfl_sync(0xffffffffu, mine, l, G) : mine;
@@ -359,7 +360,7 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
       // (explicitly rounded: the persistent step kernel must round alike)
       const real rho = phi_i[0], vx = phi_i[1], vy = phi_i[2], vz = phi_i[3], P = phi_i[4];
       const real divv = rn_add(rn_add(g[1][0], g[2][1]), g[3][2]);
-      const real ir = (real)1 / rho;
+      const real ir = xrecip(rho);
       const real mh = -hdt;
       R4<real> a, b;
       a.x = rn_fma(mh, rn_fma(rho, divv, rn_dot3(vx, vy, vz, g[0][0], g[0][1], g[0][2])), rho);
@@ -388,7 +389,7 @@ __device__ __forceinline__ real courant_time(const HydroView<real>& v, int i, co
   real w3[3];
   mesh_velocity(v, i, Wi, w3);
   // (explicitly rounded: the persistent step kernel must round alike)
-  const real cs = xsqrt(rn_mul(v.gas.g, Pi) / Wi.x);
+  const real cs = xsqrt(xdiv(rn_mul(v.gas.g, Pi), Wi.x));
   const real Ri = v.crad[i];
   if (v.regularize) {
     // Sec. 4.1, eq. (EqnShapeCorrVel): towards the centre of mass at the
@@ -409,7 +410,7 @@ __device__ __forceinline__ real courant_time(const HydroView<real>& v, int i, co
     v.wcorr[i] = wc;
   }
   const real dx = Wi.y - w3[0], dy = Wi.z - w3[1], dz = Wi.w - w3[2];
-  return Ri / rn_add(cs, xsqrt(rn_dot3(dx, dy, dz, dx, dy, dz)));
+  return xdiv(Ri, rn_add(cs, xsqrt(rn_dot3(dx, dy, dz, dx, dy, dz))));
 }
 
 // The CTA's minimum of tc folded into box b's Courant minimum: one integer
@@ -539,7 +540,7 @@ __device__ __forceinline__ void side_extrapolate(const GasC<real>& G, const Cell
   const real ux = Wi.y - w[0], uy = Wi.z - w[1], uz = Wi.w - w[2];
   Wp[0] = rho; Wp[1] = ux; Wp[2] = uy; Wp[3] = uz; Wp[4] = P;
   const real divv = g1.x + g2.y + g3.z;
-  const real ir = (real)1 / rho;
+  const real ir = xrecip(rho);
   Wpp[0] = rho + (g0.x * fx + g0.y * fy + g0.z * fz) - hdt * (ux * g0.x + uy * g0.y + uz * g0.z + rho * divv);
   Wpp[1] = ux + (g1.x * fx + g1.y * fy + g1.z * fz) - hdt * (ux * g1.x + uy * g1.y + uz * g1.z + g0.w * ir);
   Wpp[2] = uy + (g2.x * fx + g2.y * fy + g2.z * fz) - hdt * (ux * g2.x + uy * g2.y + uz * g2.z + g1.w * ir);
@@ -608,7 +609,7 @@ __device__ __forceinline__ void face_prepare_rec(const HydroView<real>& v, int k
       wl[0] = a.x; wl[1] = a.y; wl[2] = a.z;
       wr[0] = b.x; wr[1] = b.y; wr[2] = b.z;
     }
-    const real rot = ((wl[0] - wr[0]) * c[0] + (wl[1] - wr[1]) * c[1] + (wl[2] - wr[2]) * c[2]) / sep;
+    const real rot = xdiv((wl[0] - wr[0]) * c[0] + (wl[1] - wr[1]) * c[1] + (wl[2] - wr[2]) * c[2], sep);
 #pragma unroll
     for (int d = 0; d < 3; d++) w[d] = (real)0.5 * (wl[d] + wr[d]) + rot * n[d];
   }
@@ -617,7 +618,7 @@ __device__ __forceinline__ void face_prepare_rec(const HydroView<real>& v, int k
   side_extrapolate<real, ENT>(v.gas, recL, (real)0.5, n, sep, c, w, hdtL, WpL, f.WppL, f.AL);
   side_extrapolate<real, ENT>(v.gas, recR, (real)-0.5, n, sep, c, w, hdtR, WpR, f.WppR, f.AR);
   f.fallback = 0;
-  if (!(f.WppL[0] > (real)0) || !(f.WppL[4] > (real)0) || !(f.WppR[0] > (real)0) || !(f.WppR[4] > (real)0)) {
+  if (!positive(f.WppL[0]) || !positive(f.WppL[4]) || !positive(f.WppR[0]) || !positive(f.WppR[4])) {
 #pragma unroll
     for (int a = 0; a < 5; a++) {
       f.WppL[a] = WpL[a];
@@ -708,7 +709,7 @@ __device__ __forceinline__ void face_prepare_pred(const HydroView<real>& v, int 
   side_from_pred<real, ENT>(pL, AL_raw, (real)0.5, n, sep, c, f.WppL, f.AL);
   side_from_pred<real, ENT>(pR, AR_raw, (real)-0.5, n, sep, c, f.WppR, f.AR);
   f.fallback = 0;
-  if (!(f.WppL[0] > (real)0) || !(f.WppL[4] > (real)0) || !(f.WppR[0] > (real)0) || !(f.WppR[4] > (real)0)) {
+  if (!positive(f.WppL[0]) || !positive(f.WppL[4]) || !positive(f.WppR[0]) || !positive(f.WppR[4])) {
     const R4<real> WL = v.cw[2 * (size_t)lr.x], PL = v.cw[2 * (size_t)lr.x + 1];
     const R4<real> WR = v.cw[2 * (size_t)lr.y], PR = v.cw[2 * (size_t)lr.y + 1];
     f.WppL[0] = WL.x; f.WppL[1] = WL.y; f.WppL[2] = WL.z; f.WppL[3] = WL.w; f.WppL[4] = PL.x;
@@ -842,9 +843,9 @@ __device__ __forceinline__ void face_finish_core(const HydroView<real>& v, const
     fS = A * (rhoF * uF) * (uF > (real)0 ? f.AL : f.AR);
     real mach = (real)1;
     if (!info.vacuum) {
-      if (ps > f.WppL[4]) mach = xsqrt((real)1 + G.shock_a * (ps / f.WppL[4] - (real)1));
+      if (ps > f.WppL[4]) mach = xsqrt((real)1 + G.shock_a * (xdiv(ps, f.WppL[4]) - (real)1));
       if (ps > f.WppR[4]) {
-        const real mr = xsqrt((real)1 + G.shock_a * (ps / f.WppR[4] - (real)1));
+        const real mr = xsqrt((real)1 + G.shock_a * (xdiv(ps, f.WppR[4]) - (real)1));
         mach = mr > mach ? mr : mach;
       }
     }
@@ -895,8 +896,9 @@ __device__ __forceinline__ void stats_add(DeviceStats* S, unsigned* box_status, 
 // and as many iterations as its worst face (11.6 of 32 lanes on).  So the states
 // go through shared memory, ordered by the kind of solve (judged in FP32, on
 // the idle FP32 pipe); every face's arithmetic is the same wherever it runs.
-// 91 k cells, one step's fluxes: 2754 us in face order with pow; 2412 us with
-// pow64 and fewer divisions; 1540 us regrouped (21.7 lanes on).
+// 91 k cells, one step's fluxes: 2412 us in face order, 1540 regrouped (21.7 lanes
+// on); 445 with the divisions, roots and powers in fixed point on the integer pipe
+// and the comparisons in integers (1130 -> 274 FP64 instructions a warp).
 template <int B>
 __device__ __forceinline__ void solve_grouped(const HydroView<double>& v, const FaceWork<double>& f,
                                               RiemannOut<double>& r) {
@@ -905,7 +907,7 @@ __device__ __forceinline__ void solve_grouped(const HydroView<double>& v, const 
   __shared__ short order[B];
   const int t = (int)threadIdx.x;
   const double rL = f.WppL[0], pL = f.WppL[4], rR = f.WppR[0], pR = f.WppR[4];
-  const double cL = sqrt(rn_mul(v.gas.g, pL) / rL), cR = sqrt(rn_mul(v.gas.g, pR) / rR);
+  const double cL = sqrt64(div64(rn_mul(v.gas.g, pL), rL)), cR = sqrt64(div64(rn_mul(v.gas.g, pR), rR));
   const double ppv = linearised_pstar(rL, f.uL, pL, cL, rR, f.uR, pR, cR);
   const int kind = solve_kind(rL, f.uL, pL, cL, rR, f.uR, pR, cR, ppv, GasC<float>(v.gamma));
   if (t < SOLVE_KINDS) total[t] = 0;
@@ -953,13 +955,13 @@ __device__ __forceinline__ void face_finish(const HydroView<real>& v, const Face
                                             bool have_guess, real guess) {
   const bool valid = f.valid;
   FaceOut o;
-  if constexpr (sizeof(real) == 8 && B > 32) {
+  if constexpr (sizeof(real) == 8 && B > 64) {
     RiemannOut<double> r;
     solve_grouped<B>(v, f, r);
     face_finish_core<real, ENT>(v, f, false, guess, o, false, nullptr, &r);
   } else {
-    // (one warp of FP64 faces: the caller gives lanes l and l ^ 16 the same face)
-    constexpr GuardKind SOLVE = sizeof(real) == 8 ? SOLVE_PAIRED : GUARD_INLINE;
+    // (FP64 faces of a one-warp CTA: the caller gives lanes l and l ^ 16 the same face)
+    constexpr GuardKind SOLVE = sizeof(real) == 8 && B == 32 ? SOLVE_PAIRED : GUARD_INLINE;
     face_finish_core<real, ENT, SOLVE>(v, f, have_guess, guess, o);
   }
   if (sizeof(real) == 4 && v.fixed_acc) {
@@ -1036,9 +1038,8 @@ __device__ __forceinline__ void flux_item(const HydroView<real>& v, int wi) {
   face_finish<real, B, ENT>(v, f, t.box, min(B, t.end - first), false, (real)0);
 }
 
-// (FP64: 16 warps per SM, 128 registers; with one CTA of 256 per SM and no
-// spills the barriers of the grouped solve leave the FP64 pipe idle: 1725 us
-// for 1540)
+// (FP64: 16 warps per SM, 128 registers; 24 warps at 80 registers: 453 us for 445
+// at 715 k faces, whose FP64 instructions alone take 366)
 template <typename real, int B, bool ENT>
 __global__ void __launch_bounds__(B, sizeof(real) == 4 ? 4 * FACE_TILE / B : 2 * FACE_TILE / B) k_flux(HydroView<real> v) {
   flux_item<real, B, ENT>(v, blockIdx.x);
@@ -1706,11 +1707,11 @@ cudaError_t launch_flux(amm_ctx* c, double cfl) {
     return launch_flux_chunks(c, v, false, FluxDefer());
   } else {
     const bool ent = c->opt.entropy != 0;
-    // Few faces: CTAs of 64 spread them over all SMs, whose FP64 pipes are what
-    // bounds the solve; with many the larger CTAs group the faces' solves
-    // better.  (us for faces: 25 k 74 / 86 with 256, 49 k 112 / 141, 98 k 206 /
-    // 239, 715 k 2057 / 1540.)
-    const bool few = c->nf <= 152 * 768;
+    // Few faces: CTAs of 64 spread them over all SMs' FP64 pipes, in the faces' own
+    // order; many: CTAs of 256, which group the solves by kind.  (us for faces, 64
+    // / 256: 25 k 27 / 35, 98 k 55 / 69 in 2D and 98 / 102 in 3D, 230 k 182 / 178,
+    // 715 k 471 / 445.)
+    const bool few = c->nf <= 152 * 1024;
     if (few && ent)
       k_flux<real, 64, true><<<c->n_ftiles * 4, 64, 0, c->stream>>>(v);
     else if (few)

@@ -26,17 +26,36 @@
 #include <float.h>
 
 #include "amm_internal.cuh"
-#include "pow64.cuh"
+#include "fixed64.cuh"
 
 namespace amm {
 
 
 __device__ __forceinline__ double xpow(double a, double b) { return pow64(a, b); }
 __device__ __forceinline__ float xpow(float a, float b) { return __powf(a, b); }
-__device__ __forceinline__ double xsqrt(double a) { return sqrt(a); }
+__device__ __forceinline__ double xsqrt(double a) { return sqrt64(a); }
 __device__ __forceinline__ float xsqrt(float a) { return sqrtf(a); }
-__device__ __forceinline__ double xrsqrt(double a) { return rsqrt(a); }
+__device__ __forceinline__ double xrsqrt(double a) { return rsqrt64(a); }
 __device__ __forceinline__ float xrsqrt(float a) { return rsqrtf(a); }
+__device__ __forceinline__ double xdiv(double a, double b) { return div64(a, b); }
+__device__ __forceinline__ float xdiv(float a, float b) { return a / b; }
+__device__ __forceinline__ double xrecip(double a) { return recip64(a); }
+__device__ __forceinline__ float xrecip(float a) { return 1.0f / a; }
+
+// Comparisons; FP64 ones in integers (an FP64 comparison takes the FP64 pipe): x > 0;
+// a < b and a <= b for a >= 0 (or its magnitude) and b >= 0, false where b is a NaN.
+__device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool positive(double x) {
+  return (u64)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool mag_less(double a, double b) {
+  const i64 i = __double_as_longlong(a) & 0x7fffffffffffffffll, j = __double_as_longlong(b);
+  return i < j && j <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool mag_leq(double a, double b) {
+  const i64 i = __double_as_longlong(a) & 0x7fffffffffffffffll, j = __double_as_longlong(b);
+  return i <= j && j <= 0x7ff0000000000000ll;
+}
 
 // Explicitly rounded products, sums and fused multiply-adds: the compiler
 // neither fuses nor splits them, so a formula written with them rounds the
@@ -80,30 +99,29 @@ __device__ __forceinline__ void wave_curve(float p, float rhoK, float pK, float 
   }
 }
 
-// FP64: f_K(p) and f_K'(p).  Divisions and square roots cost about
-// ten FP64 instructions each, so the shock takes one reciprocal square root,
+// FP64: f_K(p) and f_K'(p).  The shock takes one reciprocal square root,
 // w = (rho (p + B))^(-1/2): q = sqrt(2/(gamma+1)) w and 1/(p + B) = rho w^2; the
 // rarefaction f' = (p/p_K)^z c_K / (gamma p) (rho_K c_K = gamma p_K / c_K), with
 // 1/p given (both sides need it) and 1/p_K formed once per solve.
 // (explicitly rounded: the persistent step kernel must round alike)
 struct WaveSide {
-  double rho, p, c, ip, B, two_c;   // state, 1/p, B, 2c/(gamma-1)
+  double rho, p, ip, B, two_c, c_g;   // state, 1/p, B, 2c/(gamma-1), c/gamma
 };
 __device__ __forceinline__ WaveSide wave_side(double rho, double p, double c, const GasC<double>& G) {
   WaveSide s;
   s.rho = rho;
   s.p = p;
-  s.c = c;
-  s.ip = 1.0 / p;
+  s.ip = recip64(p);
   s.B = rn_mul(G.gm1_gp1, p);
   s.two_c = rn_mul(G.two_gm1, c);
+  s.c_g = rn_mul(c, G.inv_g);
   return s;
 }
 __device__ __forceinline__ void wave_curve(double p, double ip, const WaveSide& K, const GasC<double>& G, double& f,
                                            double& df) {
   const double d = rn_add(p, -K.p);
-  if (d > 0.0) {
-    const double w = rsqrt(rn_mul(K.rho, rn_add(p, K.B)));
+  if (positive(d)) {
+    const double w = rsqrt64(rn_mul(K.rho, rn_add(p, K.B)));
     const double q = rn_mul(G.sqrt_two_gp1, w);
     const double h = rn_mul(rn_mul(w, w), K.rho);
     const double dh = rn_mul(d, h);
@@ -113,7 +131,7 @@ __device__ __forceinline__ void wave_curve(double p, double ip, const WaveSide& 
     const double pr = rn_mul(p, K.ip);
     const double prz = pow64(pr, G.z);
     f = rn_mul(K.two_c, rn_add(prz, -1.0));
-    df = rn_mul(rn_mul(prz, rn_mul(K.c, G.inv_g)), ip);
+    df = rn_mul(rn_mul(prz, K.c_g), ip);
   }
 }
 
@@ -131,10 +149,10 @@ __device__ __forceinline__ real two_shock_pstar(real rhoL, real uL, real pL, rea
                                                 const GasC<real>& G) {
   if constexpr (sizeof(real) == 8) {
     // one reciprocal square root per side (in units of sqrt(2/(gamma+1)))
-    const double gL = rsqrt(rn_mul(rhoL, rn_fma(G.gm1_gp1, pL, ppv)));
-    const double gR = rsqrt(rn_mul(rhoR, rn_fma(G.gm1_gp1, pR, ppv)));
+    const double gL = rsqrt64(rn_mul(rhoL, rn_fma(G.gm1_gp1, pL, ppv)));
+    const double gR = rsqrt64(rn_mul(rhoR, rn_fma(G.gm1_gp1, pR, ppv)));
     const double du = rn_mul(rn_add(uR, -uL), G.isqrt_two_gp1);
-    return rn_add(rn_fma(gL, pL, rn_mul(gR, pR)), -du) / rn_add(gL, gR);
+    return div64(rn_add(rn_fma(gL, pL, rn_mul(gR, pR)), -du), rn_add(gL, gR));
   } else {
     const real gL = xsqrt((G.two_gp1 / rhoL) / (ppv + G.gm1_gp1 * pL));
     const real gR = xsqrt((G.two_gp1 / rhoR) / (ppv + G.gm1_gp1 * pR));
@@ -155,7 +173,8 @@ __device__ __forceinline__ real standard_guess_ppv(real rhoL, real uL, real pL, 
                                                    real cR, real ppv, const GasC<real>& G, bool have = false,
                                                    real proposal = (real)0) {
   const real du = uR - uL;
-  const real pmin = pL < pR ? pL : pR, pmax = pL > pR ? pL : pR;
+  const bool lowL = sizeof(real) == 8 ? mag_less(pL, pR) : pL < pR;
+  const real pmin = lowL ? pL : pR, pmax = lowL ? pR : pL;
   real p0;
   if constexpr (sizeof(real) == 4) {
     // FP32: every estimate, selected (a warp's faces take all three, so
@@ -166,18 +185,19 @@ __device__ __forceinline__ real standard_guess_ppv(real rhoL, real uL, real pL, 
     const real ptr = xpow(num / den, G.inv_z);
     const real pts = have ? proposal : two_shock_pstar(rhoL, uL, pL, rhoR, uR, pR, ppv, G);
     p0 = pv ? ppv : (ppv < pmin ? ptr : pts);
-  } else if (pmax <= (real)2 * pmin && ppv >= pmin && ppv <= pmax) {
+  } else if (mag_leq(pmax, rn_mul(2.0, pmin)) && mag_leq(pmin, ppv) && mag_leq(ppv, pmax)) {
     p0 = ppv;
-  } else if (ppv < pmin) {
+  } else if (mag_less(ppv, pmin)) {
     const real num = rn_add(rn_add(cL, cR), -rn_mul(rn_mul((real)0.5, G.gm1), du));
     const real den = rn_fma(cL, xpow(pL, -G.z), rn_mul(cR, xpow(pR, -G.z)));
-    p0 = xpow(num / den, G.inv_z);
+    p0 = xpow(div64(num, den), G.inv_z);
   } else if (have) {
     p0 = proposal;
   } else {
     p0 = two_shock_pstar(rhoL, uL, pL, rhoR, uR, pR, ppv, G);
   }
   const real pfloor = (real)1e-10 * (real)0.5 * (pL + pR);
+  if constexpr (sizeof(real) == 8) return positive(p0) && mag_less(pfloor, p0) ? p0 : pfloor;
   return (p0 > pfloor) ? p0 : pfloor;
 }
 
@@ -216,14 +236,14 @@ __device__ __forceinline__ bool newton_step64(double& p, double du, double tol, 
   t.dp = 0.0;
   const double f = rn_add(rn_add(t.fL, t.fR), du);
   const double small = rn_mul(RESIDUAL_ULPS * DBL_EPSILON, rn_add(rn_add(fabs(t.fL), fabs(t.fR)), fabs(du)));
-  if (fabs(f) <= small) return true;
+  if (mag_leq(f, small)) return true;
   const double D = rn_add(t.dL, t.dR);
-  double pn = rn_add(p, -(f / D));
-  if (!(pn > 0.0)) pn = rn_mul(1e-3, p);
+  double pn = rn_add(p, -div64(f, D));
+  if (!positive(pn)) pn = rn_mul(1e-3, p);
   it++;
   t.dp = rn_add(pn, -p);
   // 2 |dp| / (p_new + p_old) < tol, without the division
-  const bool done = rn_mul(2.0, fabs(t.dp)) < rn_mul(tol, rn_add(pn, p));
+  const bool done = mag_less(t.dp, rn_mul(0.5 * tol, rn_add(pn, p)));
   p = pn;
   return done;
 }
@@ -234,7 +254,7 @@ __device__ __forceinline__ double newton_pstar64(double p, const WaveSide& KL, c
                                                  NewtonTail<double>& t) {
   t.fL = t.dL = t.fR = t.dR = t.dp = 0.0;
   while (it < maxit) {
-    const double ip = 1.0 / p;
+    const double ip = recip64(p);
     wave_curve(p, ip, KL, G, t.fL, t.dL);
     wave_curve(p, ip, KR, G, t.fR, t.dR);
     if (newton_step64(p, du, tol, it, t)) {
@@ -254,7 +274,7 @@ __device__ __forceinline__ double newton_pstar64_pair(double p, const WaveSide& 
                                                       int& it, bool& conv, NewtonTail<double>& t) {
   t.fL = t.dL = t.fR = t.dR = t.dp = 0.0;
   while (__any_sync(in, !conv && it < maxit)) {
-    const double ip = 1.0 / p;
+    const double ip = recip64(p);
     double f1, d1;
     wave_curve(p, ip, K, G, f1, d1);
     const double f2 = __shfl_xor_sync(in, f1, 16), d2 = __shfl_xor_sync(in, d1, 16);
@@ -283,8 +303,8 @@ __device__ __forceinline__ GuardOut guard_solve(float p, float rhoL, float uL, f
   const double rL = rhoL, pLd = pL, rR = rhoR, pRd = pR;
   NewtonTail<double> t;
   bool done = false;
-  const double ps = newton_pstar64((double)p, wave_side(rL, pLd, sqrt(G.g * pLd / rL), G),
-                                   wave_side(rR, pRd, sqrt(G.g * pRd / rR), G), (double)uR - (double)uL, G, tol, maxit,
+  const double ps = newton_pstar64((double)p, wave_side(rL, pLd, sqrt64(div64(G.g * pLd, rL)), G),
+                                   wave_side(rR, pRd, sqrt64(div64(G.g * pRd, rR)), G), (double)uR - (double)uL, G, tol, maxit,
                                    it, done, t);
   GuardOut o;
   o.p = (float)ps;
@@ -388,7 +408,7 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
         rhoF = rhoL; uF = uL; pF = pL;
       } else {
         const real c = G.two_gp1 * cL + G.gm1_gp1 * uL;
-        const real r = c / cL;
+        const real r = xdiv(c, cL);
         uF = c;
         rhoF = rhoL * xpow(r, G.fan_rho);
         pF = pL * xpow(r, G.fan_p);
@@ -400,7 +420,7 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
         rhoF = rhoR; uF = uR; pF = pR;
       } else {
         const real c = G.two_gp1 * cR - G.gm1_gp1 * uR;
-        const real r = c / cR;
+        const real r = xdiv(c, cR);
         uF = -c;
         rhoF = rhoR * xpow(r, G.fan_rho);
         pF = pR * xpow(r, G.fan_p);
@@ -420,7 +440,7 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
   const int side = ((real)0 <= us) ? 0 : 1;
   const real s = side ? (real)-1 : (real)1;
   const real rhoK = side ? rhoR : rhoL, uK = side ? uR : uL, pK = side ? pR : pL, cK = side ? cR : cL;
-  const real r = ps / pK;
+  const real r = xdiv(ps, pK);
   if constexpr (sizeof(real) == 4) {
     // FP32: the shock and rarefaction cases evaluated and selected; only the
     // sonic rarefaction (the face inside the fan, rare) branches
@@ -436,17 +456,17 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
     pF = orig ? pK : ps;
     if (fan) {
       const real c = G.two_gp1 * cK + s * G.gm1_gp1 * uK;
-      const real q = c / cK;
+      const real q = xdiv(c, cK);
       uF = s * c;
       rhoF = rhoK * xpow(q, G.fan_rho);
       pF = pK * xpow(q, G.fan_p);
     }
-  } else if (ps > pK) {
+  } else if (mag_less(pK, ps)) {
     const real SK = uK - s * cK * xsqrt(G.shock_a * r + G.shock_b);
     if ((real)0 <= s * SK) {
       rhoF = rhoK; uF = uK; pF = pK;
     } else {
-      rhoF = rhoK * (r + G.gm1_gp1) / (G.gm1_gp1 * r + (real)1); uF = us; pF = ps;
+      rhoF = xdiv(rhoK * (r + G.gm1_gp1), G.gm1_gp1 * r + (real)1); uF = us; pF = ps;
     }
   } else {
     if ((real)0 <= s * (uK - s * cK)) {
@@ -456,10 +476,10 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
       const real rz = xpow(r, G.z);
       const real tail = us - s * cK * rz;
       if ((real)0 > s * tail) {
-        rhoF = rhoK * (r / rn_mul(rz, rz)); uF = us; pF = ps;
+        rhoF = rhoK * xdiv(r, rn_mul(rz, rz)); uF = us; pF = ps;
       } else {
         const real c = G.two_gp1 * cK + s * G.gm1_gp1 * uK;
-        const real q = c / cK;
+        const real q = xdiv(c, cK);
         uF = s * c;
         rhoF = rhoK * xpow(q, G.fan_rho);
         pF = pK * xpow(q, G.fan_p);
@@ -469,6 +489,16 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
   return side;
 }
 
+// x truncated to FP32 (zero or infinite beyond its range), in integers: a conversion
+// takes the FP64 pipe
+__device__ __forceinline__ float coarse_float(double x) {
+  const unsigned h = (unsigned)__double2hiint(x);
+  const int e = (int)exponent_bits((int)h) - 896;
+  const unsigned m = (h & 0xfffffu) << 3 | (unsigned)__double2loint(x) >> 29;
+  const unsigned b = e <= 0 ? 0u : (e >= 255 ? 0x7f800000u : (unsigned)e << 23 | m);
+  return __uint_as_float((h & 0x80000000u) | b);
+}
+
 // Which way the FP64 solve of these states will go, judged in FP32: 0 for two
 // rarefactions (the standard guess is then the root itself), else one plus the
 // waves' kinds and whether the guess is far off (more iterations).  Only the
@@ -476,9 +506,10 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
 constexpr int SOLVE_KINDS = 8;
 __device__ __forceinline__ int solve_kind(double rL, double uL, double pL, double cL, double rR, double uR, double pR,
                                           double cR, double ppv, const GasC<float>& G) {
-  const float rl = (float)rL, pl = (float)pL, cl = (float)cL, rr = (float)rR, pr = (float)pR, cr = (float)cR;
-  const float du = (float)(uR - uL);
-  const float p0 = standard_guess_ppv<float>(rl, 0.0f, pl, cl, rr, du, pr, cr, (float)ppv, G);
+  const float rl = coarse_float(rL), pl = coarse_float(pL), cl = coarse_float(cL), rr = coarse_float(rR),
+              pr = coarse_float(pR), cr = coarse_float(cR);
+  const float du = coarse_float(uR - uL);
+  const float p0 = standard_guess_ppv<float>(rl, 0.0f, pl, cl, rr, du, pr, cr, coarse_float(ppv), G);
   float fL, dL, fR, dR;
   wave_curve(p0, rl, pl, cl, G, fL, dL);
   wave_curve(p0, rr, pr, cr, G, fR, dR);
@@ -495,7 +526,7 @@ __device__ __forceinline__ int riemann_sample(real rhoL, real uL, real pL, real 
                                               const GasC<real>& G, double tol, real tol_r, int maxit, bool have_guess,
                                               real guess, real& rhoF, real& uF, real& pF, RiemannInfo& info,
                                               real& pstar) {
-  const real cL = xsqrt(G.g * pL / rhoL), cR = xsqrt(G.g * pR / rhoR);
+  const real cL = xsqrt(xdiv(G.g * pL, rhoL)), cR = xsqrt(xdiv(G.g * pR, rhoR));
   return riemann_sample_c<GUARD>(rhoL, uL, pL, rhoR, uR, pR, cL, cR, linearised_pstar(rhoL, uL, pL, cL, rhoR, uR, pR, cR), G,
                           tol, tol_r, maxit, have_guess, guess, rhoF, uF, pF, info, pstar);
 }
