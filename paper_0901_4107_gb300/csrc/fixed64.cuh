@@ -129,6 +129,31 @@ __device__ __forceinline__ double sqrt64(double x) {
   return __longlong_as_double((i64)(((u64)(1022 + a.half) << 52) + r));
 }
 
+// x 2^-k, exact
+__device__ __forceinline__ double scale2(double x, int k) {
+  const int h = __double2hiint(x), e = (int)exponent_bits(h);
+  if (common((unsigned)e) && (unsigned)(e - k - 1) < 2046u)
+    return __hiloint2double(h - k * 0x100000, __double2loint(x));
+  return ldexp(x, -k);
+}
+
+// Conversions between FP64 and FP32, the narrowing one to nearest even, as the
+// instructions do, which take the FP64 pipe
+__device__ __forceinline__ float to_float(double x) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const int e = (int)exponent_bits((int)h) - 896;
+  const unsigned r = ((unsigned)e << 23) + ((h & 0xfffffu) << 3 | l >> 29);
+  const unsigned b = r + (((l & 0x1fffffffu) + 0x0fffffffu + (r & 1u)) >> 29) + (h & 0x80000000u);
+  if ((unsigned)(e - 1) < 254u) return __uint_as_float(b);
+  return (h << 1 | l) == 0u ? __uint_as_float(h) : (float)x;
+}
+__device__ __forceinline__ double to_double(float x) {
+  const unsigned b = __float_as_uint(x);
+  if ((b & 0x7f800000u) - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+  return (b << 1) == 0u ? __hiloint2double((int)b, 0) : (double)x;
+}
+
 // x^a for positive x by a table-driven logarithm and exponential (the method of Tang, ACM
 // TOMS 15 (1989) 144 and 16 (1990) 378):
 //   x = 2^e m, 1 <= m < 2, c from a table a little above 1/m, r = m c - 1 >= 0 (exact),

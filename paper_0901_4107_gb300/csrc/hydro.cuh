@@ -55,18 +55,18 @@ __device__ __forceinline__ real prims_from_Q(const HydroView<real>& v, int i, do
   real P;
   if constexpr (sizeof(real) == 8) {
     const double iV = v.cgeo[i].x;
-    const double im = 1.0 / m;
+    const double im = recip64(m);
     const double rho = m * iV;
     const double vx = px * im, vy = py * im, vz = pz * im;
     P = (v.gamma - 1.0) * (E * iV - 0.5 * rho * (vx * vx + vy * vy + vz * vz));
     w.x = rho; w.y = vx; w.z = vy; w.w = vz;
   } else {
     const float iV = v.cgeo[i].x;
-    const float mf = (float)m;
+    const float mf = to_float(m);
     const float im = 1.0f / mf;
-    const double kin = (px * px + py * py + pz * pz) * (double)(0.5f * im);
-    P = v.gas.gm1 * ((float)(E - kin) * iV);
-    w.x = mf * iV; w.y = (float)px * im; w.z = (float)py * im; w.w = (float)pz * im;
+    const double kin = (px * px + py * py + pz * pz) * to_double(0.5f * im);
+    P = v.gas.gm1 * (to_float(E - kin) * iV);
+    w.x = mf * iV; w.y = to_float(px) * im; w.z = to_float(py) * im; w.w = to_float(pz) * im;
   }
   v.cw[2 * (size_t)i] = w;
   reinterpret_cast<real*>(v.cw + 2 * (size_t)i + 1)[0] = P;   // .x; s - r stays in .yzw
@@ -80,7 +80,7 @@ __global__ void k_primitives(HydroView<real> v, unsigned long long* bad) {
   const double m = v.Q[i], px = v.Q[v.n + i], py = v.Q[2 * (size_t)v.n + i], pz = v.Q[3 * (size_t)v.n + i];
   const double E = v.Q[4 * (size_t)v.n + i];
   const real P = prims_from_Q(v, i, m, px, py, pz, E);
-  if (v.entropy) v.Aw[i] = (real)(v.S[i] / m);
+  if (v.entropy) v.Aw[i] = bulk<real>(div64(v.S[i], m));
   if (bad && (!(m > 0.0) || !(P > (real)0))) atomicAdd(bad, 1ull);
 }
 
@@ -240,7 +240,7 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
   if (cold) {
     mesh_velocity(v, ii, Wi, wi3);
     const real dx = Wi.y - wi3[0], dy = Wi.z - wi3[1], dz = Wi.w - wi3[2];
-    ekm = (real)0.5 * (real)v.Q[ii] * (dx * dx + dy * dy + dz * dz);
+    ekm = (real)0.5 * bulk<real>(v.Q[ii]) * (dx * dx + dy * dy + dz * dz);
   }
   // the neighbour index of the next incidence (the last word of its record)
   // is loaded one iteration ahead, so the neighbour's state load does not
@@ -273,7 +273,7 @@ __device__ __forceinline__ void grad_cell(const HydroView<real>& v, int i, int i
     if constexpr (ENT) phi_j[5] = v.Aw[j];
     if (cold) {
       const real dx = Wj.y - wi3[0], dy = Wj.z - wi3[1], dz = Wj.w - wi3[2];
-      const real ek = (real)0.5 * (real)v.Q[j] * (dx * dx + dy * dy + dz * dz);
+      const real ek = (real)0.5 * bulk<real>(v.Q[j]) * (dx * dx + dy * dy + dz * dz);
       ekm = ek > ekm ? ek : ekm;
     }
 #pragma unroll
@@ -1092,17 +1092,14 @@ __device__ __forceinline__ long long fixed_total(const FixDigits& d, int count, 
 // (largest magnitudes below 2^-105 keep a coarser image)
 __device__ __forceinline__ int fixed_exponent(int eb) { return min(148 - eb, 127); }
 
-// 2^-k in FP64 (exact), |k| < 1023
-__device__ __forceinline__ double pow2_neg(int k) { return __longlong_as_double((long long)(1023 - k) << 52); }
-
 // rho^gamma in the bulk precision (the FP32 forms' entropy switch takes it
 // in FP32, like the rest of their bulk arithmetic)
 template <typename real>
 __device__ __forceinline__ double rho_pow_gamma(const HydroView<real>& v, double rho) {
   if constexpr (sizeof(real) == 8) {
-    return pow(rho, v.gamma);
+    return pow64(rho, v.gamma);
   } else {
-    return (double)xpow((float)rho, v.gas.g);
+    return to_double(xpow(to_float(rho), v.gas.g));
   }
 }
 
@@ -1130,14 +1127,17 @@ static_assert(FIX_RUN % UPD_BATCH == 0, "a run is whole batches");
 // G consecutive lanes share a cell (as in the gradient kernel); lane l sums
 // the cell's incidences l, l+G, ..., and the lane sums are combined with
 // shuffles.  The cells of the CTA are then finished by its first CELL_TILE / G
-// threads, one each, and the others leave: finishing takes about thirty FP64
-// instructions per cell, and the narrow FP64 pipe takes a whole warp's time for
-// each whether 8 or 32 of its lanes are on.  What bounds it: the latency of the
+// threads, one each, and the others leave: finishing takes about twenty-five FP64
+// instructions per cell (thirty-eight with the FP64 pipe's conversions in place of
+// fixed64.cuh's, and 112 with the entropy switch, its divisions most of them), and
+// the narrow FP64 pipe takes a whole warp's time for each whether 8 or 32 of its
+// lanes are on.  What bounds it: the latency of the
 // chain list -> face index -> flux (long scoreboard; DRAM at a third, issue at a
 // third), so two fluxes and the next two indices are in flight per lane.
 // 1.4 M cells of 7.8 faces, 4 lanes per cell with lane 0 of each group
-// finishing its own cell: 471 us; 2 lanes, as here: 192 us (1 lane 217, 4
-// lanes 236).  ENT: the entropy switch of
+// finishing its own cell: 471 us; 2 lanes, as here: 192 us, 174 without FP64
+// conversions (1 lane 212, 4 lanes 233); 348 k cells with the entropy switch: 111 us,
+// 86 without FP64 conversions and divisions.  ENT: the entropy switch of
 // Sec. 3.5 (a sixth flux component, the entropy, and the per-cell choice
 // between the advected entropy and the energy update).
 template <typename real, int G, bool ENT = false>
@@ -1168,7 +1168,7 @@ __device__ __forceinline__ void update_item(const HydroView<real>& v, int wi) {
   if (tid == CELL_TILE - 1) {
     const double dt = box_dt(v, t.box);
     for (int a = 0; a < NA; a++)
-      s_dts[a] = (F32 && v.fixed_acc) ? dt * pow2_neg(fixed_exponent(largest_exponent(v, t.box, a)) + l2 + l3) : dt;
+      s_dts[a] = (F32 && v.fixed_acc) ? scale2(dt, fixed_exponent(largest_exponent(v, t.box, a)) + l2 + l3) : dt;
   }
   if (F32 && v.fixed_acc) {
     // Exact sums: every face flux is converted to an integer multiple of 2^-s
@@ -1319,22 +1319,23 @@ __device__ __forceinline__ void update_item(const HydroView<real>& v, int wi) {
       const double Sadv = v.S[i] - s_dts[5] * d[5];
       const double m = q[0];
       const double V = v.cgeo64[i].x;
-      const double rho = m / V;
-      const double kin = 0.5 * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) / m;
-      keep = ((double)mach < v.mach_thresh) ? 1u : 0u;
-      if (!keep && v.alpha_s > 0.0) keep = (q[4] - kin < v.alpha_s * (double)v.ekmax[i]) ? 1u : 0u;
+      const double iV = recip64(V), im = recip64(m);
+      const double rho = m * iV;
+      const double kin = 0.5 * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) * im;
+      keep = (widen(mach) < v.mach_thresh) ? 1u : 0u;
+      if (!keep && v.alpha_s > 0.0) keep = (q[4] - kin < v.alpha_s * widen(v.ekmax[i])) ? 1u : 0u;
       double Snew;
       if (keep) {
-        const double Pk = (Sadv / m) * rho_pow_gamma(v, rho);
-        q[4] = kin + Pk * V / (v.gamma - 1.0);
+        const double Pk = (Sadv * im) * rho_pow_gamma(v, rho);
+        q[4] = kin + div64(Pk * V, v.gamma - 1.0);
         Snew = Sadv;
       } else {
-        const double Pe = (v.gamma - 1.0) * (q[4] - kin) / V;
-        Snew = m * Pe / rho_pow_gamma(v, rho);
+        const double Pe = (v.gamma - 1.0) * (q[4] - kin) * iV;
+        Snew = div64(m * Pe, rho_pow_gamma(v, rho));
       }
       v.S[i] = Snew;
       v.kept[i] = (unsigned char)keep;
-      v.Aw[i] = (real)(Snew / m);
+      v.Aw[i] = bulk<real>(Snew * im);
     }
 #pragma unroll
     for (int a = 0; a < 5; a++) v.Q[a * n + i] = q[a];
@@ -1495,11 +1496,12 @@ __global__ void k_set_state(HydroView<real> v, const double* Qa, int dim, unsign
   if (v.entropy) {
     // S = M P / rho^gamma from the new state, in FP64
     const double V = v.cgeo64[i].x;
-    const double rho = m / V;
-    const double P64 = (v.gamma - 1.0) * (E - 0.5 * (px * px + py * py + pz * pz) / m) / V;
-    const double S = m * P64 / pow(rho, v.gamma);
+    const double iV = recip64(V), im = recip64(m);
+    const double rho = m * iV;
+    const double P64 = (v.gamma - 1.0) * (E - 0.5 * (px * px + py * py + pz * pz) * im) * iV;
+    const double S = div64(m * P64, pow64(rho, v.gamma));
     v.S[i] = S;
-    v.Aw[i] = (real)(S / m);
+    v.Aw[i] = bulk<real>(S * im);
     v.kept[i] = 0;
   }
   if (!(m > 0.0) || !(P > (real)0)) atomicAdd(bad, 1ull);

@@ -42,6 +42,18 @@ __device__ __forceinline__ float xdiv(float a, float b) { return a / b; }
 __device__ __forceinline__ double xrecip(double a) { return recip64(a); }
 __device__ __forceinline__ float xrecip(float a) { return 1.0f / a; }
 
+// an FP64 value in the bulk precision
+template <typename real>
+__device__ __forceinline__ real bulk(double x) {
+  if constexpr (sizeof(real) == 4)
+    return to_float(x);
+  else
+    return x;
+}
+
+__device__ __forceinline__ double widen(float x) { return to_double(x); }
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // Comparisons; FP64 ones in integers (an FP64 comparison takes the FP64 pipe): x > 0;
 // a < b and a <= b for a >= 0 (or its magnitude) and b >= 0, false where b is a NaN.
 __device__ __forceinline__ bool positive(float x) { return x > 0.0f; }

@@ -1,5 +1,5 @@
 """The fixed-point FP64 reciprocal, quotient, square roots and power of
-csrc/fixed64.cuh, compiled for the host with the two FP32 approximations
+csrc/fixed64.cuh, and its conversions, compiled for the host with the two FP32 approximations
 replaced by correctly rounded ones moved by -1, 0 or +1 ulp (their documented
 error), against long double.
 
@@ -44,6 +44,9 @@ static inline double __longlong_as_double(long long l) { double d; memcpy(&d, &l
 static inline int __double2hiint(double d) { return (int)(__double_as_longlong(d) >> 32); }
 static inline ulonglong2 __ldg(const ulonglong2* p) { return *p; }
 static inline unsigned long long __ldg(const unsigned long long* p) { return *p; }
+static inline unsigned __float_as_uint(float f) { unsigned u; memcpy(&u, &f, 4); return u; }
+static inline int __double2loint(double d) { return (int)__double_as_longlong(d); }
+static inline double __hiloint2double(int h, int l) { return __longlong_as_double((long long)h << 32 | (unsigned)l); }
 static double rsqrt(double x) { return 1 / std::sqrt(x); }
 """
 
@@ -72,6 +75,22 @@ int main() {
     m[4] = std::fmax(m[4], err(pow64(b, p), std::pow((long double)b, (long double)p)));
   }
   std::printf("recip %.6f\ndiv %.6f\nrsqrt %.6f\nsqrt %.6f\npow %.6f\n", m[0], m[1], m[2], m[3], m[4]);
+  // conversions and scaling: the same bits as the instructions', over all exponents, ties and neighbours of ties
+  long bad = 0;
+  for (long n = 0; n < 4000000; n++) {
+    unsigned long long b = rg();
+    if (n % 2) b = (b & 0x800fffffffffffffull) | (unsigned long long)(895 + rg() % 257) << 52;
+    if (n % 8 == 3) b = (b & ~0x1fffffffull) | (0x10000000ull + rg() % 3 - 1);
+    const double x = __longlong_as_double((long long)b);
+    const float f = to_float(x), f0 = (float)x, h = __uint_as_float((unsigned)rg());
+    const double d = to_double(h), d0 = (double)h;
+    bad += !(f == f0 || (f != f && f0 != f0)) + !(d == d0 || (d != d && d0 != d0));
+    const int k = (int)(rg() % 400) - 200;
+    const double s = std::ldexp(1 + U(), (int)(rg() % 1200) - 600);
+    bad += scale2(s, k) != std::ldexp(s, -k);
+  }
+  bad += std::signbit(to_float(-0.0)) == 0 || std::signbit(to_double(-0.0f)) == 0;
+  std::printf("convert %ld\n", bad);
   // arguments outside the fixed-point ranges take the library's results
   const bool ok = recip64(0.0) == INFINITY && recip64(-INFINITY) == 0 && div64(0.0, 2.0) == 0 && std::isnan(div64(NAN, 1.0)) &&
                   sqrt64(0.0) == 0 && std::isnan(sqrt64(-1.0)) && rsqrt64(INFINITY) == 0 && pow64(0.0, 0.2) == 0 &&
@@ -96,6 +115,6 @@ def test_fixed_point_functions(tmp_path):
     exe = tmp_path / "fixed64"
     subprocess.run([gxx, "-O2", "-w", "-std=c++17", "-o", str(exe), str(src)], check=True)
     out = dict(line.split() for line in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.splitlines())
-    assert float(out.pop("special")) == 0
+    assert float(out.pop("special")) == 0 and float(out.pop("convert")) == 0
     for name, bound in BOUND.items():
         assert float(out[name]) <= bound, (name, out)
