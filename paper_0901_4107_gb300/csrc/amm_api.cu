@@ -52,7 +52,7 @@ void free_ctx(amm_ctx* c) {
   void* ptrs[] = {c->gen,   c->box,     c->Q,       c->lr,       c->csr_off, c->csr,     c->ctiles,
                   c->ftiles, c->box_first_ctile, c->fgeo, c->igAB, c->cgeo64, c->cw,     c->grad, c->cwp, c->Apw,
                   c->wmesh, c->cgeo, c->crad, c->flux,    c->fluxE,   c->cour_bits, c->fmax_bits, c->wcorr, c->S, c->Aw, c->gradA, c->fluxS, c->machf, c->ekmax, c->kept, c->cell_perm, c->face_perm, c->barrier, c->box_status, c->dt_box, c->dt_used, c->partial,
-                  c->totals, c->stats,  c->closure, c->mlp,      c->defer_list, c->defer_count, c->scratch, c->counter,
+                  c->totals, c->segment, c->segment_count, c->stats,  c->closure, c->mlp,      c->defer_list, c->defer_count, c->scratch, c->counter,
                   c->ind_bin, c->ind_act, c->ind_list, c->ind_flist, c->ind_count, c->ind_fstamp, c->ind_cstamp,
                   c->ind_fdt, c->ind_hist, c->ind_cell_slot, c->ind_leaf_off, c->ind_level_off,
                   c->ind_rec, c->ind_rec32, c->ind_node, c->ind_loop, c->geo_ws, c->retess_ws, c->guard_mask};
@@ -406,6 +406,7 @@ int amm_create(amm_ctx** out, int dim, int64_t n, const double* gen, int64_t nf,
   c->n_ctiles = (int)ct.size();
   c->n_ftiles = (int)ft.size();
   c->box_first_ctile_h = bfc;
+  for (size_t b = 0; b + 1 < bfc.size(); b++) c->largest_box_ctiles = std::max(c->largest_box_ctiles, bfc[b + 1] - bfc[b]);
   // padded 3-vectors
   std::vector<double> gen3((size_t)n * 3, 0.0), cen3((size_t)nf * 3, 0.0), box3((size_t)nb * 3, 1.0);
   std::vector<int8_t> sh3((size_t)nf * 3, 0);
@@ -478,6 +479,9 @@ int amm_create(amm_ctx** out, int dim, int64_t n, const double* gen, int64_t nf,
   CUB(dalloc(&c->dt_used, (size_t)nb));
   CUB(dalloc(&c->partial, (size_t)5 * 8 * ct.size()));
   CUB(dalloc(&c->totals, (size_t)5 * nb));
+  CUB(dalloc(&c->segment, (size_t)5 * amm::FINISH_SEGMENTS * nb));
+  CUB(dalloc(&c->segment_count, (size_t)nb));
+  CUB(cudaMemsetAsync(c->segment_count, 0, sizeof(unsigned) * nb, c->stream));
   CUB(dalloc(&c->stats, 1));
   CUB(dalloc(&c->box_status, (size_t)nb));
   CUB(cudaMemsetAsync(c->box_status, 0, sizeof(unsigned) * nb, c->stream));

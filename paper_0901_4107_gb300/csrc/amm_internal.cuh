@@ -55,6 +55,7 @@ enum StatusBits : unsigned { ST_NEWTON_CAP = 1u, ST_NONPOS = 2u, ST_TIMEOUT = 4u
 
 // per-box largest |A F| slots: m, p (3), E, and the entropy flux
 constexpr int FMAX_STRIDE = 6;
+constexpr int FINISH_SEGMENTS = 64;   // most CTAs that add up one box's block partials
 
 struct DeviceStats {
   unsigned long long steps, faces, newton_iters, newton_fail, fallback, vacuum, guard, nonpos;
@@ -152,6 +153,8 @@ struct HydroView {
   const int* face_perm;
   double* partial;            // [n_ctiles][5]
   double* totals;             // [nboxes][5]
+  double* segment;            // [nboxes][FINISH_SEGMENTS][5] sums of parts of the partials
+  unsigned* segment_count;    // [nboxes] parts done, back to 0 when the last one is
   const int* box_first_ctile; // [nboxes+1]
   DeviceStats* stats;
   unsigned* box_status;        // [nboxes] StatusBits of each box
@@ -261,6 +264,9 @@ struct amm_ctx {
   void* flux = nullptr;
   void* fluxE = nullptr;
   unsigned long long* cour_bits = nullptr;
+  double* segment = nullptr;
+  unsigned* segment_count = nullptr;
+  int largest_box_ctiles = 0;
   unsigned* fmax_bits = nullptr;   // [nboxes][FMAX_STRIDE]
   void* wcorr = nullptr;           // regularity correction: [n] R4<real>
   double* S = nullptr;             // entropy switch: [n] total entropy

@@ -1428,24 +1428,31 @@ __global__ void __launch_bounds__(CELL_TILE) k_partial_sums(HydroView<real> v) {
   }
 }
 
-// One CTA per box: sum of the box's block partials in a fixed order; time step
-// record.  The partials are read as one run of doubles: a thread count that is
-// a multiple of 5 keeps each thread on one component, so the loads are
-// coalesced and eight are in flight per thread (latency bound; with one
-// 40-byte record per thread and a barrier per halving this took 41 us for 22k
-// records).
-constexpr int FINISH_THREADS = 1024;
+// Sum of a box's block partials in a fixed order; time step record.  The partials are
+// read as one run of doubles: a thread count that is a multiple of 5 keeps each
+// thread on one component, so the loads are coalesced and eight are in flight per
+// thread.  A box's run is cut into `segs` segments, a CTA each, about one round of
+// loads; the CTA that finishes last adds the segments' sums in order.  (One CTA of
+// 1024 threads per box: 21 us for 11 k blocks of 5 sums and 10 for 2 k, bound by
+// the FP64 additions of 32 warps on one SM; 9 and 8 now.)
+constexpr int FINISH_THREADS = 256;
 template <typename real, int NT>
-__device__ __forceinline__ void finish_item(const HydroView<real>& v, int b, int count_step) {
+__device__ __forceinline__ void finish_item(const HydroView<real>& v, int b, int count_step, int seg = 0, int segs = 1) {
   constexpr int NU = NT / 5 * 5;       // threads that read
   const int tid = (int)threadIdx.x;
   const size_t t0 = 5 * (size_t)v.box_first_ctile[b] * v.update_lanes;
-  const size_t t1 = 5 * (size_t)v.box_first_ctile[b + 1] * v.update_lanes;
+  const size_t te = 5 * (size_t)v.box_first_ctile[b + 1] * v.update_lanes;
+  const size_t run = ((te - t0) / 5 + segs - 1) / segs * 5;
+  const size_t ts = min(t0 + seg * run, te), t1 = min(ts + run, te);
   __shared__ double red[NT];
+  if (tid == NT - 1 && count_step && seg == 0) {
+    v.dt_used[b] = box_dt(v, b);
+    if (b == 0) atomicAdd(&v.stats->steps, 1ull);
+  }
   double s = 0.0;
   if (tid < NU) {
 #pragma unroll 1
-    for (size_t q = t0 + tid; q < t1; q += 8 * NU) {
+    for (size_t q = ts + tid; q < t1; q += 8 * NU) {
       double x[8];
 #pragma unroll
       for (int u = 0; u < 8; u++) x[u] = q + (size_t)u * NU < t1 ? v.partial[q + (size_t)u * NU] : 0.0;
@@ -1462,18 +1469,28 @@ __device__ __forceinline__ void finish_item(const HydroView<real>& v, int b, int
     for (int q = c + 5 * (tid & 31); q < NU; q += 160) r += red[q];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-    if ((tid & 31) == 0) v.totals[5 * b + c] = r;
+    if ((tid & 31) == 0) (segs > 1 ? v.segment : v.totals)[5 * ((size_t)b * segs + seg) + c] = r;
   }
-  if (tid == NT - 1 && count_step) {
-    v.dt_used[b] = box_dt(v, b);
-    if (b == 0) atomicAdd(&v.stats->steps, 1ull);
+  if (segs > 1) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicInc(v.segment_count + b, (unsigned)segs - 1u) == (unsigned)segs - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (tid < 5) {
+      double r = 0.0;
+      for (int k = 0; k < segs; k++) r += __ldcg(v.segment + 5 * ((size_t)b * segs + k) + tid);
+      v.totals[5 * b + tid] = r;
+    }
   }
   __syncthreads();   // `red` is reused when one CTA finishes several boxes
 }
 
 template <typename real>
 __global__ void __launch_bounds__(FINISH_THREADS) k_finish(HydroView<real> v, int count_step) {
-  finish_item<real, FINISH_THREADS>(v, blockIdx.x, count_step);
+  finish_item<real, FINISH_THREADS>(v, blockIdx.x, count_step, blockIdx.y, gridDim.y);
 }
 
 // ------------------------------------------------------------ layout moves
@@ -1605,6 +1622,8 @@ HydroView<real> make_view(amm_ctx* c, double cfl) {
   v.dt_box = c->dt_box;
   v.dt_used = c->dt_used;
   v.cour_bits = c->cour_bits;
+  v.segment = c->segment;
+  v.segment_count = c->segment_count;
   v.Q = c->Q;
   v.cw = (R4<real>*)c->cw;
   v.grad = (R4<real>*)c->grad;
@@ -1754,11 +1773,14 @@ cudaError_t launch_update(amm_ctx* c, double cfl) {
 template <typename real>
 cudaError_t launch_finish(amm_ctx* c, double cfl) {
   auto v = make_view<real>(c, cfl);
+  const int64_t sums = 5 * (int64_t)c->largest_box_ctiles * c->update_lanes;
+  const int segs = (int)std::min<int64_t>((sums + 8 * FINISH_THREADS - 1) / (8 * FINISH_THREADS), FINISH_SEGMENTS);
+  const dim3 grid(c->nboxes, segs);
   if (cfl < 0.0) {  // totals of the current state, no step
     k_partial_sums<real><<<c->n_ctiles, CELL_TILE, 0, c->stream>>>(v);
-    k_finish<real><<<c->nboxes, FINISH_THREADS, 0, c->stream>>>(v, 0);
+    k_finish<real><<<grid, FINISH_THREADS, 0, c->stream>>>(v, 0);
   } else {
-    k_finish<real><<<c->nboxes, FINISH_THREADS, 0, c->stream>>>(v, 1);
+    k_finish<real><<<grid, FINISH_THREADS, 0, c->stream>>>(v, 1);
   }
   return cudaGetLastError();
 }
