@@ -58,6 +58,7 @@ void free_ctx(amm_ctx* c) {
                   c->ind_rec, c->ind_rec32, c->ind_node, c->ind_loop, c->geo_ws, c->retess_ws, c->guard_mask};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  if (c->note) cudaFreeHost(c->note);
 
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   if (c->aux_stream) cudaStreamDestroy(c->aux_stream);
@@ -487,6 +488,8 @@ int amm_create(amm_ctx** out, int dim, int64_t n, const double* gen, int64_t nf,
   CUB(cudaMemsetAsync(c->box_status, 0, sizeof(unsigned) * nb, c->stream));
   CUB(dalloc(&c->closure, (size_t)n));
   CUB(dalloc(&c->counter, 4));
+  CUB(cudaMemsetAsync(c->counter, 0, sizeof(unsigned long long), c->stream));
+  CUB(cudaHostAlloc((void**)&c->note, sizeof(amm::HostNote), cudaHostAllocDefault));
   CUB(dalloc(&c->barrier, 2));
   CUB(cudaMemsetAsync(c->barrier, 0, sizeof(unsigned) * 2, c->stream));
   CUB(cudaMemsetAsync(c->stats, 0, sizeof(amm::DeviceStats), c->stream));
@@ -583,16 +586,18 @@ int amm_destroy(amm_ctx* c) {
 }
 
 static int set_state_common(amm_ctx* c, const double* Qdev_aos) {
-  CU(cudaMemsetAsync(c->counter, 0, sizeof(unsigned long long), c->stream));
+  c->note->bad = 0;
   CU(dispatch(c, [&] { return amm::launch_set_state<double>(c, Qdev_aos, c->counter); },
               [&] { return amm::launch_set_state<float>(c, Qdev_aos, c->counter); }));
-  unsigned long long bad = 0;
-  CU(cudaMemcpyAsync(&bad, c->counter, sizeof(bad), cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
   c->grads_fresh = false;
   c->totals_fresh = false;
-  if (bad) return fail(c, AMM_ERR_NONPOSITIVE_STATE, std::to_string(bad) + " cells with m <= 0 or P <= 0");
-  return AMM_OK;
+  if (!c->note->bad) return AMM_OK;
+  unsigned long long bad = 0;
+  CU(cudaMemcpyAsync(&bad, c->counter, sizeof(bad), cudaMemcpyDeviceToHost, c->stream));
+  CU(cudaMemsetAsync(c->counter, 0, sizeof(bad), c->stream));
+  CU(cudaStreamSynchronize(c->stream));
+  return fail(c, AMM_ERR_NONPOSITIVE_STATE, std::to_string(bad) + " cells with m <= 0 or P <= 0");
 }
 
 int amm_set_state(amm_ctx* c, const double* Q) {
@@ -977,19 +982,21 @@ int amm_get_state(amm_ctx* c, double* Q) {
   if (!c || !Q) return fail(c, AMM_ERR_INVALID_ARG, "null argument");
   const size_t cnt = (size_t)c->n * (c->dim + 2);
   CU(ensure_scratch(c, cnt));
+  c->note->status = 0;
   CU(dispatch(c, [&] { return amm::launch_get_state<double>(c, c->scratch); },
               [&] { return amm::launch_get_state<float>(c, c->scratch); }));
   CU(cudaMemcpyAsync(Q, c->scratch, sizeof(double) * cnt, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
-  return check_status(c);
+  return c->note->status ? check_status(c) : AMM_OK;
 }
 
 int amm_get_state_device(amm_ctx* c, double* Qd) {
   if (!c || !Qd) return fail(c, AMM_ERR_INVALID_ARG, "null argument");
+  c->note->status = 0;
   CU(dispatch(c, [&] { return amm::launch_get_state<double>(c, Qd); },
               [&] { return amm::launch_get_state<float>(c, Qd); }));
   CU(cudaStreamSynchronize(c->stream));
-  return check_status(c);
+  return c->note->status ? check_status(c) : AMM_OK;
 }
 
 int amm_get_primitives(amm_ctx* c, double* W) {

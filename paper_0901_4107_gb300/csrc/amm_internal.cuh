@@ -55,6 +55,13 @@ enum StatusBits : unsigned { ST_NEWTON_CAP = 1u, ST_NONPOS = 2u, ST_TIMEOUT = 4u
 
 // per-box largest |A F| slots: m, p (3), E, and the entropy flux
 constexpr int FMAX_STRIDE = 6;
+// What a call needs to know from the device, written by its kernel straight to the
+// host and read after the stream's synchronisation: set only in the rare cases, so
+// that the usual call copies nothing back.
+struct HostNote {
+  unsigned bad;                    // set_state: a cell was not positive (the count is in `counter`)
+  unsigned status;                 // get_state: the step statistics' status is not zero
+};
 constexpr int FINISH_SEGMENTS = 64;   // most CTAs that add up one box's block partials
 
 struct DeviceStats {
@@ -121,6 +128,7 @@ struct HydroView {
   int fixed_acc;               // FP32 forms: exact int64 fixed-point flux sums
   int headroom;                // bits reserved for the incidence count in the fixed-point sums
   int update_lanes;            // lanes per cell of the update kernel (partial sums per block)
+  unsigned* defer_count;       // faces the learned form's flux kernel has listed (null otherwise)
   unsigned* fmax_bits;         // [nboxes][FMAX_STRIDE] max |A F| per component (float bits) of the step
   // dt source: dt_box[b] if cfl <= 0, else cfl * courant_min[b]
   double cfl;
@@ -304,7 +312,8 @@ struct amm_ctx {
   void* tess_ws = nullptr;         // amm_retessellate: the GPU tessellation's workspace (amm::vor::TessWork)
   int64_t nf_cap = 0;              // faces the face-sized buffers hold
   size_t scratch_size = 0;         // in doubles
-  unsigned long long* counter = nullptr;
+  unsigned long long* counter = nullptr;   // [4]; [0] is zero between calls
+  amm::HostNote* note = nullptr;        // page-locked host memory the kernels write to
   bool grads_fresh = false;
   bool totals_fresh = false;
   bool have_step = false;

@@ -363,9 +363,8 @@ cudaError_t launch_flux_learned(amm_ctx* c, const HydroView<float>& v) {
   d.list = c->defer_list;
   d.count = c->defer_count;
   d.capacity = (unsigned)c->nf_cap;
-  cudaError_t e = cudaMemsetAsync(c->defer_count, 0, sizeof(unsigned), c->stream);
+  cudaError_t e = launch_flux_chunks(c, v, true, d);
   if (e != cudaSuccess) return e;
-  if ((e = launch_flux_chunks(c, v, true, d)) != cudaSuccess) return e;
   int dev = 0, sms = 148;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;

@@ -482,6 +482,12 @@ __device__ __forceinline__ void grad_item(const HydroView<real>& v, int wi) {
 
 template <typename real, int G, bool ENT>
 __global__ void __launch_bounds__(CELL_TILE, sizeof(real) == 4 ? 4 : 2) k_gradients(HydroView<real> v) {
+  // the flux kernel's maxima (and the learned form's list of faces), which nothing
+  // else touches now
+  if (blockIdx.x == 0) {
+    for (int x = threadIdx.x; x < FMAX_STRIDE * v.nboxes; x += CELL_TILE) v.fmax_bits[x] = 0u;
+    if (v.defer_count && threadIdx.x == 0) *v.defer_count = 0u;
+  }
   grad_item<real, G, ENT>(v, blockIdx.x);
 }
 
@@ -1495,7 +1501,7 @@ __global__ void __launch_bounds__(FINISH_THREADS) k_finish(HydroView<real> v, in
 
 // ------------------------------------------------------------ layout moves
 template <typename real>
-__global__ void k_set_state(HydroView<real> v, const double* Qa, int dim, unsigned long long* bad) {
+__global__ void k_set_state(HydroView<real> v, const double* Qa, int dim, unsigned long long* bad, HostNote* note) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= v.n) return;
   const int nv = dim + 2;
@@ -1521,12 +1527,16 @@ __global__ void k_set_state(HydroView<real> v, const double* Qa, int dim, unsign
     v.Aw[i] = bulk<real>(S * im);
     v.kept[i] = 0;
   }
-  if (!(m > 0.0) || !(P > (real)0)) atomicAdd(bad, 1ull);
+  if (!(m > 0.0) || !(P > (real)0)) {
+    atomicAdd(bad, 1ull);
+    note->bad = 1u;
+  }
 }
 
 template <typename real>
-__global__ void k_get_state(HydroView<real> v, double* Qa, int dim) {
+__global__ void k_get_state(HydroView<real> v, double* Qa, int dim, HostNote* note) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0 && v.stats->status) note->status = v.stats->status;
   if (i >= v.n) return;
   const int nv = dim + 2;
   const size_t n = (size_t)v.n;
@@ -1622,6 +1632,7 @@ HydroView<real> make_view(amm_ctx* c, double cfl) {
   v.dt_box = c->dt_box;
   v.dt_used = c->dt_used;
   v.cour_bits = c->cour_bits;
+  v.defer_count = c->defer_count;
   v.segment = c->segment;
   v.segment_count = c->segment_count;
   v.Q = c->Q;
@@ -1696,8 +1707,6 @@ cudaError_t launch_gradients(amm_ctx* c, double cfl) {
   // mesh it finds the Courant minimum itself
   cudaError_t e = v.pred ? launch_courant<real>(c)
                          : cudaMemsetAsync(c->cour_bits, 0xff, sizeof(unsigned long long) * c->nboxes, c->stream);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(c->fmax_bits, 0, sizeof(unsigned) * FMAX_STRIDE * c->nboxes, c->stream);
   if (e != cudaSuccess) return e;
   if (c->opt.entropy) {
     switch (c->grad_lanes) {
@@ -1788,14 +1797,14 @@ cudaError_t launch_finish(amm_ctx* c, double cfl) {
 template <typename real>
 cudaError_t launch_set_state(amm_ctx* c, const double* Qa, unsigned long long* bad) {
   auto v = make_view<real>(c, 0.0);
-  k_set_state<real><<<nblk(c->n, 256), 256, 0, c->stream>>>(v, Qa, c->dim, bad);
+  k_set_state<real><<<nblk(c->n, 256), 256, 0, c->stream>>>(v, Qa, c->dim, bad, c->note);
   return cudaGetLastError();
 }
 
 template <typename real>
 cudaError_t launch_get_state(amm_ctx* c, double* Qa) {
   auto v = make_view<real>(c, 0.0);
-  k_get_state<real><<<nblk(c->n, 256), 256, 0, c->stream>>>(v, Qa, c->dim);
+  k_get_state<real><<<nblk(c->n, 256), 256, 0, c->stream>>>(v, Qa, c->dim, c->note);
   return cudaGetLastError();
 }
 
