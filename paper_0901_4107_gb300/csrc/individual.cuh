@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(32 * BINS_WARPS, 4) k_ind_cells(HydroView<real
 // bounds the few faces of most ticks is the chain of one warp's FP64 instructions,
 // which cost the same however few lanes are on; so warps (B = 32) take few faces each,
 // down to one, with a lane for each side of a face, and the pipes of all SMs are used (70 us a tick
-// with CTAs of 128 for some 340 faces, 47 now).  Many faces go to CTAs of 128, which group their solves.
+// with CTAs of 128 for some 340 faces, 47 so, 22 with fixed64.cuh).  Many faces go to CTAs of 128, which group their solves.
 template <typename real, int B>
 __global__ void __launch_bounds__(B) k_ind_flux(HydroView<real> v, IndView d, int above, int most) {
   const int count = d.count[1];
@@ -616,7 +616,7 @@ __global__ void __launch_bounds__(B) k_ind_flux(HydroView<real> v, IndView d, in
 // --------------------------------------------------- the pairwise exchange
 // Four lanes per cell, each with every fourth incidence, its face's stamp, step
 // and flux loaded whether or not the face is active (a thread per cell waited for
-// each in turn: 31 us a tick, 15 now, 32768 cells with few touched).
+// each in turn: 31 us a tick, 13 now, 32768 cells with few touched).
 template <typename real>
 __global__ void __launch_bounds__(256) k_ind_update(HydroView<real> v, IndView d) {
   constexpr int G = 4;
