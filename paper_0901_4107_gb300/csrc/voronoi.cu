@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "amm.h"
+#include "half_list.cuh"
 #include "scan.cuh"
 
 namespace amm {
@@ -73,17 +74,23 @@ struct HalfFace {
 // later pass.)
 struct HalfList {
   HalfFace* f;
-  int* first;
-  int* used;
-  int cap;
+  int64_t* first;
+  unsigned long long* used;
+  int64_t cap;
 };
 
 // room for m faces of cell i, by one lane; -1 if the list is full
-__device__ __forceinline__ int half_room(const HalfList& H, int i, int m) {
-  const int at = atomicAdd(H.used, m);
-  H.first[i] = at;
-  return at >= 0 && at <= H.cap - m ? at : -1;
+__device__ __forceinline__ int64_t half_room(const HalfList& H, int i, int m) {
+  const unsigned long long at = atomicAdd(H.used, (unsigned long long)m);
+  H.first[i] = (int64_t)at;
+  return half_place(at, m, H.cap);
 }
+
+// what a build tells the host
+struct TessCount {
+  int err, left;               // error; cells left to k_cells3
+  unsigned long long used;     // half-faces taken
+};
 
 __device__ __forceinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
@@ -912,7 +919,7 @@ __global__ void __launch_bounds__(32 * FWARPS, 5) k_cells3_fast(const __grid_con
       int mf = 0;
       for (int k0 = 6; k0 < np; k0 += 32)
         mf += __popc(__ballot_sync(full, k0 + lane < np && S.u.f.start[k0 + lane] < 64));
-      int room = 0;
+      int64_t room = 0;
       if (lane == 0) room = half_room(H, i, mf);
       room = __shfl_sync(full, room, 0);
       // faces: lane per plane, its vertices from one to the next
@@ -1115,7 +1122,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_cells3(Grid G, HalfList H, int* 
     int nf = 0;
     double V = 0.0, M[3] = {0.0, 0.0, 0.0};
     if (rc == 0) {
-      int room = 0;
+      int64_t room = 0;
       if (lane == 0) room = half_room(H, i, MAXHF);
       room = __shfl_sync(0xffffffffu, room, 0);
       for (int k0 = 6; k0 < C.np; k0 += 32) {
@@ -1369,7 +1376,7 @@ __global__ void k_cells2(Grid G, HalfList H, int* nhf, double* vol, double* com,
       nf++;
     }
   }
-  H.first[i] = i * 32;
+  H.first[i] = (int64_t)i * 32;
   nhf[i] = rc == 0 ? nf : 0;
   vol[i] = V;
   com[(size_t)i * 2] = ri[0] + (V > 0.0 ? M[0] / V : 0.0);
@@ -1392,17 +1399,26 @@ __device__ __forceinline__ bool keep_face(int i, const HalfFace& f, int dim) {
 // other, each from its own sector).
 constexpr int FLANES = 16;
 
-__global__ void k_keep_count(int n, int dim, const HalfFace* hf, const int* first, const int* nhf, int* keep) {
+__global__ void k_keep_count(int n, int dim, const HalfFace* hf, const int64_t* first, const int* nhf, int* keep) {
   const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / FLANES), l = threadIdx.x % FLANES;
   int c = 0;
   if (i < n)
-    for (int f = l; f < nhf[i]; f += FLANES) c += keep_face(i, hf[(size_t)first[i] + f], dim) ? 1 : 0;
+    for (int f = l; f < nhf[i]; f += FLANES) c += keep_face(i, hf[first[i] + f], dim) ? 1 : 0;
 #pragma unroll
   for (int o = FLANES / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if (i < n && l == 0) keep[i] = c;
 }
 
-__global__ void k_emit(int n, int dim, const double* pts, const HalfFace* hf, const int* first, const int* nhf,
+// their sum over all cells, where the scan's 32 bits might not hold it
+__global__ void __launch_bounds__(256) k_keep_total(int n, const int* keep, unsigned long long* total) {
+  unsigned long long c = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) c += keep[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  if ((threadIdx.x & 31) == 0) atomicAdd(total, c);
+}
+
+__global__ void k_emit(int n, int dim, const double* pts, const HalfFace* hf, const int64_t* first, const int* nhf,
                        const int* off, int32_t* cells, int8_t* shift, double* area, double* cen) {
   const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / FLANES), l = threadIdx.x % FLANES;
   const int base = (threadIdx.x & 31) / FLANES * FLANES;   // the group's first lane
@@ -1432,14 +1448,14 @@ __global__ void k_emit(int n, int dim, const double* pts, const HalfFace* hf, co
 // missing ones, the largest relative area mismatch (positive doubles order
 // like their bit patterns; one atomic per warp, and only where it would
 // change the maximum)
-__global__ void k_mirror(int n, int dim, const HalfFace* hf, const int* first, const int* nhf,
+__global__ void k_mirror(int n, int dim, const HalfFace* hf, const int64_t* first, const int* nhf,
                          unsigned long long* missing, unsigned long long* maxrel_bits) {
   const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / FLANES), l = threadIdx.x % FLANES;
   double rel = 0.0;
   int miss = 0;
   if (i < n)
     for (int f = l; f < nhf[i]; f += FLANES) {
-      const HalfFace& h = hf[(size_t)first[i] + f];
+      const HalfFace& h = hf[first[i] + f];
       if (!keep_face(i, h, dim)) continue;
       const HalfFace* other = hf + first[h.j];
       const int mo = nhf[h.j];
@@ -1491,8 +1507,9 @@ struct TessWork {
   int cap_dim = 0;
   char *cell_ws = nullptr, *face_ws = nullptr;
   int *binof = nullptr, *count = nullptr, *start = nullptr, *cursor = nullptr, *bin_pts = nullptr;
-  int *nhf = nullptr, *keep = nullptr, *off = nullptr, *left = nullptr, *part = nullptr, *first = nullptr;
-  int* err = nullptr;                  // error, cells left to k_cells3, half-faces taken
+  int *nhf = nullptr, *keep = nullptr, *off = nullptr, *left = nullptr, *part = nullptr;
+  int64_t* first = nullptr;
+  TessCount* told = nullptr;
   unsigned long long* chk = nullptr;   // missing mirrors, largest area mismatch
   HalfFace* hf = nullptr;
   double *vol = nullptr, *com = nullptr;
@@ -1602,7 +1619,7 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
       at(w->start, nbins + 1);
       at(w->cursor, nbins);
       at(w->part, std::max(scan_scratch(n), scan_scratch(nbins)));
-      at(w->err, 4);
+      at(w->told, 1);
       at(w->chk, 2);
       if (pass == 0 && !cu(cudaMalloc(&w->cell_ws, at.bytes), "alloc")) return rc;
     }
@@ -1614,7 +1631,7 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
   // generators); a build that needs more is repeated with that
   const auto hf_room = [&](int64_t want) {
     if (want <= w->cap_hf && w->hf) return true;
-    if (want > 0x7fffffffll - 64) {
+    if (dim == 2 && want > INT32_MAX - 64) {
       g_tess_err = "more half-faces than the builder can index";
       rc = AMM_ERR_NUMERIC;
       return false;
@@ -1625,13 +1642,13 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
     if (cu(cudaMalloc((void**)&w->hf, sizeof(HalfFace) * (size_t)want), "alloc")) w->cap_hf = want;
     return rc == AMM_OK;
   };
-  if (!hf_room(dim == 3 ? std::min<int64_t>(18 * n + 1024, 0x7fffffffll - 64) : 32 * n)) return rc;
+  if (!hf_room(dim == 3 ? 18 * n + 1024 : 32 * n)) return rc;
   const int nb256 = (int)((n + 255) / 256);
   G.pts = gen_d;
   cu(cudaMemsetAsync(w->count, 0, sizeof(int) * nbins, st), "memset");
-  cu(cudaMemsetAsync(w->err, 0, 4 * sizeof(int), st), "memset");
+  cu(cudaMemsetAsync(w->told, 0, sizeof(TessCount), st), "memset");
   cu(cudaMemsetAsync(w->chk, 0, sizeof(unsigned long long) * 2, st), "memset");
-  k_check_range<<<nb256, 256, 0, st>>>(G, w->err);
+  k_check_range<<<nb256, 256, 0, st>>>(G, &w->told->err);
   k_bin_count<<<nb256, 256, 0, st>>>(G, w->binof, w->count);
   cu(exclusive_scan(w->count, w->start, nbins, w->part, st), "scan");
   cu(cudaMemcpyAsync(w->cursor, w->start, sizeof(int) * nbins, cudaMemcpyDeviceToDevice, st), "copy");
@@ -1641,9 +1658,9 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
   G.bin_pts = w->bin_pts;
   const double thr = 1e-12 * std::pow(hcell, dim - 1);
   const int nbf = (int)((n * FLANES + 255) / 256);
-  int herr[4] = {0, 0, 0, 0};
+  TessCount told{};
   for (;;) {
-    const HalfList H{w->hf, w->first, w->err + 2, (int)w->cap_hf};
+    const HalfList H{w->hf, w->first, &w->told->used, w->cap_hf};
     if (dim == 3) {
       const size_t smem = sizeof(Cell3) * WARPS, fsmem = sizeof(Fast3) * FWARPS;
       cu(cudaFuncSetAttribute(k_cells3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "attribute");
@@ -1651,32 +1668,46 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
       // the ordinary cells, then whatever they left (often nothing)
       const int64_t fblocks = std::min<int64_t>((n + FWARPS - 1) / FWARPS, 152 * 5);
       const int64_t blocks = std::min<int64_t>((n + WARPS - 1) / WARPS, 152 * 4);
-      k_cells3_fast<<<(int)fblocks, 32 * FWARPS, fsmem, st>>>(G, H, w->nhf, w->vol, w->com, w->binof, w->left, w->err + 1,
-                                                            thr);
-      k_cells3<<<(int)blocks, 32 * WARPS, smem, st>>>(G, H, w->nhf, w->vol, w->com, w->err, w->left, w->err + 1, thr);
+      k_cells3_fast<<<(int)fblocks, 32 * FWARPS, fsmem, st>>>(G, H, w->nhf, w->vol, w->com, w->binof, w->left,
+                                                            &w->told->left, thr);
+      k_cells3<<<(int)blocks, 32 * WARPS, smem, st>>>(G, H, w->nhf, w->vol, w->com, &w->told->err, w->left, &w->told->left,
+                                                      thr);
     } else {
-      k_cells2<<<nb256, 256, 0, st>>>(G, H, w->nhf, w->vol, w->com, w->err, thr);
+      k_cells2<<<nb256, 256, 0, st>>>(G, H, w->nhf, w->vol, w->com, &w->told->err, thr);
     }
     cu(cudaGetLastError(), "cells");
-    cu(cudaMemcpyAsync(herr, w->err, 3 * sizeof(int), cudaMemcpyDeviceToHost, st), "read");
+    cu(cudaMemcpyAsync(&told, w->told, sizeof told, cudaMemcpyDeviceToHost, st), "read");
     // (the pass below reads the list: only where it holds every face)
     cu(cudaStreamSynchronize(st), "sync");
     if (rc != AMM_OK) return rc;
-    if (herr[0] != 0) {
-      g_tess_err = tess_msg(herr[0]);
-      return herr[0] == -5 ? AMM_ERR_INVALID_ARG : AMM_ERR_NUMERIC;
+    if (told.err != 0) {
+      g_tess_err = tess_msg(told.err);
+      return told.err == -5 ? AMM_ERR_INVALID_ARG : AMM_ERR_NUMERIC;
     }
-    if (dim == 2 || (herr[2] >= 0 && herr[2] <= w->cap_hf)) break;
     // (each warp's count is added whether or not it fits, so this is enough)
-    if (!hf_room(herr[2] < 0 ? 0x7fffffffll : (int64_t)herr[2] + 1024)) return rc;
-    cu(cudaMemsetAsync(w->err, 0, 4 * sizeof(int), st), "memset");
+    const int64_t more = half_more(told.used, w->cap_hf);
+    if (more == 0) break;
+    if (!hf_room(more)) return rc;
+    cu(cudaMemsetAsync(w->told, 0, sizeof(TessCount), st), "memset");
   }
   k_keep_count<<<nbf, 256, 0, st>>>((int)n, dim, w->hf, w->first, w->nhf, w->keep);
+  if ((dim == 3 ? (int64_t)told.used : 32 * n) > INT32_MAX) {   // (faces are half-faces or fewer)
+    cu(cudaMemsetAsync(&w->told->used, 0, sizeof told.used, st), "memset");
+    k_keep_total<<<152 * 8, 256, 0, st>>>((int)n, w->keep, &w->told->used);
+    cu(cudaMemcpyAsync(&told, w->told, sizeof told, cudaMemcpyDeviceToHost, st), "read");
+    cu(cudaStreamSynchronize(st), "sync");
+    if (rc != AMM_OK) return rc;
+    if (told.used > INT32_MAX) {
+      g_tess_err = "more faces than the builder can index";
+      return AMM_ERR_NUMERIC;
+    }
+  }
   cu(exclusive_scan(w->keep, w->off, n, w->part, st), "scan");
-  cu(cudaMemcpyAsync(&herr[1], w->off + n, sizeof(int), cudaMemcpyDeviceToHost, st), "read");
+  int kept = 0;
+  cu(cudaMemcpyAsync(&kept, w->off + n, sizeof(int), cudaMemcpyDeviceToHost, st), "read");
   cu(cudaStreamSynchronize(st), "sync");
   if (rc != AMM_OK) return rc;
-  const int64_t nf = herr[1];
+  const int64_t nf = kept;
   if (nf < 1) {
     g_tess_err = "no faces";
     return AMM_ERR_NUMERIC;
