@@ -46,7 +46,8 @@ constexpr int MAXP = 128;     // planes per cell: 6 of the box + the cutting bis
 constexpr int MAXT = 384;     // vertex slots (dual triangles), dead ones included
 constexpr int MAXC = 192;     // candidates gathered per pass
 constexpr int MAXFV = 48;     // vertices of one face
-constexpr int MAXHF = 64;     // output half-faces per cell (3D); 2D uses 32
+constexpr int MAXHF = 64;     // output half-faces per cell (3D)
+constexpr int HF2 = 32;       // the same in 2D
 
 // error codes, as the host tessellator's
 constexpr int E_CAPACITY = -1, E_VANISHED = -2, E_INCOMPLETE = -3, E_OPEN = -4, E_FACES = -6, E_CANDIDATES = -7;
@@ -71,13 +72,15 @@ struct HalfFace {
 // first[i].  A warp takes room for its cell's faces from `used`; past the
 // capacity nothing is written and the build is repeated with more room.  (64
 // places for every cell were 671 MB at 64^3, mostly empty and strided in every
-// later pass.)
+// later pass.)  2D (first null): a run of HF2 places for every cell.
 struct HalfList {
   HalfFace* f;
   int64_t* first;
   unsigned long long* used;
   int64_t cap;
 };
+
+__device__ __forceinline__ int64_t half_run(const int64_t* first, int i) { return first ? first[i] : (int64_t)i * HF2; }
 
 // room for m faces of cell i, by one lane; -1 if the list is full
 __device__ __forceinline__ int64_t half_room(const HalfList& H, int i, int m) {
@@ -1359,11 +1362,11 @@ __global__ void k_cells2(Grid G, HalfList H, int* nhf, double* vol, double* com,
       M[0] += at * (2.0 / 3.0) * 0.5 * (u[0] + w[0]);
       M[1] += at * (2.0 / 3.0) * 0.5 * (u[1] + w[1]);
       if (len <= thr_len) continue;
-      if (nf >= 32) {
+      if (nf >= HF2) {
         rc = E_CAPACITY;
         break;
       }
-      HalfFace& o = H.f[(size_t)i * 32 + nf];
+      HalfFace& o = H.f[half_run(nullptr, i) + nf];
       o.j = L[k].j;
       o.s[0] = L[k].s[0];
       o.s[1] = L[k].s[1];
@@ -1376,7 +1379,6 @@ __global__ void k_cells2(Grid G, HalfList H, int* nhf, double* vol, double* com,
       nf++;
     }
   }
-  H.first[i] = (int64_t)i * 32;
   nhf[i] = rc == 0 ? nf : 0;
   vol[i] = V;
   com[(size_t)i * 2] = ri[0] + (V > 0.0 ? M[0] / V : 0.0);
@@ -1403,7 +1405,7 @@ __global__ void k_keep_count(int n, int dim, const HalfFace* hf, const int64_t* 
   const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / FLANES), l = threadIdx.x % FLANES;
   int c = 0;
   if (i < n)
-    for (int f = l; f < nhf[i]; f += FLANES) c += keep_face(i, hf[first[i] + f], dim) ? 1 : 0;
+    for (int f = l; f < nhf[i]; f += FLANES) c += keep_face(i, hf[half_run(first, i) + f], dim) ? 1 : 0;
 #pragma unroll
   for (int o = FLANES / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if (i < n && l == 0) keep[i] = c;
@@ -1427,7 +1429,7 @@ __global__ void k_emit(int n, int dim, const double* pts, const HalfFace* hf, co
   // (the groups of a warp run as many rounds as the longest list)
   for (int f0 = 0; __any_sync(0xffffffffu, f0 < m); f0 += FLANES) {
     const int f = f0 + l;
-    const HalfFace* h = hf + (i < n ? first[i] : 0) + f;
+    const HalfFace* h = hf + (i < n ? half_run(first, i) : 0) + f;
     const bool keep = f < m && keep_face(i, *h, dim);
     const unsigned k = (__ballot_sync(0xffffffffu, keep) >> base) & ((1u << FLANES) - 1u);
     if (keep) {
@@ -1455,9 +1457,9 @@ __global__ void k_mirror(int n, int dim, const HalfFace* hf, const int64_t* firs
   int miss = 0;
   if (i < n)
     for (int f = l; f < nhf[i]; f += FLANES) {
-      const HalfFace& h = hf[first[i] + f];
+      const HalfFace& h = hf[half_run(first, i) + f];
       if (!keep_face(i, h, dim)) continue;
-      const HalfFace* other = hf + first[h.j];
+      const HalfFace* other = hf + half_run(first, h.j);
       const int mo = nhf[h.j];
       int g = 0;
       for (; g < mo; g++) {
@@ -1611,8 +1613,8 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
       at(w->nhf, n);
       at(w->keep, n);
       at(w->off, n + 1);
-      at(w->left, n);
-      at(w->first, n);
+      at(w->left, dim == 3 ? n : 0);
+      at(w->first, dim == 3 ? n : 0);
       at(w->vol, n);
       at(w->com, 3 * n);
       at(w->count, nbins);
@@ -1631,18 +1633,13 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
   // generators); a build that needs more is repeated with that
   const auto hf_room = [&](int64_t want) {
     if (want <= w->cap_hf && w->hf) return true;
-    if (dim == 2 && want > INT32_MAX - 64) {
-      g_tess_err = "more half-faces than the builder can index";
-      rc = AMM_ERR_NUMERIC;
-      return false;
-    }
     if (w->hf) cudaFree(w->hf);
     w->hf = nullptr;
     w->cap_hf = 0;
     if (cu(cudaMalloc((void**)&w->hf, sizeof(HalfFace) * (size_t)want), "alloc")) w->cap_hf = want;
     return rc == AMM_OK;
   };
-  if (!hf_room(dim == 3 ? 18 * n + 1024 : 32 * n)) return rc;
+  if (!hf_room(dim == 3 ? 18 * n + 1024 : HF2 * n)) return rc;
   const int nb256 = (int)((n + 255) / 256);
   G.pts = gen_d;
   cu(cudaMemsetAsync(w->count, 0, sizeof(int) * nbins, st), "memset");
@@ -1659,6 +1656,7 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
   const double thr = 1e-12 * std::pow(hcell, dim - 1);
   const int nbf = (int)((n * FLANES + 255) / 256);
   TessCount told{};
+  const int64_t* first = dim == 3 ? w->first : nullptr;
   for (;;) {
     const HalfList H{w->hf, w->first, &w->told->used, w->cap_hf};
     if (dim == 3) {
@@ -1690,8 +1688,8 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
     if (!hf_room(more)) return rc;
     cu(cudaMemsetAsync(w->told, 0, sizeof(TessCount), st), "memset");
   }
-  k_keep_count<<<nbf, 256, 0, st>>>((int)n, dim, w->hf, w->first, w->nhf, w->keep);
-  if ((dim == 3 ? (int64_t)told.used : 32 * n) > INT32_MAX) {   // (faces are half-faces or fewer)
+  k_keep_count<<<nbf, 256, 0, st>>>((int)n, dim, w->hf, first, w->nhf, w->keep);
+  if ((dim == 3 ? (int64_t)told.used : HF2 * n) > INT32_MAX) {   // (faces are half-faces or fewer)
     cu(cudaMemsetAsync(&w->told->used, 0, sizeof told.used, st), "memset");
     k_keep_total<<<152 * 8, 256, 0, st>>>((int)n, w->keep, &w->told->used);
     cu(cudaMemcpyAsync(&told, w->told, sizeof told, cudaMemcpyDeviceToHost, st), "read");
@@ -1727,9 +1725,9 @@ int tess_build_work(TessWork* w, int dim, int64_t n, const double* gen_d, const 
     }
     w->cap_f = cap;
   }
-  k_emit<<<nbf, 256, 0, st>>>((int)n, dim, gen_d, w->hf, w->first, w->nhf, w->off, w->cells, w->shift, w->area,
+  k_emit<<<nbf, 256, 0, st>>>((int)n, dim, gen_d, w->hf, first, w->nhf, w->off, w->cells, w->shift, w->area,
                                 w->cen);
-  if (check) k_mirror<<<nbf, 256, 0, st>>>((int)n, dim, w->hf, w->first, w->nhf, w->chk, w->chk + 1);
+  if (check) k_mirror<<<nbf, 256, 0, st>>>((int)n, dim, w->hf, first, w->nhf, w->chk, w->chk + 1);
   cu(cudaGetLastError(), "faces");
   unsigned long long h[2] = {0, 0};
   if (check) cu(cudaMemcpyAsync(h, w->chk, sizeof h, cudaMemcpyDeviceToHost, st), "read");
