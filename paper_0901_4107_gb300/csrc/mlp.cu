@@ -11,6 +11,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -590,13 +591,31 @@ int mfail(amm_mlp* m, int code, const std::string& msg) {
 size_t mlp_smem_bytes() { return sizeof(amm::MlpSmem) + 1024; }
 size_t train_smem_bytes() { return sizeof(amm::TrainSmem) + 1024; }
 
+// Clears the arrays before it returns.  (cudaMemset runs on the legacy stream, which a
+// non-blocking stream of the handle is not ordered after: behind other work there the
+// clear could land on weights already set.  On the handle's stream it would be taken
+// into a graph that the caller captures.)
+struct Cleared {
+  void* p;
+  size_t bytes;
+};
+cudaError_t clear_now(std::initializer_list<Cleared> arrays) {
+  cudaStream_t st = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  for (const Cleared& a : arrays)
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.p, 0, a.bytes, st);
+  const cudaError_t w = cudaStreamSynchronize(st);
+  cudaStreamDestroy(st);
+  return e != cudaSuccess ? e : w;
+}
+
 int ensure_train(amm_mlp* m, int ctas) {
   if (!m->adam_m) {
     MCU(cudaMalloc(&m->adam_m, sizeof(float) * amm::NPARAMS));
     MCU(cudaMalloc(&m->adam_v, sizeof(float) * amm::NPARAMS));
     MCU(cudaMalloc(&m->grads, sizeof(float) * (amm::NPARAMS + 1)));
-    MCU(cudaMemset(m->adam_m, 0, sizeof(float) * amm::NPARAMS));
-    MCU(cudaMemset(m->adam_v, 0, sizeof(float) * amm::NPARAMS));
+    MCU(clear_now({{m->adam_m, sizeof(float) * amm::NPARAMS}, {m->adam_v, sizeof(float) * amm::NPARAMS}}));
   }
   if (m->partial_ctas < ctas) {
     if (m->partial) cudaFree(m->partial);
@@ -651,9 +670,9 @@ int amm_mlp_create(amm_mlp** out, double gamma, void* stream) {
   if (cudaMalloc(&m->params, sizeof(float) * amm::NPARAMS) != cudaSuccess) return bail(AMM_ERR_CUDA);
   if (cudaMalloc(&m->packed, sizeof(amm::MlpDevice)) != cudaSuccess) return bail(AMM_ERR_CUDA);
   if (cudaMalloc(&m->status, sizeof(unsigned)) != cudaSuccess) return bail(AMM_ERR_CUDA);
-  if (cudaMemset(m->params, 0, sizeof(float) * amm::NPARAMS) != cudaSuccess) return bail(AMM_ERR_CUDA);
-  if (cudaMemset(m->packed, 0, sizeof(amm::MlpDevice)) != cudaSuccess) return bail(AMM_ERR_CUDA);
-  if (cudaMemset(m->status, 0, sizeof(unsigned)) != cudaSuccess) return bail(AMM_ERR_CUDA);
+  if (clear_now({{m->params, sizeof(float) * amm::NPARAMS}, {m->packed, sizeof(amm::MlpDevice)}, {m->status, sizeof(unsigned)}}) !=
+      cudaSuccess)
+    return bail(AMM_ERR_CUDA);
   if (cudaFuncSetAttribute(amm::k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem_bytes()) !=
       cudaSuccess)
     return bail(AMM_ERR_CUDA);
