@@ -763,7 +763,9 @@ static int individual_setup(amm_ctx* c) {
   const int leaves = 1 << (dim * L);
   const int side = 1 << L;
   std::vector<double> g((size_t)n * 3);
-  CU(cudaMemcpy(g.data(), c->gen, sizeof(double) * g.size(), cudaMemcpyDeviceToHost));
+  // (on the context's stream throughout: the legacy one is not ordered with it)
+  CU(cudaMemcpyAsync(g.data(), c->gen, sizeof(double) * g.size(), cudaMemcpyDeviceToHost, c->stream));
+  CU(cudaStreamSynchronize(c->stream));
   std::vector<int> bucket((size_t)n), off((size_t)leaves + 1, 0), cell_slot((size_t)n);
   for (int64_t i = 0; i < n; i++) {
     int ib[3] = {0, 0, 0};
@@ -797,12 +799,13 @@ static int individual_setup(amm_ctx* c) {
   CU(dalloc((float4**)&c->ind_rec32, 2 * (size_t)n));
   CU(dalloc(&c->ind_loop, 1));
   CU(dalloc((float2**)&c->ind_node, (size_t)c->ind_level_off_h[c->ind_levels]));
-  CU(cudaMemcpy(c->ind_cell_slot, cell_slot.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->ind_leaf_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->ind_level_off, c->ind_level_off_h.data(), sizeof(int) * c->ind_level_off_h.size(),
-                cudaMemcpyHostToDevice));
-  CU(cudaMemset(c->ind_fstamp, 0xff, sizeof(int) * c->nf_cap));
-  CU(cudaMemset(c->ind_cstamp, 0xff, sizeof(int) * n));
+  CU(cudaMemcpyAsync(c->ind_cell_slot, cell_slot.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
+  CU(cudaMemcpyAsync(c->ind_leaf_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, c->stream));
+  CU(cudaMemcpyAsync(c->ind_level_off, c->ind_level_off_h.data(), sizeof(int) * c->ind_level_off_h.size(),
+                     cudaMemcpyHostToDevice, c->stream));
+  CU(cudaMemsetAsync(c->ind_fstamp, 0xff, sizeof(int) * c->nf_cap, c->stream));
+  CU(cudaMemsetAsync(c->ind_cstamp, 0xff, sizeof(int) * n, c->stream));
+  CU(cudaStreamSynchronize(c->stream));   // the host arrays go out of scope
   c->ind_stamp = 0;
   c->ind_ready = true;
   return AMM_OK;
