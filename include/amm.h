@@ -336,7 +336,8 @@ int amm_get_kernel_times(amm_ctx* ctx, float* ms);
 
 /* Launch shapes.  grad_lanes / update_lanes: consecutive threads that share
  * one cell in the gradient and update kernels (1, 2, 4 or 8); flux_block:
- * faces (threads) per CTA of the flux kernel (128 or 256).  Results do not
+ * faces (threads) per CTA of the flux kernel (128 or 256; in the FP64 form
+ * also 64, the default of meshes of up to 152 * 1024 faces).  Results do not
  * depend on them except for the FP64 rounding order of sums. */
 typedef struct amm_tuning {
   int grad_lanes;

@@ -79,13 +79,18 @@ void free_ctx(amm_ctx* c) {
 //    13.8 k       86 / 29        60 / 20        67 / 21        76 / 18
 //    33 k         86 / 29       102 / 28       118 / 35       150 / 41
 //    91 k        208 / 68       217 / 59       264 / 76       374 / 92
-void default_lanes(amm_ctx* c) {
+// The FP64 flux kernel: few faces go to CTAs of 64, which spread them over all SMs'
+// FP64 pipes in the faces' own order; many to CTAs of 256, which group the solves by
+// kind.  (us for faces, 64 / 256: 25 k 27 / 35, 98 k 55 / 69 in 2D and 98 / 102 in 3D,
+// 230 k 182 / 178, 715 k 471 / 445.)
+void default_shapes(amm_ctx* c) {
   const int64_t few = 40000;   // threads below which more lanes still pay (two warps for each of the chip's 608 FP64 pipes)
   c->update_lanes = 8 * c->n <= few ? 8 : (4 * c->n <= few ? 4 : 2);
   if (c->is_fp64())
     c->grad_lanes = 4 * c->n <= few ? 4 : (2 * c->n <= few ? 2 : 1);
   else
     c->grad_lanes = c->n <= 300000 ? 4 : 2;
+  c->flux_block = c->is_fp64() && c->nf <= 152 * 1024 ? 64 : 256;
 }
 
 template <typename F64, typename F32>
@@ -268,7 +273,7 @@ int amm_create(amm_ctx** out, int dim, int64_t n, const double* gen, int64_t nf,
   c->box_cells = bc;
   c->box_faces = bf;
   c->nf_cap = nf;
-  default_lanes(c);
+  default_shapes(c);
   int dev = 0;
   cudaError_t e0 = cudaGetDevice(&dev);
   if (e0 != cudaSuccess) {
@@ -1163,7 +1168,8 @@ int amm_get_kernel_times(amm_ctx* c, float* ms) {
 int amm_set_tuning(amm_ctx* c, const amm_tuning* t) {
   if (!c || !t) return fail(c, AMM_ERR_INVALID_ARG, "null argument");
   auto ok_lanes = [](int g) { return g == 1 || g == 2 || g == 4 || g == 8; };
-  if (!ok_lanes(t->grad_lanes) || !ok_lanes(t->update_lanes) || (t->flux_block != 128 && t->flux_block != 256))
+  if (!ok_lanes(t->grad_lanes) || !ok_lanes(t->update_lanes) ||
+      (t->flux_block != 128 && t->flux_block != 256 && !(t->flux_block == 64 && c->is_fp64())))
     return fail(c, AMM_ERR_INVALID_ARG, "tuning values out of range");
   if (t->persistent != 0 && t->persistent != 1) return fail(c, AMM_ERR_INVALID_ARG, "persistent must be 0 or 1");
   c->grad_lanes = t->grad_lanes;
@@ -1199,11 +1205,12 @@ int amm_autotune(amm_ctx* c, double cfl, int reps, amm_tuning* out) {
   const bool prof = c->profiling;
   int rc = amm_profile(c, 1);
   static const int lanes[4] = {1, 2, 4, 8};
-  static const int blocks[2] = {128, 256};
+  static const int blocks32[4] = {128, 256, 128, 256}, blocks64[4] = {64, 128, 256, 64};
+  const int* blocks = c->is_fp64() ? blocks64 : blocks32;
   float best[3] = {1e30f, 1e30f, 1e30f};
   int pick[3] = {c->grad_lanes, c->update_lanes, c->flux_block};
   for (int v = 0; v < 4 && rc == AMM_OK; v++) {
-    amm_tuning t{lanes[v], lanes[v], blocks[v % 2], 0, 0.f};
+    amm_tuning t{lanes[v], lanes[v], blocks[v], 0, 0.f};
     rc = amm_set_tuning(c, &t);
     std::vector<float> g, f, u;
     for (int r = 0; r < reps + 1 && rc == AMM_OK; r++) {
@@ -1237,7 +1244,7 @@ int amm_autotune(amm_ctx* c, double cfl, int reps, amm_tuning* out) {
     const float mg = med(g), mf = med(f), mu = med(u);
     if (mg < best[0]) { best[0] = mg; pick[0] = lanes[v]; }
     if (mu < best[2]) { best[2] = mu; pick[1] = lanes[v]; }
-    if (mf < best[1]) { best[1] = mf; pick[2] = blocks[v % 2]; }
+    if (mf < best[1]) { best[1] = mf; pick[2] = blocks[v]; }
   }
   cudaMemcpyAsync(c->Q, saved, sizeof(double) * qn, cudaMemcpyDeviceToDevice, c->stream);
   dispatch(c, [&] { return amm::launch_primitives<double>(c); }, [&] { return amm::launch_primitives<float>(c); });

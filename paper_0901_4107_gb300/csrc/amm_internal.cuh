@@ -287,7 +287,7 @@ struct amm_ctx {
   int headroom = 7;
   int grad_lanes = 4;              // lanes per cell in the gradient kernel (amm_create's rule, amm_set_tuning)
   int update_lanes = 2;            // lanes per cell in the update kernel (likewise)
-  int flux_block = 256;            // threads (faces) per CTA of the flux kernel
+  int flux_block = 256;            // threads (faces) per CTA of the flux kernel (likewise)
   float tuned_ms = 0.f;
   int persistent = 0;              // 1: one cooperative launch per step (amm_advance)
   unsigned* barrier = nullptr;     // grid-barrier counter and generation

@@ -1764,14 +1764,11 @@ cudaError_t launch_flux(amm_ctx* c, double cfl) {
     return launch_flux_chunks(c, v, false, FluxDefer());
   } else {
     const bool ent = c->opt.entropy != 0;
-    // Few faces: CTAs of 64 spread them over all SMs' FP64 pipes, in the faces' own
-    // order; many: CTAs of 256, which group the solves by kind.  (us for faces, 64
-    // / 256: 25 k 27 / 35, 98 k 55 / 69 in 2D and 98 / 102 in 3D, 230 k 182 / 178,
-    // 715 k 471 / 445.)
-    const bool few = c->nf <= 152 * 1024;
-    if (few && ent)
+    // (the default by the number of faces: default_shapes)
+    const bool b64 = c->flux_block == 64;
+    if (b64 && ent)
       k_flux<real, 64, true><<<c->n_ftiles * 4, 64, 0, c->stream>>>(v);
-    else if (few)
+    else if (b64)
       k_flux<real, 64, false><<<c->n_ftiles * 4, 64, 0, c->stream>>>(v);
     else if (b128 && ent)
       k_flux<real, 128, true><<<c->n_ftiles * 2, 128, 0, c->stream>>>(v);
