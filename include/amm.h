@@ -338,7 +338,9 @@ int amm_get_kernel_times(amm_ctx* ctx, float* ms);
  * one cell in the gradient and update kernels (1, 2, 4 or 8); flux_block:
  * faces (threads) per CTA of the flux kernel (128 or 256; in the FP64 form
  * also 64, the default of meshes of up to 152 * 1024 faces).  Results do not
- * depend on them except for the FP64 rounding order of sums. */
+ * depend on them except for the rounding order of sums: of a cell's fluxes in
+ * the FP64 form (the FP32 forms' are exact) and of its gradient, in the form's
+ * precision.  The defaults depend on the context's size. */
 typedef struct amm_tuning {
   int grad_lanes;
   int update_lanes;

@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(CELL_TILE) k_step_persistent_learned(HydroView
     learned_faces<PL_H, ENT>(v, s, tile, tile.begin, phase);
   }
   grid_barrier(bar, bar + 1, gridDim.x, &v.stats->status);
-  for (int wi = blockIdx.x; wi < v.n_ctiles; wi += gridDim.x) update_item<float, 1, ENT>(v, wi);
+  for (int wi = blockIdx.x; wi < v.n_ctiles; wi += gridDim.x) update_item<float, 1, ENT, true>(v, wi);
   grid_barrier(bar, bar + 1, gridDim.x, &v.stats->status);
   for (int b = blockIdx.x; b < v.nboxes; b += gridDim.x) finish_item<float, CELL_TILE>(v, b, 1);
   learned_teardown<PL_H>(v, s);

@@ -1128,6 +1128,9 @@ __device__ __forceinline__ void finish_barrier() {
     __syncwarp();
 }
 
+// barrier of all threads of a CTA that its warps reach at different places
+__device__ __forceinline__ void item_barrier() { asm volatile("bar.sync 2, %0;" ::"n"(CELL_TILE) : "memory"); }
+
 constexpr int UPD_BATCH = 2;
 static_assert(FIX_RUN % UPD_BATCH == 0, "a run is whole batches");
 // G consecutive lanes share a cell (as in the gradient kernel); lane l sums
@@ -1145,8 +1148,9 @@ static_assert(FIX_RUN % UPD_BATCH == 0, "a run is whole batches");
 // conversions (1 lane 212, 4 lanes 233); 348 k cells with the entropy switch: 111 us,
 // 86 without FP64 conversions and divisions.  ENT: the entropy switch of
 // Sec. 3.5 (a sixth flux component, the entropy, and the per-cell choice
-// between the advected entropy and the energy update).
-template <typename real, int G, bool ENT = false>
+// between the advected entropy and the energy update).  LOOP: the CTA goes on to
+// another item (the shared memory is reused).
+template <typename real, int G, bool ENT = false, bool LOOP = false>
 __device__ __forceinline__ void update_item(const HydroView<real>& v, int wi) {
   constexpr int CELLS = CELL_TILE / G;
   constexpr int NA = ENT ? 6 : 5;
@@ -1296,7 +1300,10 @@ __device__ __forceinline__ void update_item(const HydroView<real>& v, int wi) {
       s_bad[tid / G] = bad;
     }
     __syncthreads();
-    if (tid >= CELLS) return;
+    if (tid >= CELLS) {
+      if constexpr (LOOP) item_barrier();
+      return;
+    }
 #pragma unroll
     for (int a = 0; a < NA; a++) d[a] = s_d[a][tid];
     if constexpr (ENT) mach = s_mach[tid];
@@ -1401,8 +1408,7 @@ __device__ __forceinline__ void update_item(const HydroView<real>& v, int wi) {
       if (nkeep) atomicAdd(&v.stats->kept, (unsigned long long)nkeep);
     }
   }
-  // (a persistent CTA, G == 1, goes on to its next work item)
-  if constexpr (G == 1) __syncthreads();
+  if constexpr (LOOP) item_barrier();
 }
 
 template <typename real, int G, bool ENT>
