@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "amm.h"
+#include "face_walk.cuh"
 #include "half_list.cuh"
 #include "scan.cuh"
 
@@ -881,7 +882,7 @@ __global__ void __launch_bounds__(32 * FWARPS, 5) k_cells3_fast(const __grid_con
           open |= (V.tri[e] & 255) < 6 || ((V.tri[e] >> 8) & 255) < 6 || ((V.tri[e] >> 16) & 255) < 6;
       if (__any_sync(full, open)) rc = -1;
     }
-    int nf = 0;
+    int nf = 0, walked = 0;
     double sum[4] = {0.0, 0.0, 0.0, 0.0};   // volume, first moment
     __syncwarp();
     if (rc == 0) {
@@ -930,6 +931,7 @@ __global__ void __launch_bounds__(32 * FWARPS, 5) k_cells3_fast(const __grid_con
         const int k = k0 + lane;
         double area = 0.0, fc[3] = {0.0, 0.0, 0.0};
         bool keep = false;
+        int met = 0;
         const int t0 = k < np ? S.u.f.start[k] : 64;
         if (t0 < 64) {
           const double* pk = S.u.f.P[k];
@@ -938,36 +940,20 @@ __global__ void __launch_bounds__(32 * FWARPS, 5) k_cells3_fast(const __grid_con
           const int cu = ax == 2 ? 0 : ax + 1, cv = ax == 0 ? 2 : ax - 1;
           const double ou = S.u.f.v[t0][cu], ov = S.u.f.v[t0][cv];
           double e1u = 0.0, e1v = 0.0, A = 0.0, Cu = 0.0, Cv = 0.0;
-          int t = t0, m = 0;
-          bool ok = true;
-          for (;;) {
-            // the vertex (k, x, y): its successor on the face is (k, y, .)
-            const unsigned tr = S.u.f.tri[t];
-            const int p0 = tr & 255, p1 = (tr >> 8) & 255, p2 = (tr >> 16) & 255;
-            const int y = p0 == k ? p2 : (p1 == k ? p0 : p1);
-            m++;
-            const int tn = S.u.f.next[k][y];
-            if (tn == t0) break;
-            // the table is not cleared: check that this entry is of this cell
-            bool good = m < MAXFV && tn < 64 && (((tn < 32 ? L[0] : L[1]) >> (tn & 31)) & 1u);
-            if (good) {
-              const unsigned tq = S.u.f.tri[tn];
-              const int g0 = tq & 255, g1 = (tq >> 8) & 255, g2 = (tq >> 16) & 255;
-              good = (g0 == k && g1 == y) || (g1 == k && g2 == y) || (g2 == k && g0 == y);
-            }
-            if (!good) {
-              ok = false;
-              break;
-            }
-            const double e2u = S.u.f.v[tn][cu] - ou, e2v = S.u.f.v[tn][cv] - ov;
-            const double at = e1u * e2v - e1v * e2u;
-            A += at;
-            Cu += at * (e1u + e2u);
-            Cv += at * (e1v + e2v);
-            e1u = e2u;
-            e1v = e2v;
-            t = tn;
-          }
+          const int m = walk_face(
+              k, t0, S.u.f.tri, S.u.f.next, MAXFV,
+              [&](int tn) { return tn < 64 && (((tn < 32 ? L[0] : L[1]) >> (tn & 31)) & 1u); },
+              [&](int tn) {
+                const double e2u = S.u.f.v[tn][cu] - ou, e2v = S.u.f.v[tn][cv] - ov;
+                const double at = e1u * e2v - e1v * e2u;
+                A += at;
+                Cu += at * (e1u + e2u);
+                Cv += at * (e1v + e2v);
+                e1u = e2u;
+                e1v = e2v;
+              });
+          met = m;
+          const bool ok = m > 0;
           if (!ok) rc = -1;
           if (ok && m >= 3) {
             // one division for both 1 / n_ax and 1 / (3 A)
@@ -1004,8 +990,11 @@ __global__ void __launch_bounds__(32 * FWARPS, 5) k_cells3_fast(const __grid_con
           }
         }
         nf += __popc(km);
+        walked += __reduce_add_sync(full, met);
       }
       if (__any_sync(full, rc != 0)) rc = -1;
+      // (a pinched cell: k_cells3 decides)
+      if (!walks_complete(walked, __popc(L[0]) + __popc(L[1]))) rc = -1;
       if (nf > MAXHF) rc = -1;
     }
     // the four sums over the lanes: two levels that halve the components a
