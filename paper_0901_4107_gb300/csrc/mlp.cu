@@ -237,9 +237,26 @@ __device__ __forceinline__ void tr_store32(uint8_t* tile, int t, int c0, int K, 
   for (int q = 0; q < 4; q++) tc::st_bf16x8(tile, tc::kmajor_offset(t, c0 + 8 * q, K), v + 8 * q);
 }
 
-// the logistic function from the hardware's exponential and reciprocal (each
-// good to a few ulp)
-__device__ __forceinline__ float logistic(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
+// the larger; a NaN if either is one
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+  return m;
+}
+
+// silu(z) = z / q with q = 1 + exp(-z), and its derivative s (1 + z (1 - s)), s = 1 / q.
+// The hardware's reciprocal (good to an ulp) and the product z s are corrected with their
+// remainders, which leaves both quotients the nearest floats but for rare ties: 4
+// multiply-adds.  A step of 2^20 samples: 182 us; 162 with neither corrected, at a quarter
+// more error of the output weights' gradients than rounded divisions have, which take 252.
+// Below -87 (where both are under 2e-36) z is held there: exp(87) keeps 1 / q normal.
+__device__ __forceinline__ void silu_both(float zz, float& h, float& d) {
+  const float z = max_nan(zz, -87.0f);
+  const float q = 1.0f + __expf(-z), r = approx_rcp(q);
+  const float s = __fmaf_rn(__fmaf_rn(-q, r, 1.0f), r, r), a = z * s;
+  h = __fmaf_rn(__fmaf_rn(-a, q, z), s, a);
+  d = s * __fmaf_rn(z, 1.0f - s, 1.0f);
+}
 
 // Gradient of L = sum over the batch of (y - t)^2 / n_total with respect to
 // every parameter; each CTA processes tiles blockIdx.x, blockIdx.x+gridDim.x,
@@ -318,9 +335,7 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_mlp_grads(const MlpDevice* M,
       tc::tmem_ld32(tc::tmem_lane_addr(tm, quad, TC_Z1 + c0), z);
 #pragma unroll
       for (int j = 0; j < 32; j++) {
-        const float zz = z[j] + s.bias1[c0 + j], sg = logistic(zz), h = zz * sg;
-        d1[j] = sg + h * (1.0f - sg);
-        z[j] = h;
+        silu_both(z[j] + s.bias1[c0 + j], z[j], d1[j]);
       }
       tr_store32(s.hx, row, c0, TR_HX, z);
     }
@@ -340,9 +355,9 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_mlp_grads(const MlpDevice* M,
       float y = 0.0f;
 #pragma unroll
       for (int j = 0; j < 32; j++) {
-        const float zz = h2[j] + s.bias2[c0 + j], sg = logistic(zz), w = s.w3[c0 + j];
-        h2[j] = zz * sg;
-        d2[j] = w * (sg + h2[j] * (1.0f - sg));
+        const float w = s.w3[c0 + j];
+        silu_both(h2[j] + s.bias2[c0 + j], h2[j], d2[j]);
+        d2[j] *= w;
         y += w * h2[j];
       }
       s.ysum[half][row] = y;
