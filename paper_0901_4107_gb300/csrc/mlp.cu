@@ -11,7 +11,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -579,6 +578,7 @@ __global__ void k_mlp_targets(double gamma, int64_t m, const float* st, double t
 struct amm_mlp {
   double gamma = 5.0 / 3.0;
   cudaStream_t stream = nullptr;
+  char* block = nullptr;              // holds the arrays below but `partial`
   float* params = nullptr;            // FP32 master parameters [NPARAMS]
   amm::MlpDevice* packed = nullptr;   // BF16 weights for the kernels
   unsigned* status = nullptr;
@@ -606,32 +606,37 @@ int mfail(amm_mlp* m, int code, const std::string& msg) {
 size_t mlp_smem_bytes() { return sizeof(amm::MlpSmem) + 1024; }
 size_t train_smem_bytes() { return sizeof(amm::TrainSmem) + 1024; }
 
-// Clears the arrays before it returns.  (cudaMemset runs on the legacy stream, which a
-// non-blocking stream of the handle is not ordered after: behind other work there the
-// clear could land on weights already set.  On the handle's stream it would be taken
-// into a graph that the caller captures.)
-struct Cleared {
-  void* p;
-  size_t bytes;
-};
-cudaError_t clear_now(std::initializer_list<Cleared> arrays) {
-  cudaStream_t st = nullptr;
-  cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+// Allocates the handle's arrays, all in one block, and clears them before it returns.
+// (cudaMemset runs on the legacy stream, which a non-blocking stream of the handle is not
+// ordered after: behind other work there the clear could land on weights already set.  On
+// the handle's stream it would be taken into a graph that the caller captures.)
+cudaError_t alloc_cleared(amm_mlp* m) {
+  size_t bytes = 0;
+  const auto part = [&](size_t b) {
+    const size_t at = bytes;
+    bytes += (b + 255) / 256 * 256;
+    return at;
+  };
+  const size_t np = sizeof(float) * (amm::NPARAMS + 1);
+  const size_t packed = part(sizeof(amm::MlpDevice)), params = part(np), adam_m = part(np), adam_v = part(np), grads = part(np),
+               status = part(sizeof(unsigned));
+  cudaError_t e = cudaMalloc(&m->block, bytes);
   if (e != cudaSuccess) return e;
-  for (const Cleared& a : arrays)
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.p, 0, a.bytes, st);
+  cudaStream_t st = nullptr;
+  if ((e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking)) != cudaSuccess) return e;
+  e = cudaMemsetAsync(m->block, 0, bytes, st);
   const cudaError_t w = cudaStreamSynchronize(st);
   cudaStreamDestroy(st);
+  m->packed = reinterpret_cast<amm::MlpDevice*>(m->block + packed);
+  m->params = reinterpret_cast<float*>(m->block + params);
+  m->adam_m = reinterpret_cast<float*>(m->block + adam_m);
+  m->adam_v = reinterpret_cast<float*>(m->block + adam_v);
+  m->grads = reinterpret_cast<float*>(m->block + grads);
+  m->status = reinterpret_cast<unsigned*>(m->block + status);
   return e != cudaSuccess ? e : w;
 }
 
 int ensure_train(amm_mlp* m, int ctas) {
-  if (!m->adam_m) {
-    MCU(cudaMalloc(&m->adam_m, sizeof(float) * amm::NPARAMS));
-    MCU(cudaMalloc(&m->adam_v, sizeof(float) * amm::NPARAMS));
-    MCU(cudaMalloc(&m->grads, sizeof(float) * (amm::NPARAMS + 1)));
-    MCU(clear_now({{m->adam_m, sizeof(float) * amm::NPARAMS}, {m->adam_v, sizeof(float) * amm::NPARAMS}}));
-  }
   if (m->partial_ctas < ctas) {
     if (m->partial) cudaFree(m->partial);
     m->partial = nullptr;
@@ -676,18 +681,11 @@ int amm_mlp_create(amm_mlp** out, double gamma, void* stream) {
   m->gamma = gamma;
   m->stream = (cudaStream_t)stream;
   auto bail = [&](int rc) {
-    if (m->params) cudaFree(m->params);
-    if (m->packed) cudaFree(m->packed);
-    if (m->status) cudaFree(m->status);
+    if (m->block) cudaFree(m->block);
     delete m;
     return rc;
   };
-  if (cudaMalloc(&m->params, sizeof(float) * amm::NPARAMS) != cudaSuccess) return bail(AMM_ERR_CUDA);
-  if (cudaMalloc(&m->packed, sizeof(amm::MlpDevice)) != cudaSuccess) return bail(AMM_ERR_CUDA);
-  if (cudaMalloc(&m->status, sizeof(unsigned)) != cudaSuccess) return bail(AMM_ERR_CUDA);
-  if (clear_now({{m->params, sizeof(float) * amm::NPARAMS}, {m->packed, sizeof(amm::MlpDevice)}, {m->status, sizeof(unsigned)}}) !=
-      cudaSuccess)
-    return bail(AMM_ERR_CUDA);
+  if (alloc_cleared(m) != cudaSuccess) return bail(AMM_ERR_CUDA);
   if (cudaFuncSetAttribute(amm::k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem_bytes()) !=
       cudaSuccess)
     return bail(AMM_ERR_CUDA);
@@ -701,7 +699,7 @@ int amm_mlp_create(amm_mlp** out, double gamma, void* stream) {
 void amm_mlp_destroy(amm_mlp* m) {
   if (!m) return;
   cudaStreamSynchronize(m->stream);
-  void* ptrs[] = {m->params, m->packed, m->status, m->adam_m, m->adam_v, m->grads, m->partial};
+  void* ptrs[] = {m->block, m->partial};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete m;
