@@ -6,9 +6,10 @@
 // 64 x 64-bit product's upper half (about eight instructions) is several times
 // cheaper than one FP64 multiply-add, and a division, square root or power is
 // some 10, 10 and 26 of those.  The operands' significands become 64-bit fixed-point
-// numbers (Qn: n fractional bits), the arithmetic below keeps about 60 bits, and the
-// result is rounded to nearest once: at most 0.53 ulp against 80-bit references
-// (CUDA documents 0.5, 0.5, 1 and 1 for its division, sqrt, rsqrt and pow).
+// numbers (Qn: n fractional bits), and the arithmetic below keeps about 60 bits.
+// Reciprocal, quotient and square root are then rounded by their exact remainders, so
+// they are the bits of the divisions and roots of IEEE 754; x^(-1/2) and x^a are rounded
+// from the 60 bits, to at most 0.52 and 0.59 ulp (CUDA documents 1 and 1).
 // Every value is the same in every kernel that inlines these.  Arguments outside
 // the ranges stated (zero, negative, infinite, NaN, extreme exponents) go to
 // CUDA's own functions.
@@ -74,12 +75,21 @@ __device__ __forceinline__ unsigned exponent_bits(int hi) { return ((unsigned)hi
 // the exponent field of an argument lies within 2^+-900
 __device__ __forceinline__ bool common(unsigned e) { return e - 123u < 1801u; }
 
+// Rounding by the remainder: the quotient's 53 bits are cut off a little below it (by
+// BELOW of its last places, more than its error), so that the integer R is at most it and
+// less than 1.5 short of it, and the remainder N - R D, which fits 64 bits and so needs
+// only the products' lower halves, tells whether R or R + 1 is the nearest.
+constexpr u64 BELOW = 8;
+
 // 1 / x, x of either sign
 __device__ __forceinline__ double recip64(double x) {
   const int h = __double2hiint(x);
   const unsigned e = exponent_bits(h);
   if (!common(e)) return div64_rare(1.0, x);
-  const u64 r = (recip_q61(significand(x)) + 128) >> 8;
+  const u64 m = significand(x);
+  u64 r = (recip_q61(m) - BELOW) >> 8;                                      // 2^105 / m
+  const i64 rem = (i64)(0 - r * m);
+  r += 2 * rem > (i64)m ? 1 : 0;
   return __longlong_as_double((i64)(((u64)(2044 - e) << 52) + r) | ((i64)h & 0x80000000ll) << 32);
 }
 
@@ -88,9 +98,12 @@ __device__ __forceinline__ double div64(double a, double b) {
   const int ha = __double2hiint(a), hb = __double2hiint(b);
   const unsigned ea = exponent_bits(ha), eb = exponent_bits(hb);
   if (!(common(ea) && common(eb) && ea - eb + 900u < 1801u)) return div64_rare(a, b);
-  const u64 q = __umul64hi(significand(a) << 11, recip_q61(significand(b)));   // in (1/2, 2), Q60
+  const u64 ma = significand(a), mb = significand(b);
+  const u64 q = __umul64hi(ma << 11, recip_q61(mb));                        // in (1/2, 2), Q60
   const bool low = q < (1ull << 60);
-  const u64 r = low ? (q + 64) >> 7 : (q + 128) >> 8;
+  u64 r = (q - BELOW) >> (low ? 7 : 8);                                     // 2^53 ma / mb or half that
+  const i64 rem = (i64)((ma << (low ? 53 : 52)) - r * mb);
+  r += 2 * rem > (i64)mb ? 1 : 0;
   return __longlong_as_double((i64)(((u64)(1022 + ea - eb - (low ? 1u : 0u)) << 52) + r) |
                               ((i64)(ha ^ hb) & 0x80000000ll) << 32);
 }
@@ -125,7 +138,9 @@ __device__ __forceinline__ double sqrt64(double x) {
   const RootArg a = root_arg(x);
   if (!a.ok) return __double_as_longlong(x) == 0ll ? 0.0 : sqrt64_rare(x);
   const u64 s = __umul64hi(a.m, rsqrt_q61(a.m, a.f));                       // in [1, 2], Q59
-  const u64 r = (s + 64) >> 7;
+  u64 r = (s - BELOW) >> 7;
+  const i64 rem = (i64)((a.m << 42) - r * r);                               // (r + 1/2)^2 = r^2 + r + 1/4
+  r += rem > (i64)r ? 1 : 0;
   return __longlong_as_double((i64)(((u64)(1022 + a.half) << 52) + r));
 }
 
