@@ -94,7 +94,8 @@ struct GasC {
   real fan_rho;      // 2/(g-1)
   real fan_p;        // 2g/(g-1)
   real inv_gm1;      // 1/(g-1)
-  real sqrt_two_gp1, isqrt_two_gp1;   // (2/(g+1))^(+-1/2)
+  real half_gp1;     // (g+1)/2
+  real isqrt_two_gp1;   // its square root
   GasC() = default;
   __host__ __device__ explicit GasC(double gamma) {
     g = (real)gamma;
@@ -111,7 +112,7 @@ struct GasC {
     fan_rho = (real)(2.0 / (gamma - 1.0));
     fan_p = (real)(2.0 * gamma / (gamma - 1.0));
     inv_gm1 = (real)(1.0 / (gamma - 1.0));
-    sqrt_two_gp1 = (real)sqrt(2.0 / (gamma + 1.0));
+    half_gp1 = (real)(0.5 * (gamma + 1.0));
     isqrt_two_gp1 = (real)sqrt(0.5 * (gamma + 1.0));
   }
 };

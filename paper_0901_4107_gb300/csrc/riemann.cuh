@@ -111,19 +111,20 @@ __device__ __forceinline__ void wave_curve(float p, float rhoK, float pK, float 
   }
 }
 
-// FP64: f_K(p) and f_K'(p).  The shock takes one reciprocal square root,
-// w = (rho (p + B))^(-1/2): q = sqrt(2/(gamma+1)) w and 1/(p + B) = rho w^2; the
-// rarefaction f' = (p/p_K)^z c_K / (gamma p) (rho_K c_K = gamma p_K / c_K), with
-// 1/p given (both sides need it) and 1/p_K formed once per solve.
+// FP64: f_K(p) and f_K'(p).  The shock takes one reciprocal square root, with h =
+// rho (gamma+1)/2: q = (h (p + B))^(-1/2), whose roundings (h, p + B, their product,
+// halved, and the root's) are no more than those of sqrt(A / (p + B)), and 1/(p + B) =
+// h q^2 for the slope; the rarefaction f' = (p/p_K)^z c_K / (gamma p) (rho_K c_K =
+// gamma p_K / c_K), with 1/p given (both sides need it).  The slopes only steer Newton's
+// iteration; the values are rounded as the formulas' own quotients and powers.
 // (explicitly rounded: the persistent step kernel must round alike)
 struct WaveSide {
-  double rho, p, ip, B, two_c, c_g;   // state, 1/p, B, 2c/(gamma-1), c/gamma
+  double h, p, B, two_c, c_g;   // (gamma+1)/2 rho, p, B, 2c/(gamma-1), c/gamma
 };
 __device__ __forceinline__ WaveSide wave_side(double rho, double p, double c, const GasC<double>& G) {
   WaveSide s;
-  s.rho = rho;
+  s.h = rn_mul(G.half_gp1, rho);
   s.p = p;
-  s.ip = recip64(p);
   s.B = rn_mul(G.gm1_gp1, p);
   s.two_c = rn_mul(G.two_gm1, c);
   s.c_g = rn_mul(c, G.inv_g);
@@ -133,15 +134,12 @@ __device__ __forceinline__ void wave_curve(double p, double ip, const WaveSide& 
                                            double& df) {
   const double d = rn_add(p, -K.p);
   if (positive(d)) {
-    const double w = rsqrt64(rn_mul(K.rho, rn_add(p, K.B)));
-    const double q = rn_mul(G.sqrt_two_gp1, w);
-    const double h = rn_mul(rn_mul(w, w), K.rho);
-    const double dh = rn_mul(d, h);
+    const double q = rsqrt64(rn_mul(K.h, rn_add(p, K.B)));
+    const double dh = rn_mul(d, rn_mul(rn_mul(q, q), K.h));
     f = rn_mul(d, q);
     df = rn_mul(q, rn_fma(-0.5, dh, 1.0));
   } else {
-    const double pr = rn_mul(p, K.ip);
-    const double prz = pow64(pr, G.z);
+    const double prz = pow64(div64(p, K.p), G.z);
     f = rn_mul(K.two_c, rn_add(prz, -1.0));
     df = rn_mul(rn_mul(prz, K.c_g), ip);
   }
@@ -484,11 +482,9 @@ __device__ __forceinline__ int riemann_sample_c(real rhoL, real uL, real pL, rea
     if ((real)0 <= s * (uK - s * cK)) {
       rhoF = rhoK; uF = uK; pF = pK;
     } else {
-      // r^(1/gamma) = r / (r^z)^2
-      const real rz = xpow(r, G.z);
-      const real tail = us - s * cK * rz;
+      const real tail = us - s * cK * xpow(r, G.z);
       if ((real)0 > s * tail) {
-        rhoF = rhoK * xdiv(r, rn_mul(rz, rz)); uF = us; pF = ps;
+        rhoF = rhoK * xpow(r, G.inv_g); uF = us; pF = ps;
       } else {
         const real c = G.two_gp1 * cK + s * G.gm1_gp1 * uK;
         const real q = xdiv(c, cK);
