@@ -10,6 +10,7 @@
 // gather yields the closure error |sum_faces A n_out| / sum A (zero for a
 // closed cell by the divergence theorem).  All in FP64.
 #include "amm_internal.cuh"
+#include "fixed64.cuh"
 
 namespace amm {
 
@@ -45,7 +46,7 @@ __global__ void k_cell_geometry(int n, int dim, const int* csr_off, const int2* 
                                 R4<double>* cg64, float* closure) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const double frac = (double)dim / (double)(dim + 1), third = 1.0 / dim;
+  const double frac = (double)dim / (double)(dim + 1);
   double V = 0.0, mx = 0.0, my = 0.0, mz = 0.0, cx = 0.0, cy = 0.0, cz = 0.0, asum = 0.0;
   for (int q = csr_off[i]; q < csr_off[i + 1]; q++) {
     const int2 e = csr[q];
@@ -53,7 +54,8 @@ __global__ void k_cell_geometry(int n, int dim, const int* csr_off, const int2* 
     const double sg = (e.x & 1) ? -1.0 : 1.0;
     const R4<double> g0 = fg64[2 * (size_t)k], g1 = fg64[2 * (size_t)k + 1];
     const double h = 0.5 * g0.w;
-    const double vp = g1.w * h * third;
+    // (a product with a rounded 1/3 would move every volume by 5e-17)
+    const double vp = div64(g1.w * h, (double)dim);
     // face centroid relative to the generator of this cell
     const double fx = sg * h * g0.x + g1.x, fy = sg * h * g0.y + g1.y, fz = sg * h * g0.z + g1.z;
     V += vp;
