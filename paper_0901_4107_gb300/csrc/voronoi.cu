@@ -36,6 +36,7 @@
 
 #include "amm.h"
 #include "face_walk.cuh"
+#include "fixed64.cuh"
 #include "half_list.cuh"
 #include "scan.cuh"
 
@@ -883,7 +884,7 @@ __global__ void __launch_bounds__(32 * FWARPS, 5) k_cells3_fast(const __grid_con
       if (__any_sync(full, open)) rc = -1;
     }
     int nf = 0, walked = 0;
-    double sum[4] = {0.0, 0.0, 0.0, 0.0};   // volume, first moment
+    double sum[4] = {0.0, 0.0, 0.0, 0.0};   // three times the volume and the first moment
     __syncwarp();
     if (rc == 0) {
       if (L[1] != 0u && __popc(L[0]) + __popc(L[1]) <= 32) {
@@ -956,21 +957,25 @@ __global__ void __launch_bounds__(32 * FWARPS, 5) k_cells3_fast(const __grid_con
           const bool ok = m > 0;
           if (!ok) rc = -1;
           if (ok && m >= 3) {
-            // one division for both 1 / n_ax and 1 / (3 A)
-            const double nax = pk[ax];
-            const double A3 = A != 0.0 ? 3.0 * A : 1.0;
-            const double inv = 1.0 / (nax * A3);
-            const double in = inv * A3, third = inv * nax, ia = fabs(in);
+            // (each reciprocal by itself, on the integer pipe: one FP64 division for both
+            // 1 / n_ax and 1 / (3 A) left them three roundings each)
+            const double in = recip64(pk[ax]), ia = fabs(in);
+            const double third = recip64(A != 0.0 ? 3.0 * A : 1.0);
             const double a2 = 0.5 * fabs(A);             // area in the projection
-            area = a2 * ia * sqrt(2.0 * pk[3]);          // |n|^2 = 2 h
+            area = a2 * sqrt64(2.0 * pk[3]) * ia;        // |n|^2 = 2 h
             const double u = ou + Cu * third, v = ov + Cv * third;
             const double z = (pk[3] - pk[cu] * u - pk[cv] * v) * in;
             fc[0] = ax == 0 ? z : (cu == 0 ? u : v);
             fc[1] = ax == 1 ? z : (cu == 1 ? u : v);
             fc[2] = ax == 2 ? z : (cu == 2 ? u : v);
             // pyramid with apex at the generator: height times area / 3 (the
-            // height is h / |n|), centroid 3/4 of the way to the face
-            const double vp = pk[3] * a2 * ia * (1.0 / 3.0);
+            // height is h / |n|), centroid 3/4 of the way to the face; three
+            // times it here (a rounded 1/3 would move every volume by -5e-17)
+            // (h is d^2 / 2 to three roundings, which an area and height of one
+            // unit normal would cancel: most of what they took off is put back)
+            const double r0 = __fma_rn(pk[ax], pk[ax], -2.0 * pk[3]);
+            const double r1 = __fma_rn(pk[cv], pk[cv], __fma_rn(pk[cu], pk[cu], r0));
+            const double vp = __fma_rn(0.5, r1, pk[3]) * a2 * ia;
             sum[0] += vp;
             for (int d = 0; d < 3; d++) sum[1 + d] += vp * 0.75 * fc[d];
             keep = area > thr_area;
@@ -1012,7 +1017,7 @@ __global__ void __launch_bounds__(32 * FWARPS, 5) k_cells3_fast(const __grid_con
       if (rc == 0) {
         if (lane == 0) {
           nhf[i] = nf;
-          vol[i] = t;
+          vol[i] = div64(t, 3.0);
         } else if ((lane & 7) == 0) {
           const double r = comp == 1 ? ri[0] : (comp == 2 ? ri[1] : ri[2]);
           com[(size_t)i * 3 + comp - 1] = r + (Vt > 0.0 ? t / Vt : 0.0);
