@@ -132,11 +132,13 @@ def peaks():
 # the sources each profiled kernel is compiled from (its DRAM traffic in
 # profiles/ncu_traffic.json and its FLOP counts in profiles/ncu_alu.json hold
 # only while these are unchanged)
-_COMMON = ["amm_internal.cuh", "hydro.cuh", "riemann.cuh", "fixed64.cuh", "hydro_f32.cu", "../../include/amm.h"]
+_COMMON = ["amm_internal.cuh", "hydro.cuh", "riemann.cuh", "fixed64.cuh", "pow64_tables.cuh", "hydro_f32.cu",
+           "../../include/amm.h"]
 KERNEL_SOURCES = {
     "gradients": _COMMON, "update": _COMMON,
     "flux": _COMMON + ["flux_chunks.cu", "learned.cuh"],
-    "flux_fp64": ["amm_internal.cuh", "hydro.cuh", "riemann.cuh", "fixed64.cuh", "hydro_f64.cu", "../../include/amm.h"],
+    "flux_fp64": ["amm_internal.cuh", "hydro.cuh", "riemann.cuh", "fixed64.cuh", "pow64_tables.cuh", "hydro_f64.cu",
+                  "../../include/amm.h"],
     "learned_flux": _COMMON + ["flux_chunks.cu", "flux_learned.cu", "learned.cuh", "tc.cuh", "persistent.cuh"],
 }
 
