@@ -11,18 +11,21 @@
 //                  active-cell list                          (Sec. 7.2)
 //  k_ind_leaf / k_ind_up   per bucket of a uniform-grid pyramid over the
 //                  box: the largest c + |v| of its cells and that cell
-//  k_ind_grad      active cells: limited gradients (eq. eqngrad2), the
-//                  neighbours entering with their stored W   (Sec. 3.1)
-//  k_ind_bins      active cells: dt_i = C min(tau_i, R_i/(c_i+|v_i|)) by a
-//                  pruned walk of the pyramid, the new bin (a shorter step
-//                  freely, a longer one at most twice the current step and
-//                  only where that step starts now), the bin histogram
-//                                                             (Sec. 7.1, 7.2)
+//  k_ind_cells     active cells: limited gradients (eq. eqngrad2), the
+//                  neighbours entering with their stored W, by every other
+//                  CTA (ind_grad)                            (Sec. 3.1);
+//                  dt_i = C min(tau_i, R_i/(c_i+|v_i|)) by a pruned walk of
+//                  the pyramid, the new bin (a shorter step freely, a longer
+//                  one at most twice the current step and only where that
+//                  step starts now) and the bin histogram, by the others
+//                  (ind_bins)                                (Sec. 7.1, 7.2)
 //  k_ind_faces     faces with an active cell: the active-face list, their
 //                  step (the smaller of the two cells') and stamps
 //  k_ind_flux      active faces: extrapolation, each side predicted from its
 //                  own last activation to the middle of the face's step,
-//                  Riemann solve, flux                        (Sec. 3.3)
+//                  Riemann solve, flux (Sec. 3.3); in the FP64 form one
+//                  launch for few faces and one for many, of which the
+//                  other leaves at once
 //  k_ind_update    touched cells: Q -= sum over active faces of
 //                  +-dt_f A F (pairwise, conservative; no atomics)
 //
@@ -696,12 +699,12 @@ cudaError_t launch_individual_tick(amm_ctx* c, const IndView& d) {
   }
   // list kernels: a fixed grid strides over the list, whose length only the
   // device knows
-  const int sms = 152;
+  constexpr int sms = 152;
   const int g_cells = nblk(c->n, BINS_WARPS), g_flux = nblk(c->nf, 128);
   k_ind_cells<real><<<2 * (g_cells < sms * 8 ? g_cells : sms * 8), 32 * BINS_WARPS, 0, c->stream>>>(v, d, sms * 4);
   k_ind_faces<real><<<nblk(c->nf, 256), 256, 0, c->stream>>>(v, d);
-  const int few = sizeof(real) == 8 ? sms * 32 * 2 : 0;
-  if (few) k_ind_flux<real, 32><<<sms * 4, 32, 0, c->stream>>>(v, d, 0, few);
+  constexpr int few = sizeof(real) == 8 ? sms * 32 * 2 : 0;
+  if constexpr (few > 0) k_ind_flux<real, 32><<<sms * 4, 32, 0, c->stream>>>(v, d, 0, few);
   k_ind_flux<real, 128><<<g_flux < sms * 8 ? g_flux : sms * 8, 128, 0, c->stream>>>(v, d, few, 0x7fffffff);
   k_ind_update<real><<<nblk(c->n * 4, 256), 256, 0, c->stream>>>(v, d);
   return cudaGetLastError();

@@ -4,8 +4,9 @@
 // feeds it (face-state harvest, exact p* targets, feature normalisation).
 // The paper has no such component; see learned.cuh for the specification.
 //
-// Tiles are 128 samples (faces), one per thread of a 4-warp CTA, so sample t
-// of the tile is row t of every MMA and lane t of tensor memory.
+// Tiles are 128 samples (faces): sample t of the tile is row t of every MMA and
+// lane t of tensor memory.  The forward kernel has a thread per sample (4 warps),
+// the gradient kernel two, which split the columns (8 warps).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
