@@ -68,21 +68,22 @@ void free_ctx(amm_ctx* c) {
 // Lanes per cell of the gradient and update kernels (amm_tuning; amm_autotune
 // measures them): with few cells more lanes put the chip's threads to work and
 // shorten each one's chain of gathers, with many they only repeat the
-// per-cell work.  Measured (us, gradients / update of one step):
-//   FP32, cells   1 lane         2 lanes        4 lanes        8 lanes
-//     1.6 k       11.9 / 12      11.9 / 10.2    11.9 / 10.2    11.8 / 9.6
-//    64 k         26 / 20        22 / 19        22 / 22        29 / 32
-//   262 k         78 / 55        64 / 49        63 / 53        82 / 80
-//   1.4 M        331 / 217      271 / 192      281 / 236      398 / 369
+// per-cell work.  Measured on static meshes (us by the step's own events, gradients with
+// the Courant pass / update):
+//   FP32, cells   1 lane        2 lanes       4 lanes       8 lanes
+//     1.6 k (2D)  15 / 10       13 / 8        14 / 8        14 / 8
+//    64 k         29 / 16       25 / 16       24 / 16       29 / 23
+//   262 k         79 / 51       66 / 45       66 / 51       87 / 76
+//   1.4 M        327 / 209     271 / 170     279 / 231     404 / 363
 //   FP64, cells
-//     8.2 k (2D)  47 / 19        38 / 14        35 / 10        44 / 12
-//    13.8 k       86 / 29        60 / 20        67 / 21        76 / 18
-//    33 k         86 / 29       102 / 28       118 / 35       150 / 41
-//    91 k        208 / 68       217 / 59       264 / 76       374 / 92
+//     8.2 k (2D)  49 / 18       39 / 14       32 / 10       43 / 12
+//    13.8 k       81 / 27       57 / 18       67 / 21       74 / 18
+//    33 k         84 / 29       98 / 27      114 / 35      148 / 41
+//    91 k        205 / 66      212 / 57      260 / 76      371 / 92
 // The FP64 flux kernel: few faces go to CTAs of 64, which spread them over all SMs'
 // FP64 pipes in the faces' own order; many to CTAs of 256, which group the solves by
-// kind.  (us for faces, 64 / 256: 25 k 27 / 35, 98 k 55 / 69 in 2D and 98 / 102 in 3D,
-// 230 k 182 / 178, 715 k 471 / 445.)
+// kind.  (us for faces, 64 / 128 / 256: 25 k in 2D 30 / 36 / 38, 109 k 196 / 198 / 200,
+// 257 k 192 / 196 / 186, 715 k 487 / 475 / 458.)
 void default_shapes(amm_ctx* c) {
   const int64_t few = 40000;   // threads below which more lanes still pay (two warps for each of the chip's 608 FP64 pipes)
   c->update_lanes = 8 * c->n <= few ? 8 : (4 * c->n <= few ? 4 : 2);

@@ -903,8 +903,8 @@ __device__ __forceinline__ void stats_add(DeviceStats* S, unsigned* box_status, 
 // go through shared memory, ordered by the kind of solve (judged in FP32, on
 // the idle FP32 pipe); every face's arithmetic is the same wherever it runs.
 // 91 k cells, one step's fluxes: 2412 us in face order, 1540 regrouped (21.7 lanes
-// on); 445 with the divisions, roots and powers in fixed point on the integer pipe
-// and the comparisons in integers (1130 -> 274 FP64 instructions a warp).
+// on); 458 with the divisions, roots and powers in fixed point on the integer pipe
+// and the comparisons in integers (1130 -> 297 FP64 instructions a warp of faces).
 template <int B>
 __device__ __forceinline__ void solve_grouped(const HydroView<double>& v, const FaceWork<double>& f,
                                               RiemannOut<double>& r) {
@@ -1044,8 +1044,8 @@ __device__ __forceinline__ void flux_item(const HydroView<real>& v, int wi) {
   face_finish<real, B, ENT>(v, f, t.box, min(B, t.end - first), false, (real)0);
 }
 
-// (FP64: 16 warps per SM, 128 registers; 24 warps at 80 registers: 453 us for 445
-// at 715 k faces, whose FP64 instructions alone take 366)
+// (FP64: 16 warps per SM, 128 registers; 24 warps at 80 registers took 2 % longer at
+// 715 k faces: 458 us, the FP64 pipe busy for four fifths of them)
 template <typename real, int B, bool ENT>
 __global__ void __launch_bounds__(B, sizeof(real) == 4 ? 4 * FACE_TILE / B : 2 * FACE_TILE / B) k_flux(HydroView<real> v) {
   flux_item<real, B, ENT>(v, blockIdx.x);
@@ -1144,8 +1144,8 @@ static_assert(FIX_RUN % UPD_BATCH == 0, "a run is whole batches");
 // chain list -> face index -> flux (long scoreboard; DRAM at a third, issue at a
 // third), so two fluxes and the next two indices are in flight per lane.
 // 1.4 M cells of 7.8 faces, 4 lanes per cell with lane 0 of each group
-// finishing its own cell: 471 us; 2 lanes, as here: 192 us, 174 without FP64
-// conversions (1 lane 212, 4 lanes 233); 348 k cells with the entropy switch: 111 us,
+// finishing its own cell: 471 us; 2 lanes, as here: 192 us, 170 without FP64
+// conversions (1 lane 209, 4 lanes 231); 348 k cells with the entropy switch: 111 us,
 // 86 without FP64 conversions and divisions.  ENT: the entropy switch of
 // Sec. 3.5 (a sixth flux component, the entropy, and the per-cell choice
 // between the advected entropy and the energy update).  LOOP: the CTA goes on to

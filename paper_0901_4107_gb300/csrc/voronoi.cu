@@ -467,7 +467,7 @@ __device__ int cut_buffer3(Cell3& C, int lane, int nc, double eps, float& R2) {
 //    summed in the two coordinates its normal projects to best (8 FP64
 //    operations per triangle instead of 30), the third follows from the plane.
 // 10 KB per cell, 20 warps per SM.  64^3 cells: 27.1 ms with k_cells3 alone,
-// 5.0 ms now (FP64 pipe 69% busy, issue 49%).
+// 5.3 ms now (FP64 pipe 66% busy, issue 47%).
 constexpr int FP = 64;         // planes
 constexpr int FWARPS = 4;      // cells per CTA
 constexpr unsigned NOKEY = 0xffffffffu;
